@@ -307,7 +307,7 @@ smtm_status_t lookup_impl(smtm_cache* c, int32_t layer, const smtm_fmap_t* f, co
                                 launch_encode_nhwc_vector_supported(e);
     // ... or, for a large fast memory scored on the tensor cores, the first lookup of a batch alone
     const bool dense = c->d_dense && dense_scoring_supported(a.D, a.n);
-    const bool pipelined_dense = c->maps_ready && allow_early && begin && dense && launch_encode_ring_supported(e);
+    const bool pipelined_dense = c->maps_ready && allow_early && begin && dense && launch_encode_split_supported(e);
     if (c->prof_events && c->prof_seq % c->L == 0) {  // a step begins: does it get a slot for the device-clock stamps?
         c->prof_step = nullptr;
         if ((c->prof_seq / c->L) % c->prof_every == 0 && c->prof_steps_used < c->prof_steps_cap) {

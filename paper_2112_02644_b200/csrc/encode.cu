@@ -14,12 +14,14 @@
 //   * unit-per-lane reducer (H*W small and odd-sized): lane i owns unit i of the chunk and
 //     walks its 16-byte vectors; the stride between lanes is an odd number of vectors, so the
 //     128-bit shared loads are conflict-free; the element -> channel map is resolved at compile time.
-//   * team-per-channel reducer (channel bytes a multiple of 16): T lanes share a channel,
-//     stride over its vectors and combine with xor-shuffles.
+//   * team reducer: T lanes share a channel, stride over its vectors and combine with xor-shuffles;
+//     channels that begin or end inside a vector have their edges added element by element.
+//   * lane-per-channel reducer (channels of odd widths below 128 bytes): 32-bit words.
+// Small batches, and the few NCHW shapes bulk copies cannot serve, are pooled by the last two straight from global
+// memory (k_pool_direct).
 // NHWC.  Consecutive 16-byte vectors of a frame are consecutive channel groups of a pixel;
 // each thread owns one channel group and a pixel phase, loads coalesced 128-bit vectors
 // directly and the phases are combined through shared memory in ascending order.
-// Any other shape falls back to a plain thread-per-(frame, channel) loop.
 #include <algorithm>
 #include <cmath>
 
@@ -33,7 +35,6 @@ constexpr int kStages = 8;             // ring depth
 constexpr int kConsumers = 8;          // consumer warps; stage s belongs to warp s % kConsumers
 constexpr int kStageCap = 25600;       // bytes per stage
 constexpr int kThreadsTma = (kConsumers + 1) * kWarp;
-constexpr size_t kSmemTma = size_t(kStages) * kStageCap + 2 * kStages * sizeof(uint64_t) + 128;
 
 struct NchwParams {
     const uint8_t* x;
@@ -42,15 +43,15 @@ struct NchwParams {
     __nv_bfloat16* sv_hi;    // optional bf16 head and tail of sv (sv = hi + lo), same indexing; may be null
     __nv_bfloat16* sv_lo;
     int* status;
-    long long total_chunks;  // B * chunks per frame
+    int B;                   // frames
     int C;
     int chunks_per_frame;
     int chunk_channels;      // channels in a full chunk
     int ch_bytes;            // bytes of one channel
     long long frame_bytes;
     float inv_hw;
-    int team;                // team-per-channel: lanes per channel (power of two)
-    int vec_per_channel;     // team-per-channel: 16-byte vectors per channel
+    int hw, es;              // elements per channel, bytes per element
+    int team;                // the team reducers: lanes per channel (power of two)
     int max_in_flight;       // copies the producer keeps outstanding (<= stages)
     int stages;              // k_encode_nchw: ring depth, 2 .. kStages (the fused kernel always uses kStages)
     int consumers;           // k_encode_nchw: consumer warps, 1 .. kConsumers; the CTA has one more warp, the producer's
@@ -80,7 +81,7 @@ struct UnitPerLane {
     static constexpr int G = 16 / gcd16(kUnitBytesRaw);
     static constexpr int UW = G * kUnitBytesRaw / 16;
 
-    static __device__ __forceinline__ void run(const uint8_t* stage, int nch, int lane, float* out, float* out_s,
+    static __device__ __forceinline__ void run(const uint8_t* stage, int, int nch, int lane, float* out, float* out_s,
                                                float inv_hw, const NchwParams& p) {
         const int units = nch / G;
         if (lane >= units) return;
@@ -121,79 +122,257 @@ struct UnitPerLane {
     }
 };
 
-// T lanes per channel; channel bytes are a multiple of 16.  Two passes (channels per team) are
-// folded at a time, one accumulator per element of a vector and two vectors of each in
-// flight: a single warp has to keep up with the copies, so the loop must not be one chain of
-// dependent additions.
-template <class E>
-struct TeamPerChannel {
-    static __device__ __forceinline__ void run(const uint8_t* stage, int nch, int lane, float* out, float* out_s,
-                                               float inv_hw, const NchwParams& p) {
-        const int T = p.team, uw = p.vec_per_channel;
-        const int per_pass = kWarp / T;
-        const int team = lane / T, r = lane - team * T;
-        const int passes = (nch + per_pass - 1) / per_pass;
-        for (int ps = 0; ps < passes; ps += 2) {
-            const int c0 = ps * per_pass + team, c1 = c0 + per_pass;  // this team's channels of the two passes
-            // a channel past the end is read as the chunk's last one and dropped afterwards
-            const uint4* u0 = reinterpret_cast<const uint4*>(stage) + size_t(min(c0, nch - 1)) * uw;
-            const uint4* u1 = reinterpret_cast<const uint4*>(stage) + size_t(min(c1, nch - 1)) * uw;
-            float a[2][E::kPerVec];
+// Writes a channel's mean wherever it is wanted.
+__device__ __forceinline__ void store_mean(const NchwParams& p, float v, int c, float* out, float* out_s) {
+    out[c] = v;
+    if (out_s) out_s[c] = v;
+    if (p.sv_hi) {
+        const ptrdiff_t at = (out + c) - p.sv;
+        const __nv_bfloat16 hh = __float2bfloat16_rn(v);
+        p.sv_hi[at] = hh;
+        p.sv_lo[at] = __float2bfloat16_rn(v - __bfloat162float(hh));
+    }
+}
+
+// T lanes per channel, 16-byte vectors.  Eight lanes read 128 consecutive bytes (one conflict-free phase of a shared
+// load, one line of global memory); channels shorter than that have as many lanes as whole vectors.  kEdges: channels
+// may begin and end inside a vector (`off`: elements of the stage before the first channel); the whole vectors in
+// between are walked as usual and the at most seven elements before and after are a load of their own in one lane
+// each, which takes T = 8.  Two channels per team are folded at a time, four vectors of each in flight: what bounds
+// a warp here is the latency of a chunk (a stage of the ring is held meanwhile), not the instructions.
+template <class E, bool kEdges>
+struct TeamVectors {
+    static constexpr int kShortChannel = 1024;  // bytes
+
+    template <int NB, int U>
+    static __device__ __forceinline__ void group(const uint8_t* stage, int off, int nch, int first, int stride, int r, int T,
+                                                 int lane, float* out, float* out_s, float inv_hw, const NchwParams& p) {
+        constexpr int V = E::kPerVec;
+        float a[NB][V];
+        const uint4* u[NB];
+        int n[NB], n_min = 1 << 30, n_max = 0;
 #pragma unroll
-            for (int j = 0; j < E::kPerVec; ++j) a[0][j] = a[1][j] = 0.f;
-            int i = r;
-            for (; i + T < uw; i += 2 * T) {
-                const uint4 v00 = u0[i], v01 = u0[i + T], v10 = u1[i], v11 = u1[i + T];
+        for (int h = 0; h < NB; ++h) {
+            const int c = min(first + h * stride, nch - 1);  // (a channel past the end: the last one, dropped below)
+            const int e0 = (kEdges ? off : 0) + c * p.hw, e1 = e0 + p.hw;
+            const int v0 = kEdges ? (e0 + V - 1) / V : e0 / V, v1 = e1 / V;
+            u[h] = reinterpret_cast<const uint4*>(stage) + v0;
+            n[h] = v1 - v0;
+            n_min = min(n_min, n[h]);
+            n_max = max(n_max, n[h]);
 #pragma unroll
-                for (int j = 0; j < E::kPerVec; ++j) {
-                    a[0][j] += E::at(v00, j);
-                    a[1][j] += E::at(v10, j);
-                }
-#pragma unroll
-                for (int j = 0; j < E::kPerVec; ++j) {
-                    a[0][j] += E::at(v01, j);
-                    a[1][j] += E::at(v11, j);
-                }
+            for (int j = 0; j < V; ++j) a[h][j] = 0.f;
+            if (kEdges) {
+                if (r < v0 * V - e0) a[h][0] = E::scalar(stage, e0 + r);
+                if (r < e1 - v1 * V) a[h][1] = E::scalar(stage, v1 * V + r);
             }
-            for (; i < uw; i += T) {
-                const uint4 v0 = u0[i], v1 = u1[i];
+        }
+        int i = r;
+        for (; i + (U - 1) * T < n_min; i += U * T) {
+            uint4 v[NB][U];
 #pragma unroll
-                for (int j = 0; j < E::kPerVec; ++j) {
-                    a[0][j] += E::at(v0, j);
-                    a[1][j] += E::at(v1, j);
-                }
-            }
-            float s[2];
+            for (int h = 0; h < NB; ++h)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                s[h] = (a[h][0] + a[h][1]) + (a[h][2] + a[h][3]);
-                if (E::kPerVec == 8)
-                    s[h] += (a[h][4 % E::kPerVec] + a[h][5 % E::kPerVec]) + (a[h][6 % E::kPerVec] + a[h][7 % E::kPerVec]);
-            }
-            for (int o = T >> 1; o > 0; o >>= 1) {
-                s[0] += __shfl_xor_sync(kFull, s[0], o);
-                s[1] += __shfl_xor_sync(kFull, s[1], o);
-            }
+                for (int k = 0; k < U; ++k) v[h][k] = u[h][i + k * T];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int c = h ? c1 : c0;
-                if (c < nch && r == 0) {
-                    const float v = s[h] * inv_hw;
-                    out[c] = v;
-                    if (out_s) out_s[c] = v;
-                    if (p.sv_hi) {
-                        const ptrdiff_t at = (out + c) - p.sv;
-                        const __nv_bfloat16 hh = __float2bfloat16_rn(v);
-                        p.sv_hi[at] = hh;
-                        p.sv_lo[at] = __float2bfloat16_rn(v - __bfloat162float(hh));
+            for (int k = 0; k < U; ++k)
+#pragma unroll
+                for (int h = 0; h < NB; ++h)
+#pragma unroll
+                    for (int j = 0; j < V; ++j) a[h][j] += E::at(v[h][k], j);
+        }
+        for (; i < n_max; i += T) {
+            uint4 v[NB];
+#pragma unroll
+            for (int h = 0; h < NB; ++h) v[h] = i < n[h] ? u[h][i] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int h = 0; h < NB; ++h)
+#pragma unroll
+                for (int j = 0; j < V; ++j) a[h][j] += E::at(v[h], j);
+        }
+        float s[NB];
+#pragma unroll
+        for (int h = 0; h < NB; ++h) {
+            s[h] = (a[h][0] + a[h][1]) + (a[h][2] + a[h][3]);
+            if (V == 8) s[h] += (a[h][4 % V] + a[h][5 % V]) + (a[h][6 % V] + a[h][7 % V]);
+        }
+        for (int o = T >> 1; o > 0; o >>= 1)
+#pragma unroll
+            for (int h = 0; h < NB; ++h) s[h] += __shfl_xor_sync(kFull, s[h], o);
+#pragma unroll
+        for (int h = 0; h < NB; ++h) {
+            const int c = first + h * stride;
+            if (c < nch && r == 0) store_mean(p, s[h] * inv_hw, c, out, out_s);
+        }
+    }
+
+    // Short channels: a few vectors per lane, so that adding the lanes up would cost more than the vectors.  NB
+    // channels per team go through the reduction together, each step halving what a lane still holds (seven
+    // exchanges for eight channels over eight lanes), and every lane writes its share.
+    template <int T, int NB>
+    static __device__ __forceinline__ void short_group(const uint8_t* stage, int off, int nch, int first, int r, float* out,
+                                                       float* out_s, float inv_hw, const NchwParams& p) {
+        constexpr int V = E::kPerVec;
+        constexpr int kStride = kWarp / T;
+        float s[NB];
+        const uint4* u[NB];
+        int n[NB], n_max = 0;
+#pragma unroll
+        for (int h = 0; h < NB; ++h) {
+            const int c = first + h * kStride;
+            const int e0 = (kEdges ? off : 0) + c * p.hw, e1 = e0 + p.hw;
+            const int v0 = kEdges ? (e0 + V - 1) / V : e0 / V, v1 = e1 / V;
+            u[h] = reinterpret_cast<const uint4*>(stage) + v0;
+            n[h] = c < nch ? v1 - v0 : 0;
+            n_max = max(n_max, n[h]);
+            s[h] = 0.f;
+            if (kEdges && c < nch) {
+                if (r < v0 * V - e0) s[h] = E::scalar(stage, e0 + r);
+                if (r < e1 - v1 * V) s[h] += E::scalar(stage, v1 * V + r);
+            }
+        }
+        for (int i = r; i < n_max; i += T) {
+            uint4 v[NB];
+#pragma unroll
+            for (int h = 0; h < NB; ++h) v[h] = i < n[h] ? u[h][i] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int h = 0; h < NB; ++h) {
+                float t = (E::at(v[h], 0) + E::at(v[h], 1)) + (E::at(v[h], 2) + E::at(v[h], 3));
+                if (V == 8) t += (E::at(v[h], 4 % V) + E::at(v[h], 5 % V)) + (E::at(v[h], 6 % V) + E::at(v[h], 7 % V));
+                s[h] += t;
+            }
+        }
+        int held = NB, h0 = 0;  // this lane ends up with the channels h0 .. h0 + held - 1 of its team
+#pragma unroll
+        for (int o = T / 2; o > 0; o >>= 1) {
+            const bool up = (r & o) != 0;
+            if (held > 1) {
+                held >>= 1;
+#pragma unroll
+                for (int e = 0; e < NB / 2; ++e)
+                    if (e < held) {
+                        const float give = up ? s[e] : s[e + held], keep = up ? s[e + held] : s[e];
+                        s[e] = keep + __shfl_xor_sync(kFull, give, o);
                     }
+                h0 += up ? held : 0;
+            } else {
+                s[0] += __shfl_xor_sync(kFull, s[0], o);
+            }
+        }
+        constexpr int kHeld = NB > T ? NB / T : 1;
+        const bool writes = NB >= T || (r & (T / NB - 1)) == 0;  // (fewer channels than lanes: one lane of each run that holds the same)
+#pragma unroll
+        for (int e = 0; e < kHeld; ++e) {
+            const int c = first + (h0 + e) * kStride;
+            if (writes && c < nch) store_mean(p, s[e] * inv_hw, c, out, out_s);
+        }
+    }
+
+    template <int T>
+    static __device__ __forceinline__ void run_short(const uint8_t* stage, int off, int nch, int lane, float* out, float* out_s,
+                                                     float inv_hw, const NchwParams& p) {
+        constexpr int kStride = kWarp / T;
+        const int team = lane / T, r = lane % T;
+        int c0 = 0;
+        for (; c0 + 2 * kStride < nch; c0 += 8 * kStride) short_group<T, 8>(stage, off, nch, c0 + team, r, out, out_s, inv_hw, p);
+        if (c0 < nch) short_group<T, 2>(stage, off, nch, c0 + team, r, out, out_s, inv_hw, p);
+    }
+
+    static __device__ __forceinline__ void run(const uint8_t* stage, int off, int nch, int lane, float* out, float* out_s,
+                                               float inv_hw, const NchwParams& p) {
+        if (p.ch_bytes < kShortChannel) {
+            if (kEdges || p.team == 8) run_short<8>(stage, off, nch, lane, out, out_s, inv_hw, p);
+            else if (p.team == 4) run_short<4>(stage, off, nch, lane, out, out_s, inv_hw, p);
+            else if (p.team == 2) run_short<2>(stage, off, nch, lane, out, out_s, inv_hw, p);
+            else run_short<1>(stage, off, nch, lane, out, out_s, inv_hw, p);
+            return;
+        }
+        constexpr int T = 8, kStride = kWarp / T;
+        const int team = lane / T, r = lane % T;
+        int c0 = 0;
+        for (; c0 + kStride < nch; c0 += 2 * kStride)
+            group<2, 4>(stage, off, nch, c0 + team, kStride, r, T, lane, out, out_s, inv_hw, p);
+        if (c0 < nch) group<1, 8>(stage, off, nch, c0 + team, kStride, r, T, lane, out, out_s, inv_hw, p);
+    }
+};
+
+// A lane per channel for short channels of any number of bytes (below 128): each is walked in 32-bit words, whichever
+// element of the stage it begins at (`off`: elements before the first channel).  With 16-bit elements a channel that
+// begins or ends inside a word gets that element by a load of its own.
+template <class E>
+struct LanePerChannel {
+    static __device__ __forceinline__ float low(uint32_t w) { return E::at(make_uint4(w, 0, 0, 0), 0); }
+    static __device__ __forceinline__ float high(uint32_t w) { return E::kSize == 2 ? E::at(make_uint4(w, 0, 0, 0), 1) : 0.f; }
+
+    static __device__ __forceinline__ void run(const uint8_t* stage, int off, int nch, int lane, float* out, float* out_s,
+                                               float inv_hw, const NchwParams& p) {
+        constexpr int kPerWord = 4 / E::kSize;
+        constexpr int kBatch = 8;  // words in flight per lane
+        const uint32_t* words = reinterpret_cast<const uint32_t*>(stage);
+        for (int c = lane; c < nch; c += kWarp) {
+            const int e0 = off + c * p.hw, e1 = e0 + p.hw;
+            int w = (e0 + kPerWord - 1) / kPerWord;   // the words that are all this channel's
+            const int w1 = e1 / kPerWord;
+            float lo[4] = {0.f, 0.f, 0.f, 0.f}, hi[4] = {0.f, 0.f, 0.f, 0.f};
+            if (kPerWord == 2 && (e0 & 1)) hi[1] = E::scalar(stage, e0);
+            if (kPerWord == 2 && (e1 & 1)) lo[1] = E::scalar(stage, e1 - 1);
+            for (; w + kBatch <= w1; w += kBatch) {
+                uint32_t v[kBatch];
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) v[u] = words[w + u];
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    lo[u & 3] += low(v[u]);
+                    if (kPerWord == 2) hi[u & 3] += high(v[u]);
                 }
             }
+            if (w < w1) {
+                uint32_t v[kBatch];
+#pragma unroll
+                for (int u = 0; u < kBatch - 1; ++u) v[u] = w + u < w1 ? words[w + u] : 0u;
+#pragma unroll
+                for (int u = 0; u < kBatch - 1; ++u) {
+                    lo[u & 3] += low(v[u]);
+                    if (kPerWord == 2) hi[u & 3] += high(v[u]);
+                }
+            }
+            float s = (lo[0] + lo[1]) + (lo[2] + lo[3]);
+            if (kPerWord == 2) s += (hi[0] + hi[1]) + (hi[2] + hi[3]);
+            store_mean(p, s * inv_hw, c, out, out_s);
         }
     }
 };
 
 // ---- persistent bulk-copy pipeline -------------------------------------------------------
+//
+// What bounds it: HBM, once a CTA's warps do next to nothing per chunk besides their own share.  A warp steps from
+// chunk to chunk by additions alone (frame and chunk-of-frame advance by constants), and only over its own chunks:
+// with a 64-bit division per chunk and every warp looking at every chunk the loop itself was the bound (1.64 GB of
+// 56x56 maps in 312 us, 5.3 TB/s).  Four 25 KB copies in flight per SM saturate the reads (7.2 TB/s in a
+// copy-only ring; 200 KB in flight are slower again).
+// Without skip flags a batch is one run of B * C channels (chunks may span frames, so that small maps make
+// full-sized copies: one thread issues a copy per 0.27 us and would cap 4 KB copies at 2.2 TB/s).  With them the
+// frames still in are listed first, a tile of frames at a time.
+constexpr int kListFrames = 2048;  // frames listed at a time
+
+// The chunk a warp is at: chunk `ci` of listed frame `f`; step(n) moves on by n * gridDim.x chunks.
+struct ChunkWalk {
+    int f, ci, df, dci, cpf;
+    __device__ __forceinline__ ChunkWalk(int first, int stride, int chunks_per_frame) : cpf(chunks_per_frame) {
+        f = first / cpf;
+        ci = first - f * cpf;
+        df = stride / cpf;
+        dci = stride - df * cpf;
+    }
+    __device__ __forceinline__ void step() {
+        f += df;
+        ci += dci;
+        if (ci >= cpf) {
+            ci -= cpf;
+            ++f;
+        }
+    }
+};
 
 template <class R>
 __global__ void __launch_bounds__(kThreadsTma, 1) k_encode_nchw(const NchwParams p) {
@@ -220,51 +399,105 @@ __global__ void __launch_bounds__(kThreadsTma, 1) k_encode_nchw(const NchwParams
     const int n_consumers = p.consumers;
     const bool producer = warp == n_consumers;  // last warp; lane 0 issues the copies
     const uint64_t stream_once = l2_evict_first_policy();
-    int it = 0;                                // chunks of this CTA that are not skipped, so far
+    int* list = reinterpret_cast<int*>(empty + n_stages);  // [kListFrames + 33], only there with skip flags
+    const int grid = int(gridDim.x), cpf = p.chunks_per_frame;
+    int it0 = 0;         // chunks of this CTA in the tiles of frames before this one
+    int issued = 0;
     bool failed = false;
-    if (!producer || lane == 0) {
-        for (long long g = blockIdx.x; g < p.total_chunks; g += gridDim.x) {
-            const int b = int(g / p.chunks_per_frame);
-            if (p.skip && p.skip[b]) continue;
-            const int ci = int(g - (long long)b * p.chunks_per_frame);
-            const int stage = it % n_stages;
-            const uint32_t use = uint32_t(it / n_stages);
-            const int c0 = ci * p.chunk_channels;
-            const int nch = min(p.chunk_channels, p.C - c0);
-            if (producer) {
-                if (use > 0 && !mbar_wait_bounded(&empty[stage], (use - 1) & 1, p.status)) {
-                    failed = true;
-                    break;
-                }
-                if (it >= p.max_in_flight) {  // bound the bytes in flight: wait for an older copy to land
-                    const int old = it - p.max_in_flight;
-                    if (!mbar_wait_bounded(&full[old % n_stages], (old / n_stages) & 1, p.status)) {
-                        failed = true;
-                        break;
+    const auto span_of = [&](int c0, int nch, long long& begin, int& off) {  // a chunk's bytes, widened to 16-byte boundaries
+        const long long lo = (long long)c0 * p.ch_bytes;
+        begin = lo & ~15ll;
+        off = int(lo - begin);
+        return uint32_t((off + nch * p.ch_bytes + 15) & ~15);
+    };
+    for (int t0 = 0; t0 < p.B; t0 += kListFrames) {
+        int frames = p.B;  // no flags: all of them (one "frame" of B * C channels), in a single round
+        if (p.skip) {
+            frames = 0;
+            int* s_scan = list + kListFrames;
+            __syncthreads();  // the list of the tile before is read to the end
+            for (int u0 = t0; u0 < min(p.B, t0 + kListFrames); u0 += int(blockDim.x)) {
+                const int b = u0 + int(threadIdx.x);
+                const int act = (b < min(p.B, t0 + kListFrames) && !p.skip[b]) ? 1 : 0;
+                int cnt;
+                const int pos = block_exclusive_scan(act, s_scan, &cnt);
+                if (act) list[frames + pos] = b;
+                frames += cnt;
+            }
+            __syncthreads();
+        }
+        const int chunks = frames * cpf;
+        const int mine = chunks > int(blockIdx.x) ? (chunks - int(blockIdx.x) + grid - 1) / grid : 0;
+        if (producer) {
+            if (lane == 0) {
+                ChunkWalk at(int(blockIdx.x), grid, cpf);
+                int stage = it0 % n_stages;
+                uint32_t phase = uint32_t(it0 / n_stages) & 1u;
+                int old = it0 - p.max_in_flight;  // the copy that has to have landed before this one is issued
+                int old_stage = old >= 0 ? old % n_stages : 0;
+                uint32_t old_phase = old >= 0 ? uint32_t(old / n_stages) & 1u : 0u;
+                for (int i = 0; i < mine; ++i, ++old) {
+                    if (it0 + i >= n_stages && !mbar_wait_bounded(&empty[stage], phase ^ 1u, p.status)) failed = true;
+                    if (!failed && old >= 0) {
+                        if (!mbar_wait_bounded(&full[old_stage], old_phase, p.status)) failed = true;
+                        if (++old_stage == n_stages) {
+                            old_stage = 0;
+                            old_phase ^= 1u;
+                        }
+                    }
+                    if (failed) break;
+                    const int c0 = at.ci * p.chunk_channels, nch = min(p.chunk_channels, p.C - c0);
+                    const long long b = p.skip ? list[at.f] : at.f;
+                    long long begin;
+                    int off;
+                    const uint32_t bytes = span_of(c0, nch, begin, off);
+                    mbar_expect_tx(&full[stage], bytes);
+                    bulk_load_hint(stages + size_t(stage) * kStageCap, p.x + b * p.frame_bytes + begin, bytes, &full[stage],
+                                   stream_once);
+                    issued = it0 + i + 1;
+                    at.step();
+                    if (++stage == n_stages) {
+                        stage = 0;
+                        phase ^= 1u;
                     }
                 }
-                const uint32_t bytes = uint32_t(nch) * uint32_t(p.ch_bytes);
-                mbar_expect_tx(&full[stage], bytes);
-                bulk_load_hint(stages + size_t(stage) * kStageCap,
-                               p.x + (long long)b * p.frame_bytes + (long long)c0 * p.ch_bytes, bytes, &full[stage], stream_once);
-            } else if (stage % n_consumers == warp) {
-                if (!mbar_wait_bounded(&full[stage], use & 1, p.status)) {
+            }
+        } else {
+            // chunk number `it` of this CTA goes to warp it % n_consumers and sits in stage it % n_stages
+            const int first = (warp - it0 % n_consumers + n_consumers) % n_consumers;
+            ChunkWalk at(int(blockIdx.x) + first * grid, n_consumers * grid, cpf);
+            int stage = (it0 + first) % n_stages;
+            uint32_t phase = uint32_t((it0 + first) / n_stages) & 1u;
+            for (int i = first; i < mine; i += n_consumers) {
+                const int c0 = at.ci * p.chunk_channels, nch = min(p.chunk_channels, p.C - c0);
+                const long long b = p.skip ? list[at.f] : at.f;
+                long long begin;
+                int off;
+                span_of(c0, nch, begin, off);
+                if (!mbar_wait_bounded(&full[stage], phase, p.status)) {
                     failed = true;
                     break;
                 }
-                R::run(stages + size_t(stage) * kStageCap, nch, lane, p.sv + (long long)b * p.C + c0, nullptr, p.inv_hw, p);
+                R::run(stages + size_t(stage) * kStageCap, off / p.es, nch, lane, p.sv + b * p.C + c0, nullptr, p.inv_hw, p);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&empty[stage]);
+                at.step();
+                stage += n_consumers;  // (no more consumers than stages)
+                if (stage >= n_stages) {
+                    stage -= n_stages;
+                    phase ^= 1u;
+                }
             }
-            ++it;
         }
+        it0 += mine;
+        if (!p.skip) break;
     }
     // No thread leaves before every copy that was issued has landed: shared memory must
     // stay allocated until the copy engine is done with it.
     const int any_failed = __syncthreads_or(failed ? 1 : 0);
     if (any_failed && producer && lane == 0) {
-        for (int s = 0; s < n_stages && s < it; ++s) {
-            const uint32_t last_use = uint32_t((it - 1 - s) / n_stages);
+        for (int s = 0; s < n_stages && s < issued; ++s) {
+            const uint32_t last_use = uint32_t((issued - 1 - s) / n_stages);
             mbar_wait_bounded(&full[s], last_use & 1, p.status);
         }
     }
@@ -454,7 +687,7 @@ __global__ void __launch_bounds__(kThreadsFused, 1) k_lookup_nchw(const FusedPar
             const int buf = i % kSvBufs, round = i / kSvBufs;
             if (round > 0 && !mbar_wait_bounded(&sv_empty[buf], (round - 1) & 1, p.status)) { failed = true; break; }
             if (!mbar_wait_bounded(&full[stage], (it / kStages) & 1, p.status)) { failed = true; break; }
-            R::run(stages + size_t(stage) * kStageCap, nch, lane, p.sv + (long long)b * p.C + c0,
+            R::run(stages + size_t(stage) * kStageCap, 0, nch, lane, p.sv + (long long)b * p.C + c0,
                    sv_s + buf * f.slice_cap + c * p.chunk_channels, p.inv_hw, p);
             __syncwarp();
             if (lane == 0) {
@@ -686,7 +919,7 @@ __global__ void __launch_bounds__(kLightThreads) k_pool_sparse(const LightParams
     __shared__ int s_scan[33];
     const NchwParams& p = f.e;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int B = int(p.total_chunks / p.chunks_per_frame);
+    const int B = p.B;
     const int ci = int(blockIdx.x) % p.chunks_per_frame, group = int(blockIdx.x) / p.chunks_per_frame;
     chain_wait();  // the exit flags are the previous kernel's
     chain_release();
@@ -737,7 +970,7 @@ __global__ void __launch_bounds__(kLightThreads) k_pool_sparse(const LightParams
         }
         __syncthreads();
         if (w_nch > 0)
-            R::run(stage + size_t(w_c0) * p.ch_bytes, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, nullptr, p.inv_hw, p);
+            R::run(stage + size_t(w_c0) * p.ch_bytes, 0, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, nullptr, p.inv_hw, p);
         __syncthreads();  // the stage is free for the next frame
     }
 }
@@ -854,7 +1087,7 @@ __global__ void __launch_bounds__(kLightThreads) k_lookup_sparse(const SparsePar
             if (u * kLightThreads + tid < vectors) dst[u * kLightThreads + tid] = r[u];
         __syncthreads();
         if (w_nch > 0)
-            R::run(stage + size_t(w_c0) * p.ch_bytes, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, sv_s + w_c0, p.inv_hw, p);
+            R::run(stage + size_t(w_c0) * p.ch_bytes, 0, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, sv_s + w_c0, p.inv_hw, p);
         __syncthreads();  // the slice is complete; the stage is free
         const uint32_t out = peer_smem(rx + ((k_it & 1) * kMaxCluster + rank) * kRxRow, 0);
         const float4* v4 = reinterpret_cast<const float4*>(sv_s);
@@ -1074,12 +1307,35 @@ __global__ void __launch_bounds__(kThreadsNhwcLookup) k_lookup_nhwc(const uint8_
     score_frame(a, b, pf, sv_s, nrm, s_cur, s_acc);
 }
 
-// ---- any shape: one thread per (frame, channel) ---------------------------------------------
+// ---- NCHW without a stage: a warp per run of channels, straight from global memory -------------
+//
+// For small batches, where the streaming kernel's set-up (a ring of most of an SM's shared memory, one copy after
+// another) costs more than the bytes, and for the shapes its copies cannot serve (frames that are no multiple of 16
+// bytes, channels longer than a stage).  The reducers are the same; nothing is shared between warps.
+constexpr int kDirectThreads = 128;
+
+template <class R>
+__global__ void __launch_bounds__(kDirectThreads) k_pool_direct(const NchwParams p) {
+    const int warp = int(blockIdx.x) * (kDirectThreads / kWarp) + int(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    chain_wait();
+    chain_release();
+    const ClockScope stamps(p.clock);
+    const int warps = int(gridDim.x) * (kDirectThreads / kWarp);
+    const long long chunks = (long long)p.B * p.chunks_per_frame;
+    for (long long g = warp; g < chunks; g += warps) {
+        const int b = int(g / p.chunks_per_frame), ci = int(g - (long long)b * p.chunks_per_frame);
+        if (p.skip && p.skip[b]) continue;
+        const int c0 = ci * p.chunk_channels, nch = min(p.chunk_channels, p.C - c0);
+        const long long lo = b * p.frame_bytes + (long long)c0 * p.ch_bytes, begin = lo & ~15ll;
+        R::run(p.x + begin, int(lo - begin) / p.es, nch, lane, p.sv + (long long)b * p.C + c0, nullptr, p.inv_hw, p);
+    }
+}
+
+// ---- NHWC, any number of channels: one thread per (frame, channel) ---------------------------
 
 template <class E>
-__global__ void k_encode_generic(const void* __restrict__ x, const uint8_t* __restrict__ skip,
-                                 float* __restrict__ sv, int B, int C, int HW, int nhwc, float inv_hw,
-                                 unsigned long long* clock) {
+__global__ void k_encode_nhwc_generic(const void* __restrict__ x, const uint8_t* __restrict__ skip, float* __restrict__ sv,
+                                      int B, int C, int HW, float inv_hw, unsigned long long* clock) {
     chain_wait();
     chain_release();
     const ClockScope stamps(clock);
@@ -1090,10 +1346,7 @@ __global__ void k_encode_generic(const void* __restrict__ x, const uint8_t* __re
         if (skip && skip[b]) continue;
         const size_t f0 = size_t(b) * C * HW;
         float s = 0.f;
-        if (nhwc)
-            for (int px = 0; px < HW; ++px) s += E::scalar(x, f0 + size_t(px) * C + c);
-        else
-            for (int px = 0; px < HW; ++px) s += E::scalar(x, f0 + size_t(c) * HW + px);
+        for (int px = 0; px < HW; ++px) s += E::scalar(x, f0 + size_t(px) * C + c);
         sv[i] = s * inv_hw;
     }
 }
@@ -1114,24 +1367,27 @@ __global__ void k_row_norm2(const float* __restrict__ sv, const uint8_t* __restr
     if (threadIdx.x == 0) out[b] = s;
 }
 
-constexpr size_t nchw_smem(int stages) { return size_t(stages) * kStageCap + 2 * size_t(stages) * sizeof(uint64_t) + 128; }
+constexpr size_t nchw_smem(int stages, bool listed) {
+    return size_t(stages) * kStageCap + 2 * size_t(stages) * sizeof(uint64_t) + 128 +
+           (listed ? (kListFrames + 33) * sizeof(int) : 0);
+}
 
 template <class R>
 cudaError_t launch_nchw(const NchwParams& p, int grid, cudaStream_t st) {
-    return launch_chained(k_encode_nchw<R>, grid, (p.consumers + 1) * kWarp, nchw_smem(p.stages), st, p);
+    return launch_chained(k_encode_nchw<R>, grid, (p.consumers + 1) * kWarp, nchw_smem(p.stages, p.skip != nullptr), st, p);
 }
 
 template <class R>
 cudaError_t opt_in() {
-    return cudaFuncSetAttribute(k_encode_nchw<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemTma));
+    return cudaFuncSetAttribute(k_encode_nchw<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(nchw_smem(kStages, true)));
 }
 
 template <class E>
-cudaError_t launch_generic(const EncodeArgs& a, cudaStream_t st) {
+cudaError_t launch_nhwc_generic(const EncodeArgs& a, cudaStream_t st) {
     const long long total = (long long)a.B * a.C;
     const int grid = int(std::min<long long>((total + 255) / 256, 148 * 16));
-    return launch_chained(k_encode_generic<E>, grid, 256, 0, st, a.x, a.skip, a.sv, a.B, a.C, a.H * a.W,
-                          int(a.layout == SMTM_NHWC), 1.0f / float(a.H * a.W), a.clock);
+    return launch_chained(k_encode_nhwc_generic<E>, grid, 256, 0, st, a.x, a.skip, a.sv, a.B, a.C, a.H * a.W,
+                          1.0f / float(a.H * a.W), a.clock);
 }
 
 template <class E>
@@ -1157,8 +1413,37 @@ int pow2_floor(int v) {
 constexpr int kMaxInFlight = 4;
 
 // Which reducer a shape is served by, and the chunking that goes with it.
-enum Reducer { kNone, kUnitBf16x49, kUnitBf16x196, kUnitF16x49, kUnitF16x196, kUnitF32x49, kTeamF32, kTeamF16, kTeamBf16 };
+enum Reducer {
+    kNone, kUnitBf16x49, kUnitBf16x196, kUnitF16x49, kUnitF16x196, kUnitF32x49, kTeamF32, kTeamF16, kTeamBf16,
+    kEdgeF32, kEdgeF16, kEdgeBf16, kLaneF32, kLaneF16, kLaneBf16
+};
 
+bool unit_reducer(Reducer r) { return r >= kUnitBf16x49 && r <= kUnitF32x49; }
+bool any_width_reducer(Reducer r) { return r >= kEdgeF32; }  // channels that are no whole 16-byte vectors
+
+Reducer of_type(Reducer f32, int dtype) { return Reducer(f32 + (dtype == SMTM_F32 ? 0 : dtype == SMTM_F16 ? 1 : 2)); }
+
+// The reducer of channels that are no whole vectors.
+Reducer any_width_of(int ch_bytes, int dtype) { return of_type(ch_bytes < 128 ? kLaneF32 : kEdgeF32, dtype); }
+
+// Channels of H*W elements whose bytes together are a multiple of 16.
+int aligned_channels(int ch_bytes) {
+    int g = 1;
+    while ((g * ch_bytes) % 16) g *= 2;
+    return g;
+}
+
+// Lanes that share a channel: eight (128 bytes in a row), fewer when it has fewer whole vectors, one below 128 bytes
+// where it has edges.
+int team_lanes(int ch_bytes) { return ch_bytes % 16 == 0 ? std::min(8, pow2_floor(ch_bytes / 16)) : ch_bytes < 128 ? 1 : 8; }
+
+// Channels a chunk of at most `cap` bytes holds, in multiples of `gran` where it holds one.
+int channels_in(int cap, int ch_bytes, int gran) {
+    const int cc = cap / ch_bytes;
+    return cc > gran ? cc - cc % gran : cc;
+}
+
+// The plan of the kernels that take a frame's chunks one by one: every chunk begins on a 16-byte boundary.
 Reducer plan_nchw(const EncodeArgs& a, NchwParams* p) {
     const int HW = a.H * a.W;
     const int es = a.dtype == SMTM_F32 ? 4 : 2;
@@ -1170,7 +1455,10 @@ Reducer plan_nchw(const EncodeArgs& a, NchwParams* p) {
     p->sv_lo = static_cast<__nv_bfloat16*>(a.sv_lo);
     p->status = a.status;
     p->clock = a.clock;
+    p->B = a.B;
     p->C = a.C;
+    p->hw = HW;
+    p->es = es;
     p->ch_bytes = HW * es;
     p->frame_bytes = (long long)a.C * p->ch_bytes;
     p->inv_hw = 1.0f / float(HW);
@@ -1178,6 +1466,14 @@ Reducer plan_nchw(const EncodeArgs& a, NchwParams* p) {
     p->stages = (a.ring_stages >= 2 && a.ring_stages <= kStages) ? a.ring_stages : kStages;
     if (p->max_in_flight > p->stages - 1) p->max_in_flight = p->stages - 1;
     p->consumers = (a.ring_consumers >= 1 && a.ring_consumers <= kConsumers) ? a.ring_consumers : kConsumers;
+    p->consumers = std::min(p->consumers, p->stages);
+    // A stage passes from warp to warp unless their number divides the ring's depth.  The warp that is next to use a stage
+    // must not look at its barrier while the copy before is still under way (the parity it waits for would be that of
+    // the copy before that, which is complete): it gets there after a chunk issued stages - consumers later, so that
+    // copy has to have been issued after the one before had landed.
+    if (p->stages % p->consumers) p->max_in_flight = std::min(p->max_in_flight, p->stages - p->consumers);
+    p->team = team_lanes(p->ch_bytes);
+    if (p->ch_bytes > kStageCap - 32) return kNone;  // a channel has to fit a stage, wherever it begins
     // unit-per-lane shapes (compile-time H*W)
     int G = 0;
     if ((HW == 49 || HW == 196) && es == 2) G = HW == 49 ? 8 : 2;
@@ -1185,25 +1481,72 @@ Reducer plan_nchw(const EncodeArgs& a, NchwParams* p) {
     if (G && a.C % G == 0) {
         p->chunk_channels = 32 * G;
         p->chunks_per_frame = (a.C + p->chunk_channels - 1) / p->chunk_channels;
-        p->total_chunks = (long long)a.B * p->chunks_per_frame;
         if (es == 4) return kUnitF32x49;
         if (a.dtype == SMTM_BF16) return HW == 49 ? kUnitBf16x49 : kUnitBf16x196;
         return HW == 49 ? kUnitF16x49 : kUnitF16x196;
     }
-    // team-per-channel: channel bytes a multiple of 16 and at most one stage
-    if (p->ch_bytes % 16 == 0 && p->ch_bytes <= kStageCap) {
-        p->vec_per_channel = p->ch_bytes / 16;
-        p->team = std::min(32, pow2_floor(std::max(1, p->vec_per_channel / 4)));
-        const int per_pass = 32 / p->team;
-        int cc = kStageCap / p->ch_bytes;
-        if (cc > per_pass) cc -= cc % per_pass;
-        p->chunk_channels = std::min(cc, a.C);
+    // team-per-channel: channel bytes a multiple of 16
+    if (p->ch_bytes % 16 == 0) {
+        p->chunk_channels = std::min(channels_in(kStageCap, p->ch_bytes, 32 / p->team), a.C);
         p->chunks_per_frame = (a.C + p->chunk_channels - 1) / p->chunk_channels;
-        p->total_chunks = (long long)a.B * p->chunks_per_frame;
-        return a.dtype == SMTM_F32 ? kTeamF32 : a.dtype == SMTM_F16 ? kTeamF16 : kTeamBf16;
+        return of_type(kTeamF32, a.dtype);
     }
-    return kNone;
+    // any other width: runs of channels that are whole 16-byte pieces, which a stage has to hold
+    const int run = aligned_channels(p->ch_bytes);
+    // (channels below one 16-byte piece are left to the plain route: a 2x2 map of 512 channels is 4 KB, and the fused
+    // kernel takes 8 us for 128 such frames, pooling and scoring apart 6)
+    if (a.C % run || run * p->ch_bytes > kStageCap || p->ch_bytes < 16) return kNone;
+    p->chunk_channels = std::min(channels_in(kStageCap, p->ch_bytes, std::max(run, 32 / p->team)), a.C);
+    p->chunk_channels -= p->chunk_channels % run;
+    p->chunks_per_frame = (a.C + p->chunk_channels - 1) / p->chunk_channels;
+    return any_width_of(p->ch_bytes, a.dtype);
 }
+
+// Short channels in batches below this many bytes are pooled without the ring: 128 frames of 512 4x4 channels (2 MB)
+// take 2.3 us straight from global memory and 4.3 us through the ring, 128 frames of 256 8x8 channels (4 MB) 2.8 and
+// 4.5, 256 of them (8 MB) 4.3 and 5.4; 32 frames of 2048 7x7 channels (6 MB) 4.4 and 3.8.  With longer channels the ring
+// is never slower.
+constexpr long long kRingLeast = 4ll << 20;
+
+// The plan of k_encode_nchw, or kNone where k_pool_direct serves.  Chunks may begin anywhere in a 16-byte piece (the copy is widened to whole pieces, which
+// lie inside the frame when its bytes are a multiple of 16), so every channel that fits a stage is served.  Chunks are cut so that every CTA gets the same number of nearly equal ones.
+Reducer plan_ring(const EncodeArgs& a, int grid, NchwParams* p) {
+    Reducer r = plan_nchw(a, p);
+    if (p->ch_bytes > kStageCap - 32 || (p->ch_bytes <= 128 && a.B * p->frame_bytes < kRingLeast)) return kNone;
+    if (r == kNone) r = any_width_of(p->ch_bytes, a.dtype);
+    if (p->frame_bytes % 16) return kNone;  // (with and without flags alike: a channel's sum does not depend on them)
+    const bool flat = !a.skip && (long long)a.B * a.C < (1ll << 30);
+    if (flat) {
+        p->frame_bytes *= a.B;
+        p->C *= a.B;
+        p->B = 1;
+    }
+    int gran = 1;  // channels a warp takes in one go
+    if (unit_reducer(r)) gran = p->chunk_channels / 32;
+    else gran = 32 / p->team;
+    int most = unit_reducer(r) ? p->chunk_channels : channels_in(any_width_reducer(r) ? kStageCap - 32 : kStageCap, p->ch_bytes, gran);
+    most = std::min(most, p->C);
+    const int runs = flat ? grid : 1;  // with flags: whole frames, dealt out chunk by chunk
+    const int rounds = (p->C + runs * most - 1) / (runs * most);
+    const int even = (p->C + runs * rounds - 1) / (runs * rounds);
+    p->chunk_channels = std::max(1, std::min(most, (even + gran - 1) / gran * gran));
+    p->chunks_per_frame = (p->C + p->chunk_channels - 1) / p->chunk_channels;
+    return r;
+}
+
+#define SMTM_FOR_TEAM_REDUCER(r, CALL)                              \
+    switch (r) {                                                    \
+        case kTeamF32: CALL(TeamVectors<F32, false>); break;        \
+        case kTeamF16: CALL(TeamVectors<F16, false>); break;        \
+        case kTeamBf16: CALL(TeamVectors<BF16, false>); break;      \
+        case kEdgeF32: CALL(TeamVectors<F32, true>); break;         \
+        case kEdgeF16: CALL(TeamVectors<F16, true>); break;         \
+        case kEdgeBf16: CALL(TeamVectors<BF16, true>); break;       \
+        case kLaneF32: CALL(LanePerChannel<F32>); break;            \
+        case kLaneF16: CALL(LanePerChannel<F16>); break;            \
+        case kLaneBf16: CALL(LanePerChannel<BF16>); break;          \
+        default: break;                                             \
+    }
 
 #define SMTM_FOR_REDUCER(r, CALL)                                   \
     switch (r) {                                                    \
@@ -1212,10 +1555,7 @@ Reducer plan_nchw(const EncodeArgs& a, NchwParams* p) {
         case kUnitF16x49: CALL(UnitPerLane<F16, 49>); break;        \
         case kUnitF16x196: CALL(UnitPerLane<F16, 196>); break;      \
         case kUnitF32x49: CALL(UnitPerLane<F32, 49>); break;        \
-        case kTeamF32: CALL(TeamPerChannel<F32>); break;            \
-        case kTeamF16: CALL(TeamPerChannel<F16>); break;            \
-        case kTeamBf16: CALL(TeamPerChannel<BF16>); break;          \
-        default: break;                                             \
+        default: SMTM_FOR_TEAM_REDUCER(r, CALL)                     \
     }
 
 template <class R>
@@ -1259,7 +1599,7 @@ cudaError_t encode_setup() {
     if (e == cudaSuccess) e = opt_in<__VA_ARGS__>();            \
     if (e == cudaSuccess) e = carveout_pipelined<__VA_ARGS__>();  \
     if (e == cudaSuccess) e = opt_in_fused<__VA_ARGS__>();
-    for (int r = kUnitBf16x49; r <= kTeamBf16; ++r) SMTM_FOR_REDUCER(r, SMTM_OPT_IN)
+    for (int r = kUnitBf16x49; r <= kLaneBf16; ++r) SMTM_FOR_REDUCER(r, SMTM_OPT_IN)
 #undef SMTM_OPT_IN
     return e;
 }
@@ -1277,7 +1617,7 @@ cudaError_t launch_encode(const EncodeArgs& a, int sm_count, cudaStream_t st, in
         }
     } else {
         NchwParams p;
-        const Reducer r = plan_nchw(a, &p);
+        const Reducer r = plan_ring(a, sm_count, &p);
         if (r != kNone) {
             cudaError_t e = cudaSuccess;
             if (wrote_split) *wrote_split = p.sv_hi != nullptr;
@@ -1286,10 +1626,27 @@ cudaError_t launch_encode(const EncodeArgs& a, int sm_count, cudaStream_t st, in
 #undef SMTM_LAUNCH
             return e;
         }
+        p.chunk_channels = std::min(a.C, p.ch_bytes < 1024 && p.team > 1 ? 64 / p.team : 32 / p.team);
+        p.chunks_per_frame = (a.C + p.chunk_channels - 1) / p.chunk_channels;
+        const long long warps = (long long)a.B * p.chunks_per_frame;
+        const int ctas = int(std::min<long long>((warps + 3) / 4, 16LL * sm_count));
+        if (wrote_split) *wrote_split = p.sv_hi != nullptr;
+        const Reducer d = p.ch_bytes % 16 == 0 ? of_type(kTeamF32, a.dtype) : any_width_of(p.ch_bytes, a.dtype);
+        cudaError_t e = cudaErrorInvalidValue;
+#define SMTM_LAUNCH(...) e = launch_chained(k_pool_direct<__VA_ARGS__>, ctas, kDirectThreads, 0, st, p)
+        SMTM_FOR_TEAM_REDUCER(d, SMTM_LAUNCH)
+#undef SMTM_LAUNCH
+        return e;
     }
-    if (a.dtype == SMTM_F32) return launch_generic<F32>(a, st);
-    if (a.dtype == SMTM_F16) return launch_generic<F16>(a, st);
-    return launch_generic<BF16>(a, st);
+    if (a.dtype == SMTM_F32) return launch_nhwc_generic<F32>(a, st);
+    if (a.dtype == SMTM_F16) return launch_nhwc_generic<F16>(a, st);
+    return launch_nhwc_generic<BF16>(a, st);
+}
+
+// Channels of a chunk that must stay in one warp's share when the warps of a CTA divide it.
+static int share_granularity(Reducer r, const NchwParams& p) {
+    if (unit_reducer(r)) return p.chunk_channels / 32;
+    return std::max(any_width_reducer(r) ? aligned_channels(p.ch_bytes) : 1, 32 / std::max(1, p.team));
 }
 
 bool launch_encode_nhwc_vector_supported(const EncodeArgs& a) {
@@ -1297,35 +1654,28 @@ bool launch_encode_nhwc_vector_supported(const EncodeArgs& a) {
     return a.C % (a.dtype == SMTM_F32 ? 4 : 8) == 0;
 }
 
-bool launch_encode_ring_supported(const EncodeArgs& a) {
-    if (a.layout != SMTM_NCHW || a.B <= 0) return false;
-    NchwParams p;
-    return plan_nchw(a, &p) != kNone;
-}
+bool launch_encode_split_supported(const EncodeArgs& a) { return a.layout == SMTM_NCHW && a.B > 0; }
 
 bool launch_pool_sparse_supported(const EncodeArgs& a) {
     if (a.layout != SMTM_NCHW || a.B <= 0) return false;
     NchwParams p;
     const Reducer r = plan_nchw(a, &p);
-    return r != kNone && p.ch_bytes <= kLightStageCap;
+    return r != kNone && (any_width_reducer(r) ? aligned_channels(p.ch_bytes) : 1) * p.ch_bytes <= kLightStageCap;
 }
 
 cudaError_t launch_pool_sparse(const EncodeArgs& a, int sm_count, cudaStream_t st, int64_t* launches) {
     LightParams f{};
+    if (!launch_pool_sparse_supported(a)) return cudaErrorInvalidValue;
     const Reducer r = plan_nchw(a, &f.e);
-    if (r == kNone || f.e.ch_bytes > kLightStageCap) return cudaErrorInvalidValue;
     // chunks of at most kLightStageCap bytes: half the units of a unit-per-lane chunk, or as many whole channels as fit
-    const bool unit = r <= kUnitF32x49;
-    f.gran = unit ? f.e.chunk_channels / 32 : std::max(1, 32 / std::max(1, f.e.team));
-    if (unit) {
+    f.gran = share_granularity(r, f.e);
+    if (unit_reducer(r)) {
         f.e.chunk_channels /= 2;
     } else {
-        int cc = kLightStageCap / f.e.ch_bytes;
-        if (cc > f.gran) cc -= cc % f.gran;
-        f.e.chunk_channels = std::min(cc, a.C);
+        f.e.chunk_channels = std::min(channels_in(kLightStageCap, f.e.ch_bytes, f.gran), a.C);
+        if (any_width_reducer(r)) f.e.chunk_channels -= f.e.chunk_channels % aligned_channels(f.e.ch_bytes);
     }
     f.e.chunks_per_frame = (a.C + f.e.chunk_channels - 1) / f.e.chunk_channels;
-    f.e.total_chunks = (long long)a.B * f.e.chunks_per_frame;
     // about four CTAs to an SM; enough groups that no CTA is given more frames than it can list
     const int cpf = f.e.chunks_per_frame;
     int groups = std::max(1, std::min(a.B, 8 * sm_count / cpf));
@@ -1346,7 +1696,7 @@ Reducer plan_sparse(const EncodeArgs& e, const LookupArgs& a, SparseParams* f) {
     const Reducer r = plan_nchw(e, &f->e);
     if (r == kNone) return kNone;
     if (f->e.chunks_per_frame > kMaxCluster || (f->e.chunk_channels & 3) || f->e.chunk_channels > kSparseSlice) return kNone;
-    f->gran = r <= kUnitF32x49 ? f->e.chunk_channels / 32 : std::max(1, 32 / std::max(1, f->e.team));
+    f->gran = share_granularity(r, f->e);
     return r;
 }
 
@@ -1406,7 +1756,7 @@ cudaError_t launch_lookup_fused(const EncodeArgs& e, const LookupArgs& a, int sm
     // Parts per frame = CTAs per cluster.  A part must fit the scorers' registers (slice <= kMaxSlice
     // channels, a multiple of 4) and the CTA's shared memory; among 1, 2, 4, 8 take the smallest
     // that keeps the SMs 95 % busy over the rounds of frames (else the busiest).
-    static_assert(kTeamBf16 < 16 && kMaxCluster < 9, "FusedCaps holds an entry per (reducer, cluster size)");
+    static_assert(kLaneBf16 < 16 && kMaxCluster < 9, "FusedCaps holds an entry per (reducer, cluster size)");
     int best_P = 0, best_grid = 0;
     double best_eff = -1.0;
     for (int P = 1; P <= kMaxCluster; P *= 2) {

@@ -110,8 +110,8 @@ cudaError_t launch_encode(const EncodeArgs& a, int sm_count, cudaStream_t st, in
                           bool* wrote_split = nullptr);
 // Whether launch_encode serves the NHWC shape with the kernel that reads whole 16-byte pieces of a pixel's row.
 bool launch_encode_nhwc_vector_supported(const EncodeArgs& a);
-// Whether launch_encode serves the shape with the streaming ring, whose depth the ring_* fields set.
-bool launch_encode_ring_supported(const EncodeArgs& a);
+// Whether launch_encode serves the layout with kernels that write the vectors' bf16 split too.
+bool launch_encode_split_supported(const EncodeArgs& a);
 // Asks that SMs running `kernel` be configured with as much shared memory as they can have.  Kernels that
 // are meant to share an SM with a streaming kernel (whose CTAs need most of it) must not leave the SM in a
 // configuration with less: a CTA of the streaming kernel would wait until the SM has drained.
