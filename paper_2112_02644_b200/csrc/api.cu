@@ -260,11 +260,11 @@ smtm_status_t pooled_first_lookup(smtm_cache* c, const EncodeArgs& e, const Look
         SMTM_CUDA(launch_score_exit(a, st, &c->launches, kPipelinedScoreThreads));
         return SMTM_OK;
     }
-    float *dots = nullptr, *dots2 = nullptr;
+    DenseDots dots{};
     SMTM_CUDA(launch_dense_dots(a.sv, nullptr, a.B, a.centers, a.n, a.D, c->d_dense, c->max_batch, c->d_max, cur, sv_split,
-                                c->ev_pool, c->d_cen_split[a.layer], &dots, &dots2, c->d_status,
+                                c->ev_pool, c->d_cen_split[a.layer], &dots, c->d_status,
                                 a.clock ? a.clock + 2 * SMTM_PROF_SCORE_TC : nullptr, kPipelinedDenseTcStages, st, &c->launches));
-    SMTM_CUDA(launch_finish_dense(a, dots, dots2, true, st, &c->launches));
+    SMTM_CUDA(launch_finish_dense(a, dots, true, st, &c->launches));
     return SMTM_OK;
 }
 
@@ -296,7 +296,7 @@ smtm_status_t lookup_impl(smtm_cache* c, int32_t layer, const smtm_fmap_t* f, co
     a.S = c->S;
     a.status = c->d_status;
     EncodeArgs e = encode_args(c, f, b->d_done, b->d_sv[layer]);
-    bool fused = false;
+    LookupServed served = kNotServed;
     const cudaEvent_t* timing = nullptr;
     bool profiled_step_begins = false;
     // The pipelined route: a cache whose caller keeps the maps resident and alternates its carries
@@ -351,9 +351,9 @@ smtm_status_t lookup_impl(smtm_cache* c, int32_t layer, const smtm_fmap_t* f, co
         e.clock = a.clock ? a.clock + 2 * layer : nullptr;
         return pooled_first_lookup(c, e, a, st, timing, profiled_step_begins, true);
     }
-    SMTM_CUDA(launch_lookup_fused(e, a, c->sm_count, &c->fused_caps, st, &c->launches, &fused, timing));
-    if (fused) {
-        ++c->routes[SMTM_ROUTE_FUSED];
+    SMTM_CUDA(launch_lookup_fused(e, a, c->sm_count, &c->fused_caps, st, &c->launches, &served, timing));
+    if (served != kNotServed) {
+        ++c->routes[served == kServedFused ? SMTM_ROUTE_FUSED : SMTM_ROUTE_PLAIN];
         return SMTM_OK;
     }
     ++c->routes[dense ? SMTM_ROUTE_DENSE : SMTM_ROUTE_PLAIN];
@@ -366,11 +366,11 @@ smtm_status_t lookup_impl(smtm_cache* c, int32_t layer, const smtm_fmap_t* f, co
     SMTM_CUDA(launch_encode(e2, c->sm_count, st, &c->launches, &sv_split));
     if (timing) SMTM_CUDA(record_timing(timing[1], st));
     if (dense) {
-        float *dots = nullptr, *dots2 = nullptr;
+        DenseDots dots{};
         SMTM_CUDA(launch_dense_dots(a.sv, a.fresh ? nullptr : a.done, a.B, a.centers, a.n, a.D, c->d_dense, c->max_batch, c->d_max,
-                                    c->split_which, sv_split, nullptr, c->d_cen_split[layer], &dots, &dots2, c->d_status,
+                                    c->split_which, sv_split, nullptr, c->d_cen_split[layer], &dots, c->d_status,
                                     a.clock ? a.clock + 2 * SMTM_PROF_SCORE_TC : nullptr, 0, st, &c->launches));
-        SMTM_CUDA(launch_finish_dense(a, dots, dots2, false, st, &c->launches));
+        SMTM_CUDA(launch_finish_dense(a, dots, false, st, &c->launches));
         return SMTM_OK;
     }
     SMTM_CUDA(launch_score_exit(a, st, &c->launches));
@@ -526,7 +526,7 @@ smtm_status_t smtm_cache_create(const smtm_config_t* cfg, const float* const* h_
     for (int l = 0; ok && l < c->L; ++l) {
         const size_t nd = size_t(n) * c->dims[l];
         ok = ok && dev_alloc(&c->d_centers[l], nd) == cudaSuccess;
-        ok = ok && dev_alloc(&c->d_cnorm[l], n) == cudaSuccess;
+        ok = ok && dev_alloc(&c->d_cnorm[l], dense_row(n)) == cudaSuccess;  // (read in 16-byte pieces)
         ok = ok && dev_alloc(&c->d_m[l], n) == cudaSuccess;
     }
     ok = ok && dev_alloc(&c->d_ft, size_t(S) * n) == cudaSuccess;
@@ -573,6 +573,7 @@ smtm_status_t smtm_cache_create(const smtm_config_t* cfg, const float* const* h_
         if (e == cudaSuccess)
             e = cudaMemcpy(c->d_m[l], (h_counts && h_counts[l]) ? h_counts[l] : ones.data(), n * sizeof(uint32_t),
                            cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemset(c->d_cnorm[l], 0, dense_row(n) * sizeof(float));
         if (e == cudaSuccess) e = launch_center_norms(c->d_centers[l], n, c->dims[l], c->d_cnorm[l], 0, &c->launches);
         if (e == cudaSuccess) e = split_centres(c, l, 0);
     }

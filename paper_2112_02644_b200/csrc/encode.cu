@@ -594,9 +594,16 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_
 }
 
 // All threads of all CTAs of the cluster.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
+}
+__device__ __forceinline__ float peer_load(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
 }
 
 template <class R>
@@ -1175,66 +1182,395 @@ __global__ void __launch_bounds__(kLightThreads) k_lookup_sparse(const SparsePar
     if (P > 1) cluster_sync_all();  // no CTA leaves while a peer may still write to its shared memory
 }
 
-// ---- NHWC: direct coalesced loads ----------------------------------------------------------
+// ---- lookup of small frames: a cluster of small CTAs per frame, nothing persistent -----------------
+//
+// With little to stream (shallow exits with tiny maps, a single camera's frame) a lookup is bound by the number of
+// dependent trips to memory and by what a CTA sets up before the first one, not by bytes.  CTA `rank` of the
+// frame's cluster takes a slice of the semantic vector: [exit flag, stream id] -> [its part of the map, the fast
+// memory's size and classes] -> [centre slices, lengths, carries, while the map lands] -> decision.  The partial dot
+// products meet in the first CTA through distributed shared memory, whose first warp decides; a frame that has
+// exited costs CTAs that leave at once.
+constexpr int kFrameWarps = 8;
+constexpr int kFrameThreads = kFrameWarps * kWarp;
+constexpr int kFrameSlice = 8192;           // channels of a slice at most
+constexpr int kFrameStageCap = 64 * 1024;     // bytes of a slice of an NCHW map at most
+constexpr int kFrameStageWanted = 32 * 1024;  // ... that a cluster is enlarged for
+constexpr int kFrameStageLeast = 4 * 1024;    // ... below which it is not enlarged to fill the chip
+constexpr long long kFrameBatchMost = 64ll << 20;  // bytes of the batch above which the streaming kernel takes over
+constexpr int kNhwcPartLeast = 4 * 1024;      // bytes of an NHWC frame's part below which its cluster is not enlarged
+constexpr int kNhwcPartLong = 64 * 1024;      // ... once every SM has a CTA
 
-constexpr int kThreadsNhwc = 256;
+struct FrameParams {
+    NchwParams e;
+    LookupArgs a;
+    int parts;  // P: CTAs per frame
+    int slice;  // channels per CTA
+    int gran;   // channels that must stay in one warp's share
+};
 
-template <class E>
-__global__ void __launch_bounds__(kThreadsNhwc) k_encode_nhwc(const uint8_t* __restrict__ x,
-                                                              const uint8_t* __restrict__ skip,
-                                                              float* __restrict__ sv, int B, int C, int HW,
-                                                              float inv_hw, unsigned long long* clock) {
-    extern __shared__ float part[];  // [phases][min(C, 256 * kPerVec)]
+// What the scorers of a frame fetch before its semantic vector is known: the fast memory's size, the classes of this
+// warp's slots (slot j = warp + kFrameWarps * i in lane i) and, in the warp that decides, of all slots.
+struct FrameSlots {
+    int k, cls_w, ids[2];
+};
+__device__ __forceinline__ FrameSlots fetch_slots(const LookupArgs& a, int sid, bool decides) {
+    FrameSlots s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t* mem = a.members + (size_t)max(sid, 0) * a.k_max;
+    s.k = sid < 0 ? 0 : min(a.k[sid], kFusedMaxK);  // a stream id outside the cache: nothing to score against
+    const int j = warp + kFrameWarps * lane;
+    s.cls_w = j < min(a.k_max, kFusedMaxK) ? mem[j] : 0;
+    s.ids[0] = decides && lane < a.k_max ? mem[lane] : 0;
+    s.ids[1] = decides && lane + kWarp < a.k_max ? mem[lane + kWarp] : 0;
+    return s;
+}
+
+// The pieces of the centres' slices (channels c0 .., n4 16-byte pieces) for `8 >> lg` slots of this warp, from the
+// warp's slot number i0 on; a slot has at most 1 << lg pieces per lane at a time, from piece q0 on.
+__device__ __forceinline__ void fetch_centres(const LookupArgs& a, const FrameSlots& s, int i0, int lg, int c0, int q0, int n4,
+                                              float4 (&c)[8]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const int i = i0 + (e >> lg), q = q0 + lane + (e & ((1 << lg) - 1)) * kWarp;
+        const int cls = __shfl_sync(kFull, s.cls_w, min(i, kWarp - 1));
+        c[e] = (warp + kFrameWarps * i < s.k && q < n4) ? __ldg(reinterpret_cast<const float4*>(a.centers + (size_t)cls * a.D + c0) + q)
+                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
+// Eq. 1's partial dot products of this warp's slots over the slice, into this part's row of the receive buffer in the
+// cluster's first CTA (`row`: its address there).  c: the pieces of the first slots, fetched already.  Eight sums are
+// reduced over the warp together, halving what is left to exchange at every step: nine shuffles for eight.
+__device__ __forceinline__ void score_slots(const LookupArgs& a, const FrameSlots& s, int lg, int c0, int n4,
+                                            const float4* v4, uint32_t row, float4 (&c)[8]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per_trip = 8 >> lg;
+    for (int i0 = 0; warp + kFrameWarps * i0 < s.k; i0 += per_trip) {
+        float d[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) d[e] = 0.f;
+        for (int q0 = 0; q0 < n4; q0 += 8 * kWarp) {  // (once, but for slices of more than 1024 channels)
+            if (i0 > 0 || q0 > 0) fetch_centres(a, s, i0, lg, c0, q0, n4, c);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int q = q0 + lane + (e & ((1 << lg) - 1)) * kWarp;
+                const float4 x = q < n4 ? v4[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+                d[e] = fmaf(c[e].w, x.w, fmaf(c[e].z, x.z, fmaf(c[e].y, x.y, fmaf(c[e].x, x.x, d[e]))));
+            }
+        }
+        if (lg >= 1) { d[0] += d[1]; d[2] += d[3]; d[4] += d[5]; d[6] += d[7]; }
+        if (lg >= 2) { d[0] += d[2]; d[4] += d[6]; }
+        if (lg >= 3) d[0] += d[4];
+#pragma unroll
+        for (int o = 16, half = 4; half > 0; o >>= 1, half >>= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int e = 0; e < half; ++e) {
+                const float give = up ? d[e] : d[e + half], keep = up ? d[e + half] : d[e];
+                d[e] = keep + __shfl_xor_sync(kFull, give, o);
+            }
+        }
+        d[0] += __shfl_xor_sync(kFull, d[0], 2);
+        d[0] += __shfl_xor_sync(kFull, d[0], 1);
+        const int e = lane >> 2, j = warp + kFrameWarps * (i0 + (e >> lg));  // this lane's sum is number lane >> 2
+        if ((lane & 3) == 0 && (e & ((1 << lg) - 1)) == 0 && j < s.k) peer_store(row + j * 4, d[0]);
+    }
+}
+
+// Squared length of the slice, by one warp.
+__device__ __forceinline__ void slice_norm(const float4* v4, int n4, uint32_t row) {
+    const int lane = threadIdx.x & 31;
+    float nn = 0.f;
+    for (int q = lane; q < n4; q += kWarp) {
+        const float4 x = v4[q];
+        nn = fmaf(x.x, x.x, nn); nn = fmaf(x.y, x.y, nn); nn = fmaf(x.z, x.z, nn); nn = fmaf(x.w, x.w, nn);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(kFull, nn, o);
+    if (lane == 0) peer_store(row + kFusedMaxK * 4, nn);
+}
+
+// The decision by the first warp of the cluster's first CTA once every part's row is in: the parts added in rank
+// order, Eq. 1, Eq. 3, top-2, Eq. 4 / Eq. 2, the exit rule.
+__device__ __forceinline__ void decide_parts(const LookupArgs& a, int b, const FrameSlots& s, const float* rx, int P,
+                                             const float (&clen)[2], const float (&sa_old)[2]) {
+    const int lane = threadIdx.x & 31;
+    float nn = 0.f, dots[2] = {0.f, 0.f};
+    for (int r = 0; r < P; ++r) {
+        const float* row = rx + r * kRxRow;
+        nn += row[kFusedMaxK];
+        if (lane < s.k) dots[0] += row[lane];
+        if (lane + kWarp < s.k) dots[1] += row[lane + kWarp];
+    }
+    const float weight = float(1u << a.layer);  // 2^(l-1) with l = layer + 1
+    const float sv_len = __fsqrt_rn(nn);
+    float s_cur[2] = {0.f, 0.f}, s_acc[2] = {0.f, 0.f};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int j = lane + h * kWarp;
+        if (j < s.k) {
+            s_cur[h] = (nn == 0.f || clen[h] == 0.f) ? 0.f : __fdiv_rn(dots[h], __fmul_rn(sv_len, clen[h]));  // Eq. 1
+            s_acc[h] = __fmaf_rn(s_cur[h], weight, sa_old[h]);                                             // Eq. 3
+            a.sa[(size_t)b * a.k_max + j] = s_acc[h];
+        } else if (a.fresh && j < a.k_max) {
+            a.sa[(size_t)b * a.k_max + j] = 0.f;  // unused slots start from zero too
+        }
+    }
+    const Top2 ta = warp_top2_keys(s_acc, s.ids, s.k, lane);
+    Top2 ts{0.f, 0.f, -1, -1};
+    if (a.sep) ts = warp_top2_keys(s_cur, s.ids, s.k, lane);  // only Eq. 2 (a diagnostic) needs it
+    if (lane == 0) decide_from_top2(a, b, ta, ts);
+}
+
+// Lengths of the centres and carries, for the deciding warp (in flight with the centres).
+__device__ __forceinline__ void fetch_lengths(const LookupArgs& a, int b, const FrameSlots& s, float (&clen)[2], float (&sa_old)[2]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int j = lane + h * kWarp;
+        clen[h] = j < s.k ? a.cnorm[s.ids[h]] : 0.f;
+        sa_old[h] = (j < s.k && !a.fresh) ? a.sa[(size_t)b * a.k_max + j] : 0.f;
+    }
+}
+
+// log2 of the 16-byte pieces of a slice per lane, rounded up.
+__device__ __forceinline__ int pieces_log2(int n4) { return n4 <= kWarp ? 0 : n4 <= 2 * kWarp ? 1 : n4 <= 4 * kWarp ? 2 : 3; }
+
+template <class R>
+__global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FrameParams f) {
+    extern __shared__ __align__(128) uint8_t frame_smem[];  // the map's slice | [slice] semantic vector | [P][kRxRow] receive rows
+    __shared__ uint64_t landed[kFrameWarps];  // per warp: its share of the map
+    const NchwParams& p = f.e;
+    const LookupArgs& a = f.a;
+    const int P = f.parts;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int b = int(blockIdx.x) / P, rank = int(blockIdx.x) - b * P;
+    // this warp's share of the slice's channels
+    const int c0 = rank * f.slice, nch = max(0, min(f.slice, p.C - c0));
+    const int groups = (nch + f.gran - 1) / f.gran;
+    const int share = (groups + kFrameWarps - 1) / kFrameWarps * f.gran;
+    const int w_c0 = min(nch, warp * share), w_nch = min(nch, w_c0 + share) - w_c0;
+    const uint64_t stream_once = l2_evict_first_policy();
+    if (lane == 0) {
+        mbar_init(&landed[warp], 1);
+        mbar_init_fence();
+    }
+    __syncwarp();
     chain_wait();
     chain_release();
-    const ClockScope stamps(clock);
+    const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);
+    const int sid_raw = a.stream_id ? a.stream_id[b] : 0;  // in flight with the exit flag
+    // (no CTA of the cluster can have decided yet: the decision comes after a barrier all of them arrive on)
+    if (!a.fresh && a.done[b]) return;
+    if (P > 1) cluster_arrive();  // (waited for before the first store to a peer: it has to have started)
+    const uint32_t bytes = uint32_t(w_nch) * uint32_t(p.ch_bytes);
+    uint8_t* stage = frame_smem + size_t(w_c0) * p.ch_bytes;
+    if (lane == 0 && bytes) {
+        mbar_expect_tx(&landed[warp], bytes);
+        bulk_load_hint(stage, p.x + (long long)b * p.frame_bytes + (long long)(c0 + w_c0) * p.ch_bytes, bytes, &landed[warp],
+                       stream_once);
+    }
+    float* sv_s = reinterpret_cast<float*>(frame_smem + ((size_t(f.slice) * p.ch_bytes + 15) & ~size_t(15)));
+    float* rx = sv_s + f.slice;
+    const bool decides = rank == 0 && warp == 0;
+    const int sid = stream_checked(a, sid_raw);
+    const FrameSlots slots = fetch_slots(a, sid, decides);
+    const int n4 = nch >> 2, lg = pieces_log2(n4);
+    float4 cen[8];
+    fetch_centres(a, slots, 0, lg, c0, 0, n4, cen);
+    float clen[2] = {0.f, 0.f}, sa_old[2] = {0.f, 0.f};
+    if (decides) fetch_lengths(a, b, slots, clen, sa_old);
+    if (bytes) {
+        if (!mbar_wait_bounded(&landed[warp], 0, p.status)) mbar_wait_bounded(&landed[warp], 0, p.status);  // (let the copy land before leaving)
+        R::run(stage, 0, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, sv_s + w_c0, p.inv_hw, p);
+    }
+    __syncthreads();
+    if (P > 1) cluster_wait();
+    const uint32_t row = peer_smem(rx + rank * kRxRow, 0);
+    const float4* v4 = reinterpret_cast<const float4*>(sv_s);
+    if (warp == kFrameWarps - 1) slice_norm(v4, n4, row);
+    score_slots(a, slots, lg, c0, n4, v4, row, cen);
+    if (P > 1) cluster_sync_all(); else __syncthreads();  // every part has been delivered
+    if (decides) decide_parts(a, b, slots, rx, P, clen, sa_old);
+}
+
+// ---- NHWC: direct coalesced loads ----------------------------------------------------------
+
+// ---- NHWC, small fast memory: pooling, scoring and the decision by a cluster per frame ---------------
+//
+// A frame of an NHWC map is H*W rows of C channels: pooling is a column sum.  CTA `rank` of the frame's cluster sums a
+// run of pixels (thread = 16-byte column group and pixel phase, several loads in flight), the phases are added in
+// ascending order through shared memory, and then CTA r adds slice r of the columns over the cluster's CTAs in rank
+// order (distributed shared memory) and goes on with that slice as the NCHW kernel above does.
+struct FrameNhwcParams {
+    const uint8_t* x;
+    LookupArgs a;
+    float* sv;
+    int C, HW;
+    float inv_hw;
+    int parts;   // P: CTAs per frame
+    int pixels;  // per CTA
+    int slice;   // channels per CTA (a multiple of 4)
+};
+
+// First round of adding the phases' column sums up, so that narrow maps (24 channels of 16 bits: 85 phases in 256 threads)
+// do not leave most threads idle: thread (g, c) adds the phases g, g + groups, ... in place.  Returns the rows that are
+// left to add.
+template <int T>
+__device__ __forceinline__ int fold_phases(float* part, int phases, int cols) {
+    const int groups = T / cols;
+    if (groups <= 1 || phases <= 8) return phases;
+    const int g = threadIdx.x / cols, c = threadIdx.x - g * cols;
+    if (g < groups) {
+        float s = part[threadIdx.x];
+        for (int q = g + groups; q < phases; q += groups) s += part[q * cols + c];
+        part[threadIdx.x] = s;
+    }
+    __syncthreads();
+    return groups;
+}
+
+// Sums pixels [px0, px1) of a frame over this CTA; emit(c, sum) gets each column's; `part`: T / cgs x cgs * V floats.
+template <class E, int T, class Emit>
+__device__ __forceinline__ void column_sums(const uint8_t* frame, int C, int px0, int px1, float* part, Emit emit) {
     constexpr int V = E::kPerVec;
-    const int CG = C / V;            // 16-byte vectors per pixel
-    for (int b = blockIdx.x; b < B; b += gridDim.x) {
-        if (skip && skip[b]) continue;
-        const uint4* f = reinterpret_cast<const uint4*>(x + (long long)b * HW * C * E::kSize);
-        for (int cg0 = 0; cg0 < CG; cg0 += kThreadsNhwc) {
-            const int cgs = min(CG - cg0, kThreadsNhwc);  // channel groups handled in this sweep
-            const int phases = kThreadsNhwc / cgs;
-            const int ph = threadIdx.x / cgs, cg = threadIdx.x - ph * cgs;
+    constexpr int U = 8;  // loads in flight per thread
+    const int CG = C / V;  // 16-byte vectors per pixel
+    const uint4* f = reinterpret_cast<const uint4*>(frame);
+    for (int cg0 = 0; cg0 < CG; cg0 += T) {
+        const int cgs = min(CG - cg0, T);  // column groups handled in this sweep
+        const int phases = T / cgs;
+        const int ph = threadIdx.x / cgs, cg = threadIdx.x - ph * cgs;
+        if (ph < phases) {
             float acc[V];
 #pragma unroll
             for (int j = 0; j < V; ++j) acc[j] = 0.f;
-            if (ph < phases) {
-                const uint4* col = f + cg0 + cg;
-                int px = ph;
-                for (; px + 3 * phases < HW; px += 4 * phases) {
-                    const uint4 v0 = load_once(col + (long long)px * CG);
-                    const uint4 v1 = load_once(col + (long long)(px + phases) * CG);
-                    const uint4 v2 = load_once(col + (long long)(px + 2 * phases) * CG);
-                    const uint4 v3 = load_once(col + (long long)(px + 3 * phases) * CG);
+            const uint4* col = f + cg0 + cg;
+            int px = px0 + ph;
+            for (; px + (U - 1) * phases < px1; px += U * phases) {
+                uint4 v[U];
 #pragma unroll
-                    for (int j = 0; j < V; ++j) acc[j] += E::at(v0, j);
+                for (int u = 0; u < U; ++u) v[u] = load_once(col + (long long)(px + u * phases) * CG);
 #pragma unroll
-                    for (int j = 0; j < V; ++j) acc[j] += E::at(v1, j);
+                for (int u = 0; u < U; ++u)
 #pragma unroll
-                    for (int j = 0; j < V; ++j) acc[j] += E::at(v2, j);
-#pragma unroll
-                    for (int j = 0; j < V; ++j) acc[j] += E::at(v3, j);
-                }
-                for (; px < HW; px += phases) {
-                    const uint4 v = load_once(col + (long long)px * CG);
-#pragma unroll
-                    for (int j = 0; j < V; ++j) acc[j] += E::at(v, j);
-                }
-                float* dst = part + (size_t(ph) * cgs + cg) * V;
-#pragma unroll
-                for (int j = 0; j < V; ++j) dst[j] = acc[j];
+                    for (int j = 0; j < V; ++j) acc[j] += E::at(v[u], j);
             }
-            __syncthreads();
-            for (int c = threadIdx.x; c < cgs * V; c += kThreadsNhwc) {
-                float s = 0.f;
-                for (int q = 0; q < phases; ++q) s += part[size_t(q) * cgs * V + c];
-                sv[(long long)b * C + cg0 * V + c] = s * inv_hw;
+            if (px < px1) {
+                uint4 v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = load_once(col + (long long)min(px + u * phases, px1 - 1) * CG);
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (px + u * phases < px1) {
+#pragma unroll
+                        for (int j = 0; j < V; ++j) acc[j] += E::at(v[u], j);
+                    }
             }
-            __syncthreads();
+            float4* dst = reinterpret_cast<float4*>(part + (size_t(ph) * cgs + cg) * V);
+#pragma unroll
+            for (int j = 0; j < V; j += 4) dst[j / 4] = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
         }
+        __syncthreads();
+        const int cols = cgs * V, rows = fold_phases<T>(part, phases, cols);
+        for (int c = threadIdx.x; c < cols; c += T) {
+            float s = 0.f;
+            for (int q = 0; q < rows; ++q) s += part[q * cols + c];
+            emit(cg0 * V + c, s);
+        }
+        __syncthreads();
     }
+}
+
+// Pooling alone: CTA `rank` of a frame's cluster sums a run of its pixels, then slice `rank` of the columns over the
+// cluster, as k_lookup_frame_nhwc does.
+// 512 frames of 28x28x512 16-bit maps: 69 us with a CTA of four loads per thread each, 61 us here; 64 of them 54 and 11 us.
+template <class E>
+__global__ void __launch_bounds__(kFrameThreads, 4) k_encode_nhwc(const uint8_t* __restrict__ x, const uint8_t* __restrict__ skip,
+                                                                  float* __restrict__ sv, int C, int HW, float inv_hw, int P,
+                                                                  int pixels, int slice, __nv_bfloat16* hi, __nv_bfloat16* lo,
+                                                                  unsigned long long* clock) {
+    extern __shared__ __align__(16) float nhwc_smem[];  // column sums [C] | phases' sums
+    float* psum = nhwc_smem;
+    const int b = int(blockIdx.x) / P, rank = int(blockIdx.x) - b * P;
+    chain_wait();
+    chain_release();
+    const ClockScope stamps(clock);
+    if (skip && skip[b]) return;  // (the same for the whole cluster)
+    const int px0 = rank * pixels, px1 = min(HW, px0 + pixels);
+    const auto write = [&](int c, float s) {
+        s *= inv_hw;
+        const long long at = (long long)b * C + c;
+        sv[at] = s;
+        if (hi) {
+            const __nv_bfloat16 h = __float2bfloat16_rn(s);
+            hi[at] = h;
+            lo[at] = __float2bfloat16_rn(s - __bfloat162float(h));
+        }
+    };
+    const uint8_t* frame = x + (long long)b * HW * C * E::kSize;
+    if (P == 1) {
+        column_sums<E, kFrameThreads>(frame, C, 0, HW, psum, write);
+        return;
+    }
+    column_sums<E, kFrameThreads>(frame, C, px0, px1, psum + C, [&](int c, float s) { psum[c] = s; });
+    cluster_sync_all();
+    const int c0 = rank * slice, c1 = min(C, c0 + slice);
+    for (int c = c0 + threadIdx.x; c < c1; c += kFrameThreads) {
+        float s = 0.f;
+        for (int r = 0; r < P; ++r) s += peer_load(peer_smem(psum + c, r));
+        write(c, s);
+    }
+    cluster_sync_all();  // no CTA leaves while a peer reads its sums
+}
+
+template <class E>
+__global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame_nhwc(const FrameNhwcParams f) {
+    extern __shared__ __align__(16) float nhwc_smem[];  // column sums [C] | slice [slice] | receive rows [P][kRxRow] | phases' sums
+    const LookupArgs& a = f.a;
+    const int P = f.parts;
+    float* psum = nhwc_smem;
+    float* sv_s = psum + f.C;
+    float* rx = sv_s + f.slice;
+    float* part = rx + P * kRxRow;
+    const int warp = threadIdx.x >> 5;
+    const int b = int(blockIdx.x) / P, rank = int(blockIdx.x) - b * P;
+    chain_wait();
+    chain_release();
+    const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);
+    const int sid_raw = a.stream_id ? a.stream_id[b] : 0;  // in flight with the exit flag
+    // (no CTA of the cluster can have decided yet: the decision comes after a barrier all of them arrive on)
+    if (!a.fresh && a.done[b]) return;
+    const bool decides = rank == 0 && warp == 0;
+    const FrameSlots slots = fetch_slots(a, stream_checked(a, sid_raw), decides);  // in flight with the map
+    const int px0 = rank * f.pixels, px1 = min(f.HW, px0 + f.pixels);
+    column_sums<E, kFrameThreads>(f.x + (long long)b * f.HW * f.C * E::kSize, f.C, px0, px1, part,
+                                        [&](int c, float s) { psum[c] = s; });
+    const int c0 = rank * f.slice, nch = max(0, min(f.slice, f.C - c0));
+    const int n4 = nch >> 2, lg = pieces_log2(n4);
+    float4 cen[8];
+    fetch_centres(a, slots, 0, lg, c0, 0, n4, cen);  // in flight with the exchange
+    float clen[2] = {0.f, 0.f}, sa_old[2] = {0.f, 0.f};
+    if (decides) fetch_lengths(a, b, slots, clen, sa_old);
+    if (P > 1) cluster_sync_all();
+    for (int c = threadIdx.x; c < nch; c += kFrameThreads) {
+        float s = 0.f;
+        if (P > 1)
+            for (int r = 0; r < P; ++r) s += peer_load(peer_smem(psum + c0 + c, r));
+        else
+            s = psum[c];
+        s *= f.inv_hw;
+        sv_s[c] = s;
+        f.sv[(long long)b * f.C + c0 + c] = s;
+    }
+    __syncthreads();
+    const uint32_t row = peer_smem(rx + rank * kRxRow, 0);
+    const float4* v4 = reinterpret_cast<const float4*>(sv_s);
+    if (warp == kFrameWarps - 1) slice_norm(v4, n4, row);
+    score_slots(a, slots, lg, c0, n4, v4, row, cen);
+    if (P > 1) cluster_sync_all(); else __syncthreads();  // every part has been delivered (and every peer's sums are read)
+    if (decides) decide_parts(a, b, slots, rx, P, clen, sa_old);
 }
 
 // ---- NHWC, small fast memory: pooling, scoring and the decision by one CTA per frame ---------------
@@ -1293,9 +1629,10 @@ __global__ void __launch_bounds__(kThreadsNhwcLookup) k_lookup_nhwc(const uint8_
             for (int j = 0; j < V; ++j) dst[j] = acc[j];
         }
         __syncthreads();
+        const int rows = fold_phases<T>(part, phases, cgs * V);
         for (int c = threadIdx.x; c < cgs * V; c += T) {
             float s = 0.f;
-            for (int q = 0; q < phases; ++q) s += part[size_t(q) * cgs * V + c];
+            for (int q = 0; q < rows; ++q) s += part[size_t(q) * cgs * V + c];
             s *= inv_hw;
             sv_s[cg0 * V + c] = s;
             sv_out[(long long)b * C + cg0 * V + c] = s;
@@ -1388,15 +1725,6 @@ cudaError_t launch_nhwc_generic(const EncodeArgs& a, cudaStream_t st) {
     const int grid = int(std::min<long long>((total + 255) / 256, 148 * 16));
     return launch_chained(k_encode_nhwc_generic<E>, grid, 256, 0, st, a.x, a.skip, a.sv, a.B, a.C, a.H * a.W,
                           1.0f / float(a.H * a.W), a.clock);
-}
-
-template <class E>
-cudaError_t launch_nhwc(const EncodeArgs& a, cudaStream_t st) {
-    const int CG = a.C / E::kPerVec;
-    const int cgs = std::min(CG, kThreadsNhwc);
-    const size_t smem = size_t(kThreadsNhwc / cgs) * cgs * E::kPerVec * sizeof(float);
-    return launch_chained(k_encode_nhwc<E>, a.B, kThreadsNhwc, smem, st, static_cast<const uint8_t*>(a.x), a.skip, a.sv,
-                          a.B, a.C, a.H * a.W, 1.0f / float(a.H * a.W), a.clock);
 }
 
 int pow2_floor(int v) {
@@ -1558,6 +1886,69 @@ Reducer plan_ring(const EncodeArgs& a, int grid, NchwParams* p) {
         default: SMTM_FOR_TEAM_REDUCER(r, CALL)                     \
     }
 
+#define SMTM_FOR_TYPE(t, CALL)               \
+    switch (t) {                             \
+        case SMTM_F32: CALL(F32); break;     \
+        case SMTM_F16: CALL(F16); break;     \
+        default: CALL(BF16); break;          \
+    }
+
+// The plan of k_lookup_frame: a slice per CTA that is whole 16-byte pieces of the map and of the vector.
+Reducer plan_frame(const EncodeArgs& a, const LookupArgs& l, int sm_count, FrameParams* f) {
+    if (a.layout != SMTM_NCHW || l.k_max > kFusedMaxK || (a.C & 3)) return kNone;
+    const int es = a.dtype == SMTM_F32 ? 4 : 2;
+    if ((long long)a.H * a.W * es > kFrameStageCap) return kNone;
+    (void)plan_nchw(a, &f->e);
+    NchwParams& p = f->e;
+    const int run = aligned_channels(p.ch_bytes);
+    if (a.C % run) return kNone;
+    const int unit = std::max(4, run);
+    const auto slice_of = [&](int parts) { return ((a.C + parts - 1) / parts + unit - 1) / unit * unit; };
+    int best = 0;
+    for (int P = 1; P <= kMaxCluster; P *= 2) {
+        const int slice = slice_of(P);
+        const long long bytes = (long long)slice * p.ch_bytes;
+        if (P > 1 && slice * (P - 1) >= a.C) break;  // a CTA without channels
+        if (slice > kFrameSlice || bytes > kFrameStageCap) continue;
+        best = P;
+        if (bytes <= kFrameStageLeast || (bytes <= kFrameStageWanted && 2LL * a.B * P > sm_count)) break;
+    }
+    if (best == 0 || (long long)a.B * a.C * p.ch_bytes > kFrameBatchMost) return kNone;
+    f->parts = best;
+    f->slice = slice_of(best);
+    f->gran = run;
+    return p.ch_bytes % 16 == 0 ? of_type(kTeamF32, a.dtype) : any_width_of(p.ch_bytes, a.dtype);
+}
+
+// How the clusters of the NHWC kernels divide a frame: pixels between the CTAs, then columns.
+bool plan_frame_nhwc(const EncodeArgs& a, int sm_count, FrameNhwcParams* f) {
+    const int V = a.dtype == SMTM_F32 ? 4 : 8, es = a.dtype == SMTM_F32 ? 4 : 2;
+    if (a.layout != SMTM_NHWC || a.C % V || a.C > 8192) return false;
+    const int HW = a.H * a.W;
+    const long long frame = (long long)HW * a.C * es;
+    int P = 1;
+    while (P < kMaxCluster && 2 * P <= HW &&
+           (((long long)a.B * P < sm_count && frame / (2 * P) >= kNhwcPartLeast) ||
+            ((long long)a.B * P < 4 * sm_count && frame / (2 * P) >= kNhwcPartLong)))
+        P *= 2;
+    f->x = static_cast<const uint8_t*>(a.x);
+    f->sv = a.sv;
+    f->C = a.C;
+    f->HW = HW;
+    f->inv_hw = 1.0f / float(HW);
+    f->parts = P;
+    f->pixels = (HW + P - 1) / P;
+    f->slice = ((a.C + P - 1) / P + 3) / 4 * 4;
+    return true;
+}
+
+// Shared memory of the column sums: the sums and the phases' parts.
+size_t nhwc_smem_bytes(const EncodeArgs& a, const FrameNhwcParams*) {
+    const int V = a.dtype == SMTM_F32 ? 4 : 8;
+    const int cgs = std::min(a.C / V, kFrameThreads);
+    return (size_t(a.C) + size_t(kFrameThreads / cgs) * cgs * V) * sizeof(float);
+}
+
 template <class R>
 cudaError_t opt_in_fused() {
     return cudaFuncSetAttribute(k_lookup_nchw<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemLimit));
@@ -1592,9 +1983,19 @@ cudaError_t carveout_pipelined() {
 }
 
 cudaError_t encode_setup() {
-    cudaError_t e = allow_max_dynamic_smem(k_lookup_nhwc<F32>);
-    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_lookup_nhwc<F16>);
-    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_lookup_nhwc<BF16>);
+    cudaError_t e = cudaSuccess;
+#define SMTM_OPT_IN(E)                                                             \
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_lookup_frame_nhwc<E>);      \
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_lookup_frame_nhwc<E>);    \
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_lookup_nhwc<E>);            \
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_encode_nhwc<E>);
+    SMTM_OPT_IN(F32) SMTM_OPT_IN(F16) SMTM_OPT_IN(BF16)
+#undef SMTM_OPT_IN
+#define SMTM_OPT_IN(...)                                                             \
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_lookup_frame<__VA_ARGS__>);   \
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_lookup_frame<__VA_ARGS__>);
+    for (int r = kTeamF32; r <= kLaneBf16; ++r) SMTM_FOR_TEAM_REDUCER(r, SMTM_OPT_IN)
+#undef SMTM_OPT_IN
 #define SMTM_OPT_IN(...)                                        \
     if (e == cudaSuccess) e = opt_in<__VA_ARGS__>();            \
     if (e == cudaSuccess) e = carveout_pipelined<__VA_ARGS__>();  \
@@ -1609,11 +2010,17 @@ cudaError_t launch_encode(const EncodeArgs& a, int sm_count, cudaStream_t st, in
     if (a.B <= 0) return cudaSuccess;
     ++*launches;
     if (a.layout == SMTM_NHWC) {
-        const int V = a.dtype == SMTM_F32 ? 4 : 8;
-        if (a.C % V == 0) {
-            if (a.dtype == SMTM_F32) return launch_nhwc<F32>(a, st);
-            if (a.dtype == SMTM_F16) return launch_nhwc<F16>(a, st);
-            return launch_nhwc<BF16>(a, st);
+        FrameNhwcParams f{};
+        if (plan_frame_nhwc(a, sm_count, &f)) {
+            cudaError_t e = cudaSuccess;
+            if (wrote_split) *wrote_split = a.sv_hi != nullptr;
+#define SMTM_LAUNCH(E) \
+    e = launch_chained_cluster(k_encode_nhwc<E>, a.B * f.parts, kFrameThreads, nhwc_smem_bytes(a, &f), f.parts, st, f.x, a.skip, \
+                               a.sv, a.C, f.HW, f.inv_hw, f.parts, f.pixels, f.slice, static_cast<__nv_bfloat16*>(a.sv_hi), \
+                               static_cast<__nv_bfloat16*>(a.sv_lo), a.clock)
+            SMTM_FOR_TYPE(a.dtype, SMTM_LAUNCH)
+#undef SMTM_LAUNCH
+            return e;
         }
     } else {
         NchwParams p;
@@ -1650,8 +2057,9 @@ static int share_granularity(Reducer r, const NchwParams& p) {
 }
 
 bool launch_encode_nhwc_vector_supported(const EncodeArgs& a) {
-    if (a.layout != SMTM_NHWC || a.B <= 0) return false;
-    return a.C % (a.dtype == SMTM_F32 ? 4 : 8) == 0;
+    if (a.B <= 0) return false;
+    FrameNhwcParams f{};
+    return plan_frame_nhwc(a, 1, &f);
 }
 
 bool launch_encode_split_supported(const EncodeArgs& a) { return a.layout == SMTM_NCHW && a.B > 0; }
@@ -1728,25 +2136,51 @@ cudaError_t launch_lookup_sparse(const EncodeArgs& e, const LookupArgs& a, int s
 }
 
 cudaError_t launch_lookup_fused(const EncodeArgs& e, const LookupArgs& a, int sm_count, FusedCaps* caps, cudaStream_t st,
-                                int64_t* launches, bool* handled, const cudaEvent_t* timing) {
-    *handled = false;
+                                int64_t* launches, LookupServed* served, const cudaEvent_t* timing) {
+    *served = kNotServed;
     if (e.B <= 0 || a.k_max > kFusedMaxK) return cudaSuccess;
     if (e.layout == SMTM_NHWC) {
-        const int V = e.dtype == SMTM_F32 ? 4 : 8;
-        if (e.C % V || e.C > 8192) return cudaSuccess;
-        const int cgs = std::min(e.C / V, kThreadsNhwcLookup);
-        const size_t smem = (size_t(e.C) + 3 * size_t(a.k_max) + size_t(kThreadsNhwcLookup / cgs) * cgs * V) * sizeof(float);
-        const float inv_hw = 1.0f / float(e.H * e.W);
-        const uint8_t* x = static_cast<const uint8_t*>(e.x);
+        FrameNhwcParams f{};
+        if (!plan_frame_nhwc(e, sm_count, &f)) return cudaSuccess;
+        f.a = a;
         cudaError_t err = cudaSuccess;
         if (timing) record_timing(timing[0], st);
-        if (e.dtype == SMTM_F32) err = launch_chained(k_lookup_nhwc<F32>, e.B, kThreadsNhwcLookup, smem, st, x, e.C, e.H * e.W, inv_hw, e.sv, a);
-        else if (e.dtype == SMTM_F16) err = launch_chained(k_lookup_nhwc<F16>, e.B, kThreadsNhwcLookup, smem, st, x, e.C, e.H * e.W, inv_hw, e.sv, a);
-        else err = launch_chained(k_lookup_nhwc<BF16>, e.B, kThreadsNhwcLookup, smem, st, x, e.C, e.H * e.W, inv_hw, e.sv, a);
+        if (f.parts > 1) {
+            const size_t smem = nhwc_smem_bytes(e, &f) + (size_t(f.slice) + size_t(f.parts) * kRxRow) * sizeof(float);
+#define SMTM_LAUNCH(E) err = launch_chained_cluster(k_lookup_frame_nhwc<E>, e.B * f.parts, kFrameThreads, smem, f.parts, st, f)
+            SMTM_FOR_TYPE(e.dtype, SMTM_LAUNCH)
+#undef SMTM_LAUNCH
+        } else {  // frames enough for the chip: a CTA each
+            const int V = e.dtype == SMTM_F32 ? 4 : 8, cgs = std::min(e.C / V, kThreadsNhwcLookup);
+            const size_t smem = (size_t(e.C) + 3 * size_t(a.k_max) + size_t(kThreadsNhwcLookup / cgs) * cgs * V) * sizeof(float);
+#define SMTM_LAUNCH(E) \
+    err = launch_chained(k_lookup_nhwc<E>, e.B, kThreadsNhwcLookup, smem, st, f.x, e.C, f.HW, f.inv_hw, e.sv, a)
+            SMTM_FOR_TYPE(e.dtype, SMTM_LAUNCH)
+#undef SMTM_LAUNCH
+        }
         if (timing) record_timing(timing[1], st);
         ++*launches;
-        *handled = true;
+        *served = kServedFused;
         return err;
+    }
+    {
+        FrameParams f{};
+        const Reducer r = plan_frame(e, a, sm_count, &f);
+        if (r != kNone) {
+            f.a = a;
+            const size_t smem = ((size_t(f.slice) * f.e.ch_bytes + 15) & ~size_t(15)) +
+                                (size_t(f.slice) + size_t(f.parts) * kRxRow) * sizeof(float);
+            cudaError_t err = cudaErrorInvalidValue;
+            if (timing) record_timing(timing[0], st);
+#define SMTM_LAUNCH(...) err = launch_chained_cluster(k_lookup_frame<__VA_ARGS__>, e.B * f.parts, kFrameThreads, smem, f.parts, st, f)
+            SMTM_FOR_TEAM_REDUCER(r, SMTM_LAUNCH)
+#undef SMTM_LAUNCH
+            if (timing) record_timing(timing[1], st);
+            ++*launches;
+            NchwParams streamed;
+            *served = plan_nchw(e, &streamed) != kNone ? kServedFused : kServedPlain;
+            return err;
+        }
     }
     FusedParams f{};
     const Reducer r = plan_nchw(e, &f.e);
@@ -1804,7 +2238,7 @@ cudaError_t launch_lookup_fused(const EncodeArgs& e, const LookupArgs& a, int sm
 #undef SMTM_LAUNCH
     if (timing) record_timing(timing[1], st);
     ++*launches;
-    *handled = true;
+    *served = kServedFused;
     return err;
 }
 

@@ -158,9 +158,10 @@ struct LookupArgs {
 };
 // threads: CTA size (a multiple of 32, at most 256; 0 = 256).  Smaller CTAs fit beside a streaming kernel.
 cudaError_t launch_score_exit(const LookupArgs& a, cudaStream_t st, int64_t* launches, int threads = 0);
-// Encode + score + exit in one kernel (NCHW shapes the streaming pipeline serves, fast
-// memories of at most 64 entries).  *handled is false when the shape is not served, in which
-// case nothing was launched.
+// Encode + score + exit in one kernel (fast memories of at most 64 entries): NCHW shapes the streaming pipeline serves,
+// small NCHW frames of any shape whose slices are whole 16-byte pieces (counted as the plain route where the streaming
+// pipeline does not serve the shape) and NHWC shapes with whole 16-byte pixel rows.  With kNotServed nothing was launched.
+enum LookupServed { kNotServed, kServedFused, kServedPlain };
 constexpr int kFusedMaxK = 64;  // fast-memory capacity the fused path supports (two slots per lane)
 // Lookup (pooling, scoring, decision) of the frames still in at a later layer by clusters of small CTAs that fit
 // beside a streaming kernel: NCHW shapes the streaming pipeline cuts into at most 8 chunks per frame.
@@ -173,11 +174,18 @@ struct FusedCaps {
 };
 // timing: nullptr, or two events recorded on `st` right before and after the kernel.
 cudaError_t launch_lookup_fused(const EncodeArgs& e, const LookupArgs& a, int sm_count, FusedCaps* caps, cudaStream_t st,
-                                int64_t* launches, bool* handled, const cudaEvent_t* timing);
+                                int64_t* launches, LookupServed* served, const cudaEvent_t* timing);
 // ---- large fast memories: dot products against every class on the tensor cores ---------------
 bool dense_scoring_supported(int D, int n);
+int dense_row(int n);  // floats in a row of dot products: n up to a whole number of 16-byte pieces
+// The dot products as the scorer leaves them: `parts` arrays [B][ld], `stride` floats apart, that add up to them.
+struct DenseDots {
+    const float* dots;
+    int ld, parts;
+    size_t stride;
+};
 size_t dense_scratch_bytes(int max_batch, int n, int d_max);
-// DOT[b][c] = <sv[b], centers[c]> for b < B, c < n into scratch; *dots_out = the [B][n] result.
+// DOT[b][c] = <sv[b], centers[c]> for b < B, c < n into scratch; *result says where.
 // The bf16 heads and tails of the semantic vectors sit at the start of scratch, in two sets (see
 // dense_sv_split; `which` picks one); sv_split_done says whether they are already current; sv_ready: nullptr, or
 // an event `st` has to wait for before it reads the vectors or their split (the pooling of the pipelined route).
@@ -189,15 +197,14 @@ cudaError_t launch_centers_split(const float* centers, int n, int D, void* cente
                                  int64_t* launches);
 cudaError_t launch_dense_dots(const float* sv, const uint8_t* skip, int B, const float* centers, int n, int D,
                               void* scratch, int max_batch, int d_max, int which, bool sv_split_done,
-                              cudaEvent_t sv_ready, void* centers_split, float** dots_out, float** dots2_out,
-                              int* status, unsigned long long* clock, int ring_stages, cudaStream_t st,
-                              int64_t* launches);
+                              cudaEvent_t sv_ready, void* centers_split, DenseDots* result, int* status,
+                              unsigned long long* clock, int ring_stages, cudaStream_t st, int64_t* launches);
 size_t dense_centers_split_bytes(int n, int D);
-// Eq. 1 from the dot products, Eq. 3, top-2, Eq. 4 / Eq. 2 and the exit rule; dots: [B][n], and dots2
-// (nullptr, or [B][n]: the second half of the vector length, added to the first).
+// Eq. 1 from the dot products, Eq. 3, top-2, Eq. 4 / Eq. 2 and the exit rule (the parts are added in order; a.cnorm is
+// readable up to dense_row(n)).
 // beside_pooling: the next batch's pooling kernel runs meanwhile (launched in stream order, see launch_ordered).
-cudaError_t launch_finish_dense(const LookupArgs& a, const float* dots, const float* dots2, bool beside_pooling,
-                                cudaStream_t st, int64_t* launches);
+cudaError_t launch_finish_dense(const LookupArgs& a, const DenseDots& dots, bool beside_pooling, cudaStream_t st,
+                                int64_t* launches);
 // One warp that waits, bounded, on a barrier nobody arrives on (the self-test of the time-out path).
 cudaError_t launch_wait_selftest(int* status, cudaStream_t st, int64_t* launches);
 cudaError_t launch_batch_reset(float* sa, uint8_t* done, int32_t* exit_layer, int32_t* pred, int B, int k_max,

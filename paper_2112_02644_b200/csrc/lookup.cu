@@ -68,7 +68,7 @@ __device__ __forceinline__ Top2 block_top2_keys(unsigned long long b1, unsigned 
 }
 
 // Finishing kernel of the tensor-core path: one CTA per frame turns the frame's row of dot products into
-// similarities of its fast-memory slots and decides.  The row (both halves of the vector length added) and the
+// similarities of its fast-memory slots and decides.  The row (its parts added) and the
 // centres' lengths come in with coalesced 16-byte loads and are parked in shared memory, from where the slots
 // pick their class's entry: a gather straight from global memory costs a sector per slot, and a thousand slots
 // for each of a thousand frames are then bound by that.  Everything a frame needs after its stream id is fetched
@@ -77,9 +77,9 @@ __device__ __forceinline__ Top2 block_top2_keys(unsigned long long b1, unsigned 
 // by two warp-wide maxima, the CTA through shared memory.  With a.fresh the carry is taken as SA = 0, nobody done.
 constexpr int kFinishSlots = 4;  // slots a thread fetches per trip
 
-__global__ void __launch_bounds__(kFinishThreads, 10) k_finish_dense(const LookupArgs a, const float* __restrict__ dots,
-                                                                    const float* __restrict__ dots2) {
-    extern __shared__ float s_row[];  // [n] dot products, then [n] lengths of the centres
+template <bool kTwoParts>  // the usual number of parts of a problem that fills the chip
+__global__ void __launch_bounds__(kFinishThreads, kTwoParts ? 10 : 8) k_finish_dense(const LookupArgs a, const DenseDots dd) {
+    extern __shared__ __align__(16) float s_row[];  // [ld] dot products, then [ld] lengths of the centres
     __shared__ float scratch[32];
     __shared__ unsigned long long s_keys[2 * (kFinishThreads / kWarp)];
     chain_wait();
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kFinishThreads, 10) k_finish_dense(const Looku
     const int gone = a.fresh ? 0 : a.done[b];
     const int sid = stream_of(a, b);  // (in flight with the flag)
     if (gone) return;
-    float* s_len = s_row + a.n;
+    float* s_len = s_row + dd.ld;
     const int32_t* mem = a.members + (size_t)max(sid, 0) * a.k_max;
     float* sa_row = a.sa + (size_t)b * a.k_max;
     const float weight = float(1u << a.layer);
@@ -103,15 +103,21 @@ __global__ void __launch_bounds__(kFinishThreads, 10) k_finish_dense(const Looku
         cls[u] = mem[j];
         old[u] = a.fresh ? 0.f : sa_row[j];
     }
-    // ... the row of dot products and the lengths (n is a multiple of 4 on this route) ...
-    const float4* drow = reinterpret_cast<const float4*>(dots + (size_t)b * a.n);
-    const float4* drow2 = dots2 ? reinterpret_cast<const float4*>(dots2 + (size_t)b * a.n) : nullptr;
+    // ... the row of dot products (the parts of the vector length added in order) and the lengths ...
+    const float4* drow = reinterpret_cast<const float4*>(dd.dots + (size_t)b * dd.ld);
     const float4* clen = reinterpret_cast<const float4*>(a.cnorm);
-    for (int c4 = tid; c4 < a.n / 4; c4 += kFinishThreads) {
+    const size_t part = dd.stride / 4;
+    for (int c4 = tid; c4 < dd.ld / 4; c4 += kFinishThreads) {
         float4 d = drow[c4];
-        if (drow2) {  // second half of the vector length
-            const float4 e = drow2[c4];
+        if (kTwoParts) {
+            const float4 e = drow[part + c4];
             d.x += e.x; d.y += e.y; d.z += e.z; d.w += e.w;
+        } else {
+#pragma unroll 4
+            for (int s0 = 1; s0 < dd.parts; ++s0) {
+                const float4 e = drow[s0 * part + c4];
+                d.x += e.x; d.y += e.y; d.z += e.z; d.w += e.w;
+            }
         }
         reinterpret_cast<float4*>(s_row)[c4] = d;
         reinterpret_cast<float4*>(s_len)[c4] = clen[c4];
@@ -195,8 +201,10 @@ cudaError_t launch_wait_selftest(int* status, cudaStream_t st, int64_t* launches
 cudaError_t lookup_setup() {
     cudaError_t e = allow_max_dynamic_smem(k_score_exit);
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_score_exit);
-    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_finish_dense);
-    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_finish_dense);  // (two words per class: 64 KB at 8192 classes)
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_finish_dense<true>);
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_finish_dense<false>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_finish_dense<false>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_finish_dense<true>);  // (two words per class: 64 KB at 8192 classes)
     return e;
 }
 
@@ -209,13 +217,14 @@ cudaError_t launch_batch_reset(float* sa, uint8_t* done, int32_t* exit_layer, in
     return launch_chained(k_batch_reset, grid, 256, 0, st, sa, done, exit_layer, pred, B, n_sa);
 }
 
-cudaError_t launch_finish_dense(const LookupArgs& a, const float* dots, const float* dots2, bool beside_pooling,
-                                cudaStream_t st, int64_t* launches) {
+cudaError_t launch_finish_dense(const LookupArgs& a, const DenseDots& dots, bool beside_pooling, cudaStream_t st,
+                                int64_t* launches) {
     if (a.B <= 0) return cudaSuccess;
     ++*launches;
-    const size_t smem = 2 * size_t(a.n) * sizeof(float);
-    if (beside_pooling) return launch_ordered(k_finish_dense, a.B, kFinishThreads, smem, st, a, dots, dots2);
-    return launch_chained(k_finish_dense, a.B, kFinishThreads, smem, st, a, dots, dots2);
+    const size_t smem = 2 * size_t(dots.ld) * sizeof(float);
+    const auto kernel = dots.parts == 2 ? k_finish_dense<true> : k_finish_dense<false>;
+    if (beside_pooling) return launch_ordered(kernel, a.B, kFinishThreads, smem, st, a, dots);
+    return launch_chained(kernel, a.B, kFinishThreads, smem, st, a, dots);
 }
 
 cudaError_t launch_score_exit(const LookupArgs& a, cudaStream_t st, int64_t* launches, int threads) {

@@ -13,8 +13,9 @@
 // Kernel.  One CTA per 128 x 128 tile of DOT (frames x classes) and half of the vector length:
 // with N = 128 an MMA reads as many bytes of shared memory per cycle as it can use (with N = 64
 // the 128 x 16 slice of A was re-read for half the work and the instruction was operand-bound),
-// and cutting the length in two keeps 128 CTAs busy on the 1024 x 1000 problem.  The two halves
-// go to two result arrays that the finishing kernel adds in a fixed order.  Warp 0 is the TMA
+// and cutting the length in two keeps 128 CTAs busy on the 1024 x 1000 problem.  Small problems have few tiles (256
+// frames x 101 classes: two) and a k-block is 64 KB of operands, a microsecond for one SM, so their length is cut into
+// up to eight parts.  Each part goes to a result array of its own; the finishing kernel adds them in a fixed order.  Warp 0 is the TMA
 // producer (cp.async.bulk.tensor, 128-byte swizzle, three stages of 64 KB), warp 1 allocates
 // tensor memory (4 x 128 fp32 columns) and issues tcgen05.mma (M = 128, N = 128, K = 16,
 // kind::f16 with bf16 inputs), warps 2..5 read the accumulators back with tcgen05.ld and store
@@ -41,8 +42,9 @@ constexpr int kBytesB = kTileN * kTileK * 2;                   // 16 KB
 constexpr int kStageBytes = 2 * kBytesA + 2 * kBytesB;         // hi and lo of both operands
 constexpr int kTcThreads = 6 * kWarp;
 constexpr int kHeadRuns = 3;                                   // accumulators the hi*hi sum is spread over
-constexpr int kSplitK = 2;                                     // CTAs that share the vector length of a tile
+constexpr int kSplitMin = 2, kSplitMax = 8;                   // CTAs that share the vector length of a tile
 constexpr int kAccs = kHeadRuns + 1;                           // ... plus one for the cross terms
+constexpr int kTcCtas = 144;                                   // CTAs a small problem is cut up for
 constexpr int kTmemCols = 512;                                 // power of two >= kAccs * kTileN fp32 columns
 constexpr size_t kTcSmem = size_t(kTcStages) * kStageBytes + 1024 + 256;
 
@@ -118,7 +120,7 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 struct TcParams {
     int M, N, D;       // frames, classes, vector length
     int ld_out;        // floats between rows of `out`
-    float* out;        // [splits][M][ld_out] dot products over each part of the vector length
+    float* out;        // [splits][M][ld_out] dot products over each part of the vector length (ld_out: N up to a multiple of 4)
     size_t split_stride;  // floats between the result arrays of two parts
     int* status;
     unsigned long long* clock;  // nullptr, or two words for the device-clock stamps
@@ -143,6 +145,7 @@ k_score_tc(const __grid_constant__ CUtensorMap map_a_hi, const __grid_constant__
     const int n_kb_all = (p.D + kTileK - 1) / kTileK;
     const int kb0 = int(blockIdx.z) * n_kb_all / int(gridDim.z);
     const int n_kb = (int(blockIdx.z) + 1) * n_kb_all / int(gridDim.z) - kb0;
+    const int runs = min(kHeadRuns, n_kb);  // accumulators of the hi*hi sum in use (a short part has fewer k-blocks than there are)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < stages; ++s) {
@@ -196,7 +199,7 @@ k_score_tc(const __grid_constant__ CUtensorMap map_a_hi, const __grid_constant__
                 tc_fence_after();
                 const uint32_t a_hi = smem_u32(base + size_t(s) * kStageBytes);
                 const uint32_t a_lo = a_hi + kBytesA, b_hi = a_hi + 2 * kBytesA, b_lo = b_hi + kBytesB;
-                const int run = kb * kHeadRuns / n_kb;  // consecutive k-blocks share an accumulator
+                const int run = kb * runs / n_kb;  // consecutive k-blocks share an accumulator
                 // lo*hi and hi*lo into the cross-term accumulator, hi*hi into its run's
                 const uint32_t a_of[3] = {a_lo, a_hi, a_hi};
                 const uint32_t b_of[3] = {b_hi, b_lo, b_hi};
@@ -213,7 +216,6 @@ k_score_tc(const __grid_constant__ CUtensorMap map_a_hi, const __grid_constant__
                 }
                 umma_commit(&empty[s]);  // the stage may be refilled once these MMAs have read it
             }
-            if (!failed && started != (1u << kAccs) - 1u) failed = true;  // fewer k-blocks than runs: not launched
             umma_commit(acc_full);  // accumulator complete
         }
     } else {
@@ -245,13 +247,14 @@ k_score_tc(const __grid_constant__ CUtensorMap map_a_hi, const __grid_constant__
                     float* dst = p.out + size_t(blockIdx.z) * p.split_stride + (size_t)row * p.ld_out + n0 + c0;
 #pragma unroll
                     for (int j = 0; j < 16; j += 4) {
-                        if (n0 + c0 + j < p.N) {  // N and ld_out are multiples of 4
+                        if (n0 + c0 + j < p.ld_out) {  // (the columns that pad a row are zero: their classes were filled with zeros)
                             float o[4];
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 float h = __uint_as_float(r[0][j + e]);
 #pragma unroll
-                                for (int run = 1; run < kHeadRuns; ++run) h += __uint_as_float(r[run][j + e]);
+                                for (int run = 1; run < kHeadRuns; ++run)
+                                    if (run < runs) h += __uint_as_float(r[run][j + e]);
                                 o[e] = h + __uint_as_float(r[kHeadRuns][j + e]);
                             }
                             *reinterpret_cast<float4*>(dst + j) = make_float4(o[0], o[1], o[2], o[3]);
@@ -312,14 +315,29 @@ cudaError_t dense_setup() {
     return e != cudaSuccess ? e : prefer_max_smem_carveout(k_score_tc);
 }
 
-bool dense_scoring_supported(int D, int n) {
-    return D % 8 == 0 && D >= 4 * kTileK && n % 4 == 0 && encode_tiled_fn() != nullptr;
+bool dense_scoring_supported(int D, int) { return D % 8 == 0 && encode_tiled_fn() != nullptr; }
+
+namespace {
+
+int tiles_of(int B, int n) { return ((B + kTileM - 1) / kTileM) * ((n + kTileN - 1) / kTileN); }
+
+// Parts the vector length of a tile is cut into: enough CTAs for the chip, each with a k-block at least.
+int splits_of(int B, int n, int D) {
+    const int n_kb = (D + kTileK - 1) / kTileK;
+    return std::max(1, std::min(n_kb, std::min(kSplitMax, std::max(kSplitMin, kTcCtas / tiles_of(B, n)))));
 }
+
+}  // namespace
+
+int dense_row(int n) { return (n + 3) / 4 * 4; }
 
 size_t dense_scratch_bytes(int max_batch, int n, int d_max) {
     // bf16 heads and tails of the semantic vectors (two sets: the pipelined route pools a batch while the one
-    // before it is still being scored), then the dot products
-    return 2 * size_t(max_batch) * d_max * 2 * 2 + size_t(kSplitK) * max_batch * n * sizeof(float) + 1024;
+    // before it is still being scored), then the dot products: the parts of the largest batch, or of a smaller one
+    // that is cut into more
+    const size_t largest = size_t(std::max(kSplitMin, std::min(kSplitMax, kTcCtas / tiles_of(max_batch, n)))) * max_batch * dense_row(n);
+    const size_t cut = size_t(kTcCtas) * kTileM * kTileN;
+    return 2 * size_t(max_batch) * d_max * 2 * 2 + std::max(largest, std::min(cut, size_t(kSplitMax) * max_batch * dense_row(n))) * sizeof(float) + 1024;
 }
 
 size_t dense_centers_split_bytes(int n, int D) { return size_t(n) * D * 2 * 2; }
@@ -341,9 +359,7 @@ cudaError_t launch_centers_split(const float* centers, int n, int D, void* cente
 
 cudaError_t launch_dense_dots(const float* sv, const uint8_t* skip, int B, const float* centers, int n, int D,
                               void* scratch, int max_batch, int d_max, int which, bool sv_split_done,
-                              cudaEvent_t sv_ready, void* centers_split, float** dots_out, float** dots2_out,
-                              int* status, unsigned long long* clock, int ring_stages, cudaStream_t st,
-                              int64_t* launches) {
+                              cudaEvent_t sv_ready, void* centers_split, DenseDots* result, int* status, unsigned long long* clock, int ring_stages, cudaStream_t st, int64_t* launches) {
     void *hi = nullptr, *lo = nullptr;
     dense_sv_split(scratch, max_batch, d_max, which, &hi, &lo);
     __nv_bfloat16* a_hi = static_cast<__nv_bfloat16*>(hi);
@@ -353,10 +369,11 @@ cudaError_t launch_dense_dots(const float* sv, const uint8_t* skip, int B, const
     float* dots = reinterpret_cast<float*>(
         (reinterpret_cast<uintptr_t>(reinterpret_cast<__nv_bfloat16*>(scratch) + 4 * size_t(max_batch) * d_max) + 255) &
         ~uintptr_t(255));
-    // the vector length is cut in two when each part still has a k-block for every accumulator
-    const int splits = (D + kTileK - 1) / kTileK >= kSplitK * kHeadRuns ? kSplitK : 1;
-    *dots_out = dots;
-    *dots2_out = splits > 1 ? dots + size_t(max_batch) * n : nullptr;
+    const int splits = splits_of(B, n, D);
+    result->dots = dots;
+    result->ld = dense_row(n);
+    result->parts = splits;
+    result->stride = size_t(B) * result->ld;
 
     CUtensorMap ma_hi, ma_lo, mb_hi, mb_lo;
     if (!make_map(&ma_hi, a_hi, B, D, kTileM) || !make_map(&ma_lo, a_lo, B, D, kTileM) ||
@@ -377,9 +394,9 @@ cudaError_t launch_dense_dots(const float* sv, const uint8_t* skip, int B, const
     p.M = B;
     p.N = n;
     p.D = D;
-    p.ld_out = n;
+    p.ld_out = result->ld;
     p.out = dots;
-    p.split_stride = size_t(max_batch) * n;
+    p.split_stride = result->stride;
     p.status = status;
     p.clock = clock;
     p.stages = ring_stages >= 2 && ring_stages <= kTcStages ? ring_stages : kTcStages;
