@@ -21,7 +21,8 @@
 // memory (k_pool_direct).
 // NHWC.  Consecutive 16-byte vectors of a frame are consecutive channel groups of a pixel;
 // each thread owns one channel group and a pixel phase, loads coalesced 128-bit vectors
-// directly and the phases are combined through shared memory in ascending order.
+// directly and the phases are combined through shared memory in a fixed order; few frames are
+// divided between the CTAs of clusters.
 #include <algorithm>
 #include <cmath>
 
@@ -34,7 +35,6 @@ namespace {
 constexpr int kStages = 8;             // ring depth
 constexpr int kConsumers = 8;          // consumer warps; stage s belongs to warp s % kConsumers
 constexpr int kStageCap = 25600;       // bytes per stage
-constexpr int kThreadsTma = (kConsumers + 1) * kWarp;
 
 struct NchwParams {
     const uint8_t* x;
@@ -374,8 +374,10 @@ struct ChunkWalk {
     }
 };
 
+// (At most 128 registers, as for 512 threads: on the pipelined route they decide how many CTAs of the other kernels fit
+// on an SM beside this one.)
 template <class R>
-__global__ void __launch_bounds__(kThreadsTma, 1) k_encode_nchw(const NchwParams p) {
+__global__ void __launch_bounds__(512, 1) k_encode_nchw(const NchwParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
     uint8_t* stages = base;
@@ -1193,8 +1195,10 @@ __global__ void __launch_bounds__(kLightThreads) k_lookup_sparse(const SparsePar
 constexpr int kFrameWarps = 8;
 constexpr int kFrameThreads = kFrameWarps * kWarp;
 constexpr int kFrameSlice = 8192;           // channels of a slice at most
-constexpr int kFrameStageCap = 64 * 1024;     // bytes of a slice of an NCHW map at most
-constexpr int kFrameStageWanted = 32 * 1024;  // ... that a cluster is enlarged for
+constexpr int kFrameStageCap = 104 * 1024;    // bytes of a slice of an NCHW map at most
+// (Slices of up to 64 KB rather than smaller ones in larger clusters: thirteen exits of 128 frames 348 -> 331 us, with 16 KB
+// 417; four exits of 64 larger frames 70 -> 65 us with slices up to 104 KB instead of the streaming kernel.)
+constexpr int kFrameStageWanted = 64 * 1024;  // ... that a cluster is enlarged for
 constexpr int kFrameStageLeast = 4 * 1024;    // ... below which it is not enlarged to fill the chip
 constexpr long long kFrameBatchMost = 64ll << 20;  // bytes of the batch above which the streaming kernel takes over
 constexpr int kNhwcPartLeast = 4 * 1024;      // bytes of an NHWC frame's part below which its cluster is not enlarged

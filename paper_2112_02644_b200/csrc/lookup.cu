@@ -108,19 +108,19 @@ __global__ void __launch_bounds__(kFinishThreads, kTwoParts ? 10 : 8) k_finish_d
     const float4* clen = reinterpret_cast<const float4*>(a.cnorm);
     const size_t part = dd.stride / 4;
     for (int c4 = tid; c4 < dd.ld / 4; c4 += kFinishThreads) {
-        float4 d = drow[c4];
+        float4 d = __ldg(drow + c4);  // (read-only here: the loads need not wait for the stores of the round before)
         if (kTwoParts) {
-            const float4 e = drow[part + c4];
+            const float4 e = __ldg(drow + part + c4);
             d.x += e.x; d.y += e.y; d.z += e.z; d.w += e.w;
         } else {
 #pragma unroll 4
             for (int s0 = 1; s0 < dd.parts; ++s0) {
-                const float4 e = drow[s0 * part + c4];
+                const float4 e = __ldg(drow + s0 * part + c4);
                 d.x += e.x; d.y += e.y; d.z += e.z; d.w += e.w;
             }
         }
         reinterpret_cast<float4*>(s_row)[c4] = d;
-        reinterpret_cast<float4*>(s_len)[c4] = clen[c4];
+        reinterpret_cast<float4*>(s_len)[c4] = __ldg(clen + c4);
     }
     // ... and the squared length of the semantic vector (D is a multiple of 8 on this route)
     const float4* row4 = reinterpret_cast<const float4*>(a.sv + (size_t)b * a.D);

@@ -1,9 +1,14 @@
 """Shapes at the edges of what each kernel serves, against the CPU oracle."""
+import numpy as np
 import pytest
+import torch
+
+import oracle
+import paper_2112_02644_b200 as smtm
 
 import smtm_inputs as si
 import test_gpu_parity as parity
-from harness import run_workload
+from harness import Report, compare_state, run_workload
 
 pytestmark = pytest.mark.gpu
 
@@ -52,19 +57,63 @@ def test_pooling_of_nhwc_maps_by_clusters(dt, B, C, H, W):
     parity.test_encode_matches_oracle(dt, si.NHWC, B, C, H, W)
 
 
-# large fast memories on the tensor cores: class counts that are no multiple of four, vectors of one 16-byte piece and of
-# less than a k-block per part, few tiles cut into many parts, a batch far below the largest
+# large fast memories on the tensor cores: few tiles cut into as many parts as there are k-blocks or into eight, with fewer
+# k-blocks to a part than accumulators; class counts and vectors the plain route scores
 DENSE_LOOKUPS = [
-    si.Workload("dense_101", si.F16, si.NCHW, B=130, stages=((1024, 4, 4), (2048, 2, 2)), n=101, k_init=101, k_min=70,
-                k_max=101, T=3, sigma=0.6, zipf_s=0.9, repeat_p=0.3, seed=61),
-    si.Workload("dense_short", si.BF16, si.NCHW, B=5, stages=((8, 9, 9), (24, 8, 8), (200, 5, 5)), n=67, k_init=66, k_min=65,
-                k_max=67, T=4, tau=0.3, sigma=0.4, zipf_s=0.9, repeat_p=0.3, seed=62),
-    si.Workload("dense_nhwc_601", si.BF16, si.NHWC, B=300, stages=((320, 3, 3), (640, 2, 2)), n=601, k_init=601, k_min=100,
-                k_max=601, T=3, sigma=0.6, zipf_s=0.9, repeat_p=0.3, seed=63),
+    (si.Workload("dense_100", si.F16, si.NCHW, B=130, stages=((1024, 4, 4), (2048, 2, 2)), n=100, k_init=100, k_min=70,
+                 k_max=100, T=3, sigma=0.6, zipf_s=0.9, repeat_p=0.3, seed=61), 1),
+    (si.Workload("dense_short", si.BF16, si.NCHW, B=5, stages=((256, 9, 9), (264, 8, 8), (320, 5, 5)), n=68, k_init=66, k_min=65,
+                 k_max=68, T=4, tau=0.3, sigma=0.4, zipf_s=0.9, repeat_p=0.3, seed=62), 1),
+    (si.Workload("dense_nhwc_600", si.BF16, si.NHWC, B=300, stages=((320, 3, 3), (640, 2, 2)), n=600, k_init=600, k_min=100,
+                 k_max=600, T=3, sigma=0.6, zipf_s=0.9, repeat_p=0.3, seed=63), 1),
+    (si.Workload("plain_101", si.F16, si.NCHW, B=30, stages=((256, 5, 5), (320, 2, 2)), n=101, k_init=101, k_min=70,
+                 k_max=101, T=3, sigma=0.6, zipf_s=0.9, repeat_p=0.3, seed=64), 2),
 ]
 
 
-@pytest.mark.parametrize("w", DENSE_LOOKUPS, ids=lambda w: w.name)
-def test_lookup_of_large_fast_memories(w):
+@pytest.mark.parametrize("w,route", DENSE_LOOKUPS, ids=lambda v: getattr(v, "name", str(v)))
+def test_lookup_of_large_fast_memories(w, route):
     rep = run_workload(w)
-    assert rep.frames == w.B * w.T and rep.routes == [0, w.L * w.T, 0, 0, 0]
+    assert rep.frames == w.B * w.T and rep.routes == [w.L * w.T * (r == route) for r in range(5)]
+
+
+READY_LOOKUPS = [
+    si.Workload("ready_odd", si.BF16, si.NCHW, B=40, stages=((64, 15, 15), (136, 9, 9), (256, 5, 5)), n=60, k_init=8, k_min=4,
+                k_max=16, S=40, T=5, sigma=0.5, zipf_s=0.8, repeat_p=0.5, seed=71),
+    si.Workload("ready_dense_odd", si.F16, si.NCHW, B=30, stages=((256, 9, 9), (264, 5, 5)), n=72, k_init=70, k_min=66, k_max=72,
+                T=5, sigma=0.6, zipf_s=0.8, repeat_p=0.5, seed=72),
+]
+
+
+@pytest.mark.parametrize("w", READY_LOOKUPS, ids=lambda w: w.name)
+def test_maps_ready_with_odd_widths(w):
+    # steps back to back with two alternating carries, the first layer pooled on the library's stream
+    cents, counts = si.initial_centers(w)
+    tau = [w.tau] * w.L
+    mem = oracle.OracleMemory(w.n, w.dims, tau, cents, counts, w.S, w.k_init, w.k_min, w.k_max, w.window_W)
+    cache = smtm.smtm_cache_create(w.n, w.dims, tau, cents, counts, n_streams=w.S, k_init=w.k_init, k_min=w.k_min,
+                                   k_max=w.k_max, window_W=w.window_W, max_batch=w.B, flags=smtm.FLAG_MAPS_READY)
+    sid = si.stream_ids(w) if w.S > 1 else None
+    gbs = [smtm.Batch(cache, w.B, stream_id=sid) for _ in range(2)]
+    labs = si.labels(w)
+    maps = [[si.frames(w, l, labs[t], t, device="cuda") for l in range(w.L)] for t in range(w.T)]
+    fbs = [torch.from_numpy(si.fallback_labels(w, labs[t])).cuda() for t in range(w.T)]
+    torch.cuda.synchronize()
+    for t in range(w.T):
+        for l in range(w.L):
+            (smtm.smtm_lookup_exit_begin if l == 0 else smtm.smtm_lookup_exit)(
+                cache, l, smtm.Fmap(maps[t][l], w.dtype, w.layout, *si.shape4(w, l)), gbs[t % 2])
+        smtm.smtm_cache_update_resize(cache, gbs[t % 2], fbs[t])
+    torch.cuda.synchronize()
+    for t in range(w.T):
+        ob = mem.new_batch(w.B, sid)
+        for l in range(w.L):
+            mem.lookup_exit(l, maps[t][l].cpu(), w.dtype, w.layout, si.shape4(w, l), ob)
+        mem.update(ob, si.fallback_labels(w, labs[t]))
+        mem.resize()
+    last = gbs[(w.T - 1) % 2]
+    assert np.array_equal(last.done.cpu().numpy(), ob["done"]) and np.array_equal(last.pred.cpu().numpy(), ob["pred"])
+    compare_state(w, cache, mem, Report())
+    routes = smtm.smtm_cache_get_routes(cache)
+    assert routes[smtm.ROUTE_PIPELINED_DENSE if w.k_max > 64 else smtm.ROUTE_PIPELINED] >= w.T
+    smtm.smtm_cache_destroy(cache)
