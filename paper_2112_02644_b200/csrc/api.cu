@@ -434,13 +434,23 @@ smtm_status_t update_impl(smtm_cache* c, const smtm_batch_t* b, const int32_t* d
         a.cen_split[l] = has_centre_split(c, l) ? static_cast<__nv_bfloat16*>(c->d_cen_split[l]) : nullptr;
     }
     const ResizeArgs rz = resize_args(c);
-    SMTM_CUDA(launch_update(a, with_resize ? &rz : nullptr, c->sm_count, st, &c->launches));
+    SMTM_CUDA(launch_update(a, with_resize ? &rz : nullptr, c->maps_ready, c->sm_count, st, &c->launches));
     return SMTM_OK;
 }
 
 smtm_status_t resize_impl(smtm_cache* c, cudaStream_t st) {
     SMTM_CUDA(launch_resize(resize_args(c), st, &c->launches));
     return SMTM_OK;
+}
+
+// The stamps of a profiled step.  Where the update is one launch its plan is no kernel of its own: it begins with the
+// launch and ends where the first CTA begins to fold a centre.
+cudaError_t read_stamps(const smtm_cache* c, size_t step, std::vector<unsigned long long>* stamps) {
+    const cudaError_t e = cudaMemcpy(stamps->data(), c->d_prof_clock + step * stamps->size(),
+                                     stamps->size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost);
+    unsigned long long *plan = stamps->data() + 2 * SMTM_PROF_PLAN, *centers = stamps->data() + 2 * SMTM_PROF_CENTERS;
+    if (plan[0] != 0 && plan[1] == 0 && centers[1] != 0) plan[1] = ~centers[0];
+    return e;
 }
 
 smtm_status_t check_lookup(const smtm_cache* c, int32_t layer, const smtm_fmap_t* f, const smtm_batch_t* b) {
@@ -696,7 +706,7 @@ smtm_status_t smtm_cache_warmup(smtm_cache_t* c, int32_t layer, const smtm_fmap_
         a.m[l] = c->d_m[l];
         a.cen_split[l] = has_centre_split(c, l) ? static_cast<__nv_bfloat16*>(c->d_cen_split[l]) : nullptr;
     }
-    SMTM_CUDA(launch_update(a, nullptr, c->sm_count, st, &c->launches));
+    SMTM_CUDA(launch_update(a, nullptr, c->maps_ready, c->sm_count, st, &c->launches));
     return SMTM_OK;
 }
 
@@ -886,8 +896,7 @@ smtm_status_t smtm_cache_get_profile_device(smtm_cache_t* c, double* h_total_ms,
     }
     std::vector<unsigned long long> stamps(2 * SMTM_PROF_KERNELS);
     for (size_t i = 0; c->d_prof_clock && i < c->prof_steps_used; ++i) {
-        SMTM_CUDA(cudaMemcpy(stamps.data(), c->d_prof_clock + i * stamps.size(), stamps.size() * sizeof(unsigned long long),
-                             cudaMemcpyDeviceToHost));
+        SMTM_CUDA(read_stamps(c, i, &stamps));
         for (int k = 0; k < SMTM_PROF_KERNELS; ++k) {
             const unsigned long long begin = ~stamps[2 * k], end = stamps[2 * k + 1];
             if (end == 0 || end < begin) continue;  // the kernel did not run in this step
@@ -903,8 +912,7 @@ smtm_status_t smtm_cache_get_profile_timeline(smtm_cache_t* c, int64_t step, uin
     SMTM_CUDA(cudaDeviceSynchronize());
     if (!c->d_prof_clock || step < 0 || size_t(step) >= c->prof_steps_used) return SMTM_ERR_INVALID_ARG;
     std::vector<unsigned long long> stamps(2 * SMTM_PROF_KERNELS);
-    SMTM_CUDA(cudaMemcpy(stamps.data(), c->d_prof_clock + size_t(step) * stamps.size(),
-                         stamps.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost));
+    SMTM_CUDA(read_stamps(c, size_t(step), &stamps));
     for (int k = 0; k < SMTM_PROF_KERNELS; ++k) {
         const unsigned long long begin = ~stamps[2 * k], end = stamps[2 * k + 1];  // the begin is kept as its complement
         const bool ran = end != 0 && end >= begin;

@@ -559,66 +559,6 @@ constexpr size_t fused_smem(int slice_cap, int parts) {
            (2 * kStages + 2 * kSvBufs + 2 * kRx) * 8 + 192;
 }
 
-// ---- cluster primitives ------------------------------------------------------------------------
-
-// Address of the same shared-memory location in CTA `rank` of this cluster.
-__device__ __forceinline__ uint32_t peer_smem(const void* p, uint32_t rank) {
-    uint32_t out;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(smem_u32(p)), "r"(rank));
-    return out;
-}
-
-__device__ __forceinline__ void peer_store(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-
-// Arrival on a barrier of any CTA of the cluster; orders this thread's earlier writes before it.
-__device__ __forceinline__ void peer_arrive(uint32_t bar_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n"
-        "}\n"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// As mbar_wait_bounded, for a barrier that CTAs of the whole cluster arrive on.
-__device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_t parity, int* status) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    const long long t0 = clock64();
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 256; ++i)
-            if (mbar_try_wait_cluster(bar, parity)) return true;
-        if (clock64() - t0 > (1ll << 31)) {
-            set_status(status, kDevTimeout);
-            return false;
-        }
-    }
-}
-
-// All threads of all CTAs of the cluster.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync_all() {
-    cluster_arrive();
-    cluster_wait();
-}
-__device__ __forceinline__ float peer_load(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
-
 template <class R>
 __global__ void __launch_bounds__(kThreadsFused, 1) k_lookup_nchw(const FusedParams f) {
     extern __shared__ uint8_t smem_raw[];

@@ -267,7 +267,9 @@ struct ResizeArgs {
 };
 cudaError_t launch_resize(const ResizeArgs& a, cudaStream_t st, int64_t* launches);
 // Tables and centres; with rz != nullptr also the Eq. 5 / Eq. 6 refresh of every stream that
-// had a frame in the batch.  Two launches on `st`.
-cudaError_t launch_update(const UpdateArgs& a, const ResizeArgs* rz, int sm_count, cudaStream_t st, int64_t* launches);
+// had a frame in the batch.  One launch on `st`, two for large batches.  beside_pooling: the next batch's pooling kernel runs
+// meanwhile (see launch_ordered).
+cudaError_t launch_update(const UpdateArgs& a, const ResizeArgs* rz, bool beside_pooling, int sm_count, cudaStream_t st,
+                          int64_t* launches);
 
 }  // namespace smtm

@@ -5,7 +5,8 @@
 // ascending frame index, so the result is the one a frame-by-frame replay would give and does
 // not depend on scheduling.
 //
-// An update is two launches on the caller's stream.  The plan kernel writes every frame's final
+// An update of a small batch is one launch, in which every CTA finds out for itself what it has to do (k_update_direct);
+// that of a larger one is two launches on the caller's stream.  The plan kernel writes every frame's final
 // label and stop layer and lists the (layer, class) pairs Eq. 7 has to touch: up to 4096 frames and
 // 65 536 pairs a single CTA elects the pairs in a shared-memory bitmap (k_update_plan_one); past
 // that k_update_plan does it with many CTAs (the first frame to stamp a pair with the call's
@@ -14,7 +15,8 @@
 // a grid of small CTAs (128 threads, a few KB of shared memory) with two kinds of work: the
 // first B CTAs look after the tables, one per frame (the CTA of a stream's first frame in the
 // batch applies all of the stream's frames to its tables and, when asked, refreshes its fast
-// memory by Eq. 5 / Eq. 6; the others leave at once); the remaining CTAs take the listed pairs,
+// memory by Eq. 5 / Eq. 6; the others leave at once; the tables of an only stream are shared by a
+// cluster of up to eight); the remaining CTAs take the listed pairs,
 // one each, and fold the pair's frames into the centre (Eq. 7; a pair with many frames is several items, each
 // a block of the vector's columns).  Small CTAs on purpose: there
 // are hundreds of independent pieces of work, each a short chain of dependent trips to L2, so
@@ -51,13 +53,26 @@ __device__ __forceinline__ void table_step(int& ft, int& ts, bool appears, int f
 
 constexpr int kUpdThreads = 256;   // plan kernel (many-CTA form) and the stand-alone refresh
 constexpr int kApplyThreads = 128; // CTAs of the apply kernel
-constexpr int kTabPer = 8;         // consecutive frames a thread of a tables CTA looks at per trip to memory
+constexpr int kTabPer = 8;         // consecutive frames a thread of a tables CTA looks at per trip to memory ...
+constexpr int kTabPerDirect = 4;   // ... and where it makes their codes itself, from five words each
 
 // The label a finished frame ends up with: the prediction if it exited, else the fallback label
 // (the full network's answer, -1 = none); a label outside the memory counts as no label.
 __device__ __forceinline__ int final_label_of(const UpdateArgs& a, int b) {
     const int lab = (a.done && a.done[b] != 0) ? a.pred[b] : (a.fallback ? a.fallback[b] : -1);
     return lab >= a.n ? -1 : lab;
+}
+
+// Final label and stop layer of frame b packed into one word (label | stop layer << 16), or -1 for a frame without a
+// label or of a stream outside the cache; *sid: its stream.  Every load is unconditional, so that those of several frames
+// make one trip to memory (no carry at all: a warm-up batch of labelled frames).
+__device__ __forceinline__ int frame_code_of(const UpdateArgs& a, int b, int* sid) {
+    const int dn = a.done ? a.done[b] : 0, pr = a.done ? a.pred[b] : -1, el = a.done ? a.exit_layer[b] : 0;
+    const int fb = a.fallback ? a.fallback[b] : -1;
+    *sid = a.stream_id ? a.stream_id[b] : 0;
+    const bool ex = dn != 0;
+    const int lab = ex ? pr : fb;  // a label outside the memory counts as no label
+    return (lab < 0 || lab >= a.n || *sid < 0 || *sid >= a.S) ? -1 : (lab | ((ex ? el : a.L) << 16));
 }
 
 // ---- plan -----------------------------------------------------------------------------------
@@ -93,25 +108,17 @@ __global__ void __launch_bounds__(kUpdThreads) k_update_plan(const UpdateArgs a)
     const int b = blockIdx.x * kUpdThreads + threadIdx.x;
     const unsigned long long epoch = *a.plan.epoch + 1;  // this call's number; every CTA reads it before any is through
     if (b < a.B) {
-        // every load unconditional, so that they make one trip to memory (no carry at all: a warm-up batch
-        // of labelled frames)
-        const int dn = a.done ? a.done[b] : 0, pr = a.done ? a.pred[b] : -1, el = a.done ? a.exit_layer[b] : 0;
-        const int fb = a.fallback ? a.fallback[b] : -1;
-        const int sid = a.stream_id ? a.stream_id[b] : 0;
-        const bool ex = dn != 0;
-        int lab = ex ? pr : fb;
-        if (lab >= a.n) lab = -1;  // a label outside the memory counts as no label
-        if (sid < 0 || sid >= a.S) {  // a stream outside the cache: the frame takes no part in the update
-            lab = -1;
-            set_status(a.status, kDevInvalidArg);
-        }
-        a.plan.frame_code[b] = lab < 0 ? -1 : (lab | ((ex ? el : a.L) << 16));
-        if (lab >= 0) {
+        int sid;
+        const int code = frame_code_of(a, b, &sid);
+        if (sid < 0 || sid >= a.S) set_status(a.status, kDevInvalidArg);  // the frame takes no part in the update
+        a.plan.frame_code[b] = code;
+        if (code >= 0) {
+            const int lab = code & 0xffff;
             // Eq. 7 touches the layers up to the stop layer: the first frame to stamp (layer, class)
             // with the call's number lists the pair as a job, and as a single item (this form of the plan
             // does not count the frames of a pair)
             const int l_lo = a.warm_layer >= 0 ? a.warm_layer : 0;
-            const int l_hi = a.warm_layer >= 0 ? a.warm_layer + 1 : (ex ? el : a.L);
+            const int l_hi = a.warm_layer >= 0 ? a.warm_layer + 1 : code >> 16;
             for (int l = l_lo; l < l_hi; ++l)
                 if (atomicExch(a.plan.class_tag + (size_t)l * a.n + lab, epoch) != epoch) {
                     const int at = atomicAdd(a.plan.job_count + (epoch & 1), 1);
@@ -158,20 +165,14 @@ __global__ void __launch_bounds__(kPlanOneThreads) k_update_plan_one(const Updat
     const ClockScope stamps(a.clock ? a.clock + 2 * SMTM_PROF_PLAN : nullptr);
     __syncthreads();
     for (int b = tid; b < a.B; b += kPlanOneThreads) {
-        const int dn = a.done ? a.done[b] : 0, pr = a.done ? a.pred[b] : -1, el = a.done ? a.exit_layer[b] : 0;
-        const int fb = a.fallback ? a.fallback[b] : -1;
-        const int sid = a.stream_id ? a.stream_id[b] : 0;
-        const bool ex = dn != 0;
-        int lab = ex ? pr : fb;
-        if (lab >= a.n) lab = -1;
-        if (sid < 0 || sid >= a.S) {  // a stream outside the cache: the frame takes no part in the update
-            lab = -1;
-            set_status(a.status, kDevInvalidArg);
-        }
-        a.plan.frame_code[b] = lab < 0 ? -1 : (lab | ((ex ? el : a.L) << 16));
-        if (lab >= 0) {
+        int sid;
+        const int code = frame_code_of(a, b, &sid);
+        if (sid < 0 || sid >= a.S) set_status(a.status, kDevInvalidArg);  // the frame takes no part in the update
+        a.plan.frame_code[b] = code;
+        if (code >= 0) {
+            const int lab = code & 0xffff;
             const int l_lo = a.warm_layer >= 0 ? a.warm_layer : 0;
-            const int l_hi = a.warm_layer >= 0 ? a.warm_layer + 1 : (ex ? el : a.L);
+            const int l_hi = a.warm_layer >= 0 ? a.warm_layer + 1 : code >> 16;
             for (int l = l_lo; l < l_hi; ++l) {
                 const int pair = l * a.n + lab;
                 if (counted) {
@@ -280,6 +281,19 @@ __device__ __forceinline__ void adaptive_size(const ResizeArgs& a, int s, const 
         chosen = __reduce_min_sync(kFull, chosen);
     }
     if (lane == 0) a.k[s] = chosen;
+}
+
+// How many of the nz keys of s_key (16-byte aligned; two to a load, the same ones for every thread) lie above `key`: its rank.
+__device__ __forceinline__ int keys_above(const unsigned long long* s_key, int nz, unsigned long long key) {
+    int r0 = 0, r1 = 0, j = 0;
+#pragma unroll 4
+    for (; j + 1 < nz; j += 2) {
+        const ulonglong2 k2 = *reinterpret_cast<const ulonglong2*>(s_key + j);
+        r0 += k2.x > key ? 1 : 0;
+        r1 += k2.y > key ? 1 : 0;
+    }
+    if (j < nz) r0 += s_key[j] > key ? 1 : 0;
+    return r0 + r1;
 }
 
 // Descending bitonic sort of nz keys in s_key by the whole CTA (padded to a power of two with zeros: no key is zero).
@@ -419,8 +433,8 @@ __device__ void refresh_sorted_in_registers(const ResizeArgs& a, int s, const un
 // Eq. 5 / Eq. 6 for stream s when every thread of the CTA holds the scores of its PER consecutive classes
 // (c_lo ...) in registers.  The keys of the non-zero scores are appended to a list in shared memory in whatever
 // order the threads come (a key carries its class, and ranking by key does not care about the list's order);
-// the rest is one warp's work: ranks by counting (a sort by the whole CTA when the keys are many), zero-score
-// classes in ascending id for the slots that remain (they are among the first k_max ids), Eq. 6.
+// the CTA ranks them by counting, a key per thread (by a sort when they are many); the rest is one warp's work:
+// zero-score classes in ascending id for the slots that remain (they are among the first k_max ids), Eq. 6.
 // `dyn`: keys [pow2 >= n] | best scores [k_max] | zero flags [k_max] bytes.  *s_nz and *s_total are zero on entry.
 template <int PER>
 __device__ void refresh_from_registers(const ResizeArgs& a, int s, const unsigned long long (&sc)[PER], int c_lo,
@@ -449,32 +463,25 @@ __device__ void refresh_from_registers(const ResizeArgs& a, int s, const unsigne
     const int nz = *s_nz;
     const unsigned long long total = *s_total;
     if (total == 0) return;  // nothing seen yet: keep size and members (the same for every thread)
-    const bool sorted = nz > kCountRankMax;
-    if (sorted) sort_keys(s_key, nz);
-    if (tid >= kWarp) return;
     int32_t* mem = a.members + (size_t)s * a.k_max;
-    if (sorted) {
-        for (int r = lane; r < nz && r < a.k_max; r += kWarp) {
+    if (nz > kCountRankMax) {
+        sort_keys(s_key, nz);
+        for (int r = tid; r < nz && r < a.k_max; r += blockDim.x) {
             mem[r] = key_class(s_key[r]);
             s_top[r] = key_score(s_key[r]);
         }
     } else {
-        for (int i = lane; i < nz; i += kWarp) {  // rank = keys larger than this one (keys are distinct)
+        for (int i = tid; i < nz; i += blockDim.x) {
             const unsigned long long key = s_key[i];
-            int r0 = 0, r1 = 0;
-            int j = 0;
-            for (; j + 1 < nz; j += 2) {
-                r0 += s_key[j] > key ? 1 : 0;
-                r1 += s_key[j + 1] > key ? 1 : 0;
-            }
-            if (j < nz) r0 += s_key[j] > key ? 1 : 0;
-            const int r = r0 + r1;
+            const int r = keys_above(s_key, nz, key);
             if (r < a.k_max) {
                 mem[r] = key_class(key);
                 s_top[r] = key_score(key);
             }
         }
     }
+    __syncthreads();
+    if (tid >= kWarp) return;
     const unsigned lt = (1u << lane) - 1u;
     int filled = nz;
     for (int c0 = 0; c0 < a.k_max && filled < a.k_max; c0 += kWarp) {
@@ -547,14 +554,7 @@ __device__ void refresh_stream(const ResizeArgs& a, int s, unsigned char* dyn, i
         // rank = keys larger than this one (keys are distinct); rank r < k_max goes to slot r
         for (int i = tid; i < nz; i += nt) {
             const unsigned long long key = s_key[i];
-            int r0 = 0, r1 = 0;
-            int j = 0;
-            for (; j + 1 < nz; j += 2) {
-                r0 += s_key[j] > key ? 1 : 0;
-                r1 += s_key[j + 1] > key ? 1 : 0;
-            }
-            if (j < nz) r0 += s_key[j] > key ? 1 : 0;
-            const int r = r0 + r1;
+            const int r = keys_above(s_key, nz, key);
             if (r < a.k_max) {
                 mem[r] = key_class(key);
                 s_top[r] = key_score(key);
@@ -585,7 +585,7 @@ __device__ void refresh_stream(const ResizeArgs& a, int s, unsigned char* dyn, i
 }
 
 __global__ void __launch_bounds__(kResizeThreadsMax) k_resize(const ResizeArgs a) {
-    extern __shared__ unsigned long long s_dyn[];
+    extern __shared__ __align__(16) unsigned long long s_dyn[];
     __shared__ int s_scan[33];
     __shared__ unsigned long long s_part[32];
     chain_wait();
@@ -617,13 +617,144 @@ __host__ __device__ constexpr size_t tables_smem(int n, int k_max, bool with_ref
     return closed > refresh ? closed : refresh;
 }
 
+// A cache with one stream: its tables by a team of CTAs, a class per thread (the first CTAs of the grid, a cluster).
+constexpr int kTeamMost = 8;
+__host__ __device__ constexpr int lone_team(int n) {
+    int t = 1;
+    while (t * kApplyThreads < n) t *= 2;
+    return t;  // (beyond kTeamMost the single CTA of tables_of_frame)
+}
+// Shared memory of a CTA of the team: all classes' keys, the k_max best scores, a sum per warp of the team, the
+// appearances and last positions of the CTA's classes.
+__host__ __device__ constexpr size_t lone_smem(int n, int k_max) {
+    return size_t(lone_team(n)) * kApplyThreads * 8 + size_t(k_max) * 8 + size_t(kTeamMost) * (kApplyThreads / kWarp) * 8 +
+           2 * size_t(kApplyThreads) * sizeof(int);
+}
+
+// Sec. 6.1 and, if asked, Eq. 5 / Eq. 6 for the only stream of a cache, by a cluster of lone_team(n) CTAs.  Every CTA looks
+// at all frames and keeps those of its own classes, a class per thread; the ranking keys (one more than refresh_key, so
+// that classes with a zero score come behind the others in ascending id) are written to every CTA of the team, and a thread
+// counts the keys above its own.  One CTA with eight classes a thread sorted them: an update of 1024 frames of 1000 classes
+// 14 us, and ranked up to 256 non-zero scores with one warp.
+template <bool kPlanned>
+__device__ void tables_of_lone_stream(const UpdateArgs& a, const ResizeArgs& rz, int do_resize, int team, unsigned char* dyn,
+                                      int* s_list, int* s_scan) {
+    constexpr int kPer = kPlanned ? kTabPer : kTabPerDirect;
+    constexpr int nt = kApplyThreads;
+    unsigned long long* s_key = reinterpret_cast<unsigned long long*>(dyn);  // [team * nt]
+    unsigned long long* s_top = s_key + team * nt;                            // [k_max] (the first CTA's)
+    unsigned long long* s_sum = s_top + rz.k_max;                             // [team * warps]
+    int* s_cnt = reinterpret_cast<int*>(s_sum + kTeamMost * (nt / kWarp));    // [nt]
+    int* s_last = s_cnt + nt;                                                 // [nt]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = int(blockIdx.x), c_lo = rank * nt, c = c_lo + tid;
+    if (do_resize && team > 1) cluster_arrive();  // (waited for before the first store to a peer: it has to have started)
+    int f = c < a.n ? a.ft[c] : 0, t = c < a.n ? a.ts[c] : 0;  // in flight with the frames below
+    s_cnt[tid] = 0;
+    s_last[tid] = -1;
+    int m = 0;
+    if (a.forget_W == 0) {
+        // the closed form of tables_of_frame: q appearances, the last at position p
+        for (int p0 = 0; p0 < a.B; p0 += kPer * nt) {
+            const int b0 = p0 + tid * kPer;
+            int sidv[kPer], code[kPer];
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const int b = min(b0 + i, a.B - 1);
+                if (kPlanned) {
+                    sidv[i] = a.stream_id ? a.stream_id[b] : 0;
+                    code[i] = a.plan.frame_code[b];
+                } else {
+                    code[i] = frame_code_of(a, b, &sidv[i]);
+                }
+            }
+            int hits = 0;
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                sidv[i] = (b0 + i < a.B && sidv[i] == 0) ? 1 : 0;  // (another id: no stream of this cache)
+                hits += sidv[i];
+            }
+            int cnt, pos;
+            if (a.stream_id) {
+                pos = m + block_exclusive_scan(hits, s_scan, &cnt);
+            } else {
+                pos = b0;
+                cnt = min(a.B - p0, kPer * nt);
+                if (p0 == 0) __syncthreads();  // the counters are zero
+            }
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+                if (sidv[i]) {
+                    const int at = (code[i] & 0xffff) - c_lo;
+                    if (code[i] >= 0 && at >= 0 && at < nt) {
+                        atomicAdd(&s_cnt[at], 1);
+                        atomicMax(&s_last[at], pos);
+                    }
+                    ++pos;
+                }
+            m += cnt;
+        }
+        __syncthreads();
+        const int q = s_cnt[tid];
+        if (q > 0) {
+            f = int(min((long long)f + q, (long long)kFtMax));
+            t = m - 1 - s_last[tid];
+        } else {
+            t = int(min((long long)t + m, (long long)INT32_MAX));
+        }
+    } else {
+        // the forgetting table has no closed form: the frames, a tile at a time, replayed per class
+        for (int t0 = 0; t0 < a.B; t0 += nt) {
+            const int b = t0 + tid;
+            const int hit = (b < a.B && (a.stream_id ? a.stream_id[b] : 0) == 0) ? 1 : 0;
+            const int cnt = compact_tile(hit, hit ? final_label_of(a, b) : -1, s_list, s_scan);
+            for (int j = 0; j < cnt; ++j) table_step(f, t, s_list[j] == c, a.forget_W);
+        }
+    }
+    unsigned long long sc = 0ull;
+    if (c < a.n) {
+        a.ft[c] = f;
+        a.ts[c] = t;
+        sc = score_of(f, t, rz.W, rz.forgetting);
+    }
+    if (!do_resize) return;
+    const unsigned long long key = c < a.n ? refresh_key(sc, c) + 1ull : 0ull;
+    unsigned long long sum = sc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+    if (team > 1) {
+        cluster_wait();
+        for (int r = 0; r < team; ++r) {
+            peer_store(peer_smem(s_key + c, r), key);
+            if (lane == 0) peer_store(peer_smem(s_sum + rank * (nt / kWarp) + warp, r), sum);
+        }
+        cluster_sync_all();
+    } else {
+        s_key[c] = key;
+        if (lane == 0) s_sum[warp] = sum;
+        __syncthreads();
+    }
+    unsigned long long total = 0ull;
+    for (int w = 0; w < team * (nt / kWarp); ++w) total += s_sum[w];
+    if (total == 0) return;  // nothing seen yet: keep size and members (the same for every thread of the team)
+    const int r = keys_above(s_key, a.n, key);
+    if (c < a.n && r < rz.k_max) {
+        rz.members[r] = c;
+        if (team > 1) peer_store(peer_smem(s_top + r, 0), sc);
+        else s_top[r] = sc;
+    }
+    if (team > 1) cluster_sync_all(); else __syncthreads();
+    if (rank == 0 && warp == 0) adaptive_size(rz, 0, s_top, total, lane);
+}
+
 // Sec. 6.1 for the stream of frame g by one CTA, if g is the stream's first frame in the batch (else the
 // CTA of that frame does it; g < 0: the only stream of a cache that has one, whichever frame of it comes
 // first): all of the stream's frames, in ascending index, applied to its tables; then,
 // if asked, the stream's Eq. 5 / Eq. 6 refresh.  Every thread looks after a run of PER consecutive classes
 // and keeps their entries in registers from the one trip to memory that fetches them to the refresh
 // (PER == 0: any number of classes, the entries stay in global memory).
-template <int PER>
+// kPlanned: the frames' codes are the plan kernel's; else they are made here from the batch.
+template <int PER, bool kPlanned>
 __device__ void tables_of_frame(const UpdateArgs& a, const ResizeArgs& rz, int g, int do_resize, unsigned char* dyn,
                                 int* s_list, int* s_scan, unsigned long long* s_part) {
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -690,28 +821,34 @@ __device__ void tables_of_frame(const UpdateArgs& a, const ResizeArgs& rz, int g
             s_last[c] = -1;
         }
         __syncthreads();
-        // Every thread looks at a run of eight consecutive frames (their stream ids and the plan's codes in one
+        // Every thread looks at a run of consecutive frames (their stream ids and codes in one
         // trip to memory); a scan over the threads gives each of the stream's frames its position in the stream.
+        constexpr int kPer = kPlanned ? kTabPer : kTabPerDirect;
         int m = 0;
-        for (int p0 = g; p0 < a.B; p0 += kTabPer * nt) {
-            const int b0 = p0 + tid * kTabPer;
-            int sidv[kTabPer], code[kTabPer];
+        for (int p0 = g; p0 < a.B; p0 += kPer * nt) {
+            const int b0 = p0 + tid * kPer;
+            int sidv[kPer], code[kPer];
 #pragma unroll
-            for (int i = 0; i < kTabPer; ++i) {
+            for (int i = 0; i < kPer; ++i) {
                 const int b = min(b0 + i, a.B - 1);
-                sidv[i] = a.stream_id ? a.stream_id[b] : s;
-                code[i] = a.plan.frame_code[b];
+                if (kPlanned) {
+                    sidv[i] = a.stream_id ? a.stream_id[b] : s;
+                    code[i] = a.plan.frame_code[b];
+                } else {
+                    code[i] = frame_code_of(a, b, &sidv[i]);
+                    if (!a.stream_id) sidv[i] = s;
+                }
             }
             int hits = 0;
 #pragma unroll
-            for (int i = 0; i < kTabPer; ++i) {
+            for (int i = 0; i < kPer; ++i) {
                 sidv[i] = (b0 + i < a.B && sidv[i] == s) ? 1 : 0;
                 hits += sidv[i];
             }
             int cnt;
             int pos = m + block_exclusive_scan(hits, s_scan, &cnt);
 #pragma unroll
-            for (int i = 0; i < kTabPer; ++i)
+            for (int i = 0; i < kPer; ++i)
                 if (sidv[i]) {
                     if (code[i] >= 0) {  // (a frame without a label only ages the classes)
                         atomicAdd(&s_cnt[code[i] & 0xffff], 1);
@@ -775,7 +912,16 @@ __device__ void tables_of_frame(const UpdateArgs& a, const ResizeArgs& rz, int g
     }
     if (do_resize) {
         __syncthreads();  // every thread is done with the closed form's arrays (and sees its own table entries)
-        if (PER == 8)
+        // Up to 1024 classes: a sort in registers, unless the stream has seen few of them.
+        bool many = false;
+        if (PER == 8) {
+            int mine = 0, nz;
+#pragma unroll
+            for (int i = 0; i < PER; ++i) mine += sc[i] != 0 ? 1 : 0;
+            block_exclusive_scan(mine, s_scan, &nz);
+            many = nz > kCountRankMax;
+        }
+        if (many)
             refresh_sorted_in_registers<(PER ? PER : 1)>(rz, s, sc, c_lo, dyn, s_part);
         else if (PER)
             refresh_from_registers<(PER ? PER : 1)>(rz, s, sc, c_lo, dyn, &s_scan[32], &s_part[31]);
@@ -857,10 +1003,11 @@ __device__ __forceinline__ float fold_centre(const UpdateArgs& a, int l0, int cl
 // single item then renews the centre's length and count itself.  The items of a cut pair leave the squared
 // length of their blocks in norm_part and take a ticket; the last one through adds the blocks in order and
 // renews length and count (every item has read the count by then), and puts the ticket back to zero.
-__device__ void centre_item(const UpdateArgs& a, int item, const int (&first_tile)[kCenPer], int* s_list, int* s_scan,
-                            float4* s_acc) {
+// list(base) puts the pair's frames among base .. base + kCenTile - 1 into s_list and returns their number.
+template <class List>
+__device__ __forceinline__ void centre_item(const UpdateArgs& a, int l0, int cls, int blk, int nblk, const List& list,
+                                            const int* s_list, float4* s_acc) {
     const int tid = threadIdx.x, nt = blockDim.x;
-    const int cls = item & 0x1fff, l0 = (item >> 16) & 15, blk = (item >> 20) & 15, nblk = 1 << ((item >> 24) & 7);
     const int D = a.dims[l0];
     const float* sv = a.sv[l0];
     float* cen = a.centers[l0] + (size_t)cls * D;
@@ -880,7 +1027,7 @@ __device__ void centre_item(const UpdateArgs& a, int item, const int (&first_til
             // An item a few times as wide as the CTA whose frames fit one listing (the usual pair: a row or two of
             // a long vector): the frames are listed once, and a thread has its column groups of two sweeps in
             // flight together, a row at a time.  Same order of additions as below.
-            const int cnt = list_pair_frames(a, 0, cls, l0, s_list, s_scan, first_tile);
+            const int cnt = list(0);
             q = cnt;
             const double dm = double(m), inv = 1.0 / (dm + double(q));
             for (int w0 = 0; w0 < sweeps && q > 0; w0 += 2) {
@@ -890,7 +1037,7 @@ __device__ void centre_item(const UpdateArgs& a, int item, const int (&first_til
 #pragma unroll 1
                 for (int i = 0; i < cnt; ++i) {
                     const float4* rp = reinterpret_cast<const float4*>(sv + (size_t)s_list[i] * D);
-                    const float4 ra = __ldg(rp + la), rb = __ldg(rp + lb);
+                    const float4 ra = rp[la], rb = rp[lb];
                     acc_a[0] += ra.x; acc_a[1] += ra.y; acc_a[2] += ra.z; acc_a[3] += ra.w;
                     acc_b[0] += rb.x; acc_b[1] += rb.y; acc_b[2] += rb.z; acc_b[3] += rb.w;
                 }
@@ -908,7 +1055,7 @@ __device__ void centre_item(const UpdateArgs& a, int item, const int (&first_til
             float acc[4] = {0.f, 0.f, 0.f, 0.f};
             q = 0;
             for (int base = 0; base < a.B; base += kCenTile) {
-                const int cnt = list_pair_frames(a, base, cls, l0, s_list, s_scan, first_tile);
+                const int cnt = list(base);
                 if (cnt == 0) continue;  // (the same for every thread)
                 q += cnt;
                 if (!mine_col) continue;
@@ -916,7 +1063,7 @@ __device__ void centre_item(const UpdateArgs& a, int item, const int (&first_til
                     float4 r[8];
 #pragma unroll
                     for (int u = 0; u < 8; ++u)  // unconditional loads (past the end: the last row again, unused)
-                        r[u] = __ldg(reinterpret_cast<const float4*>(sv + (size_t)s_list[min(i0 + u * R, cnt - 1)] * D) + c4);
+                        r[u] = reinterpret_cast<const float4*>(sv + (size_t)s_list[min(i0 + u * R, cnt - 1)] * D)[c4];
 #pragma unroll
                     for (int u = 0; u < 8; ++u)
                         if (i0 + u * R < cnt) {
@@ -943,7 +1090,7 @@ __device__ void centre_item(const UpdateArgs& a, int item, const int (&first_til
             float acc = 0.f;
             q = 0;
             for (int base = 0; base < a.B; base += kCenTile) {
-                const int cnt = list_pair_frames(a, base, cls, l0, s_list, s_scan, first_tile);
+                const int cnt = list(base);
                 if (cnt == 0) continue;
                 q += cnt;
                 if (d < D)
@@ -974,11 +1121,27 @@ __device__ void centre_item(const UpdateArgs& a, int item, const int (&first_til
     a.m[l0][cls] = m + uint32_t(q);
 }
 
+// Tables of the stream of frame `g` (see tables_of_frame), by the variant the number of classes asks for.
+template <bool kPlanned>
+__device__ __forceinline__ void tables_cta(const UpdateArgs& a, const ResizeArgs& rz, int do_resize, unsigned char* dyn,
+                                           int* s_list, int* s_scan, unsigned long long* s_part) {
+    const ClockScope stamps(a.clock ? a.clock + 2 * SMTM_PROF_TABLES : nullptr);
+    const int g = a.S == 1 ? -1 : int(blockIdx.x), team = lone_team(a.n);
+    if (g < 0 && team <= kTeamMost)
+        tables_of_lone_stream<kPlanned>(a, rz, do_resize, team, dyn, s_list, s_scan);
+    else if (a.n <= 4 * kApplyThreads)
+        tables_of_frame<4, kPlanned>(a, rz, g, do_resize, dyn, s_list, s_scan, s_part);
+    else if (a.n <= 8 * kApplyThreads)
+        tables_of_frame<8, kPlanned>(a, rz, g, do_resize, dyn, s_list, s_scan, s_part);
+    else
+        tables_of_frame<0, kPlanned>(a, rz, g, do_resize, dyn, s_list, s_scan, s_part);
+}
+
 // The apply kernel: CTAs [0, table_ctas) are tables CTAs, one per frame (a single one for a cache with one stream);
 // the others take the listed items.
 __global__ void __launch_bounds__(kApplyThreads, 8) k_update_apply(const UpdateArgs a, const ResizeArgs rz, int do_resize,
                                                                     int table_ctas) {
-    extern __shared__ unsigned long long s_dyn[];
+    extern __shared__ __align__(16) unsigned long long s_dyn[];
     __shared__ int s_list[kCenTile];
     __shared__ int s_scan[33];
     __shared__ unsigned long long s_part[32];
@@ -986,21 +1149,14 @@ __global__ void __launch_bounds__(kApplyThreads, 8) k_update_apply(const UpdateA
     chain_wait();
     chain_release();
     if (int(blockIdx.x) < table_ctas) {
-        const ClockScope stamps(a.clock ? a.clock + 2 * SMTM_PROF_TABLES : nullptr);
-        unsigned char* dyn = reinterpret_cast<unsigned char*>(s_dyn);
-        if (a.n <= 4 * kApplyThreads)
-            tables_of_frame<4>(a, rz, a.S == 1 ? -1 : int(blockIdx.x), do_resize, dyn, s_list, s_scan, s_part);
-        else if (a.n <= 8 * kApplyThreads)
-            tables_of_frame<8>(a, rz, a.S == 1 ? -1 : int(blockIdx.x), do_resize, dyn, s_list, s_scan, s_part);
-        else
-            tables_of_frame<0>(a, rz, a.S == 1 ? -1 : int(blockIdx.x), do_resize, dyn, s_list, s_scan, s_part);
+        tables_cta<true>(a, rz, do_resize, reinterpret_cast<unsigned char*>(s_dyn), s_list, s_scan, s_part);
         return;
     }
     const int first = int(blockIdx.x) - table_ctas, stride = int(gridDim.x) - table_ctas;
     int first_tile[kCenPer];  // the codes of the first frames, the item and the count: one trip to memory
 #pragma unroll
     for (int i = 0; i < kCenPer; ++i) first_tile[i] = a.plan.frame_code[min(int(threadIdx.x) * kCenPer + i, a.B - 1)];
-    int item = a.plan.items[first];  // (the list has room for every CTA)
+    int item = a.plan.items[min(first, kItemBlocksMax * a.L * a.n - 1)];
     const int n_items = a.plan.job_count[3];
     if (first >= n_items) return;
     const ClockScope stamps(a.clock ? a.clock + 2 * SMTM_PROF_CENTERS : nullptr);
@@ -1009,8 +1165,79 @@ __global__ void __launch_bounds__(kApplyThreads, 8) k_update_apply(const UpdateA
             __syncthreads();  // the previous item's readers are done with the list
             item = a.plan.items[it];
         }
-        centre_item(a, item, first_tile, s_list, s_scan, s_acc);
+        const int cls = item & 0x1fff, l0 = (item >> 16) & 15;
+        centre_item(a, l0, cls, (item >> 20) & 15, 1 << ((item >> 24) & 7),
+                    [&](int base) { return list_pair_frames(a, base, cls, l0, s_list, s_scan, first_tile); }, s_list, s_acc);
     }
+}
+
+// ---- small updates in one launch -----------------------------------------------------------------
+//
+// The plan is a trip to memory, a kernel of one CTA and a launch before anything is folded.  For small batches every CTA
+// makes what it needs of it by itself: CTA (layer, frame) fetches the state of all frames (PER consecutive ones a thread),
+// leaves when its own frame has no label or stopped before the layer, and else counts and lists the frames of its frame's
+// pair in ascending index.  The pair's column blocks are dealt to the CTAs of its first frames, in order; the others leave.
+// No CTA waits for another, and the sums are those of the two launches.  What bounds it: trips to memory (three here, five
+// and a launch there), and with many frames the state that every CTA fetches, so the two launches stay beyond the lines
+// below.  Update with refresh, 200 classes, by two launches and by one: 16 frames in one layer of 256 channels 6.9 and 5.1
+// us, 128 frames in 13 layers 9.3 and 6.7, 256 in two of 1024 channels 8.7 and 7.2, 512 in two 9.1 and 7.7; 512 streams in
+// two layers 10.0 and 10.1, 700 frames in one layer 9.1 and 9.2, 256 in 13 layers 10.1 and 11.3.  (Six CTAs to an SM: with
+// eight the 64 registers spill, and 256 frames in two layers take 8.4.)
+constexpr int kDirectFrames = 512;
+constexpr int kDirectCtas = 9, kDirectCtasSmall = 16;  // CTAs per SM at most; the second with a frame per thread
+
+template <int PER>
+__global__ void __launch_bounds__(kApplyThreads, 6) k_update_direct(const UpdateArgs a, const ResizeArgs rz, int do_resize,
+                                                                     int table_ctas) {
+    static_assert(PER * kApplyThreads <= kCenTile, "a pair's frames fit one listing");
+    extern __shared__ __align__(16) unsigned long long s_dyn[];
+    __shared__ int s_list[kCenTile];
+    __shared__ int s_scan[33];
+    __shared__ unsigned long long s_part[32];
+    __shared__ float4 s_acc[kApplyThreads];
+    chain_wait();
+    chain_release();
+    if (int(blockIdx.x) < table_ctas) {
+        tables_cta<false>(a, rz, do_resize, reinterpret_cast<unsigned char*>(s_dyn), s_list, s_scan, s_part);
+        return;
+    }
+    const int tid = threadIdx.x;
+    const int at = int(blockIdx.x) - table_ctas, row = at / a.B, b = at - row * a.B;
+    const int l0 = a.warm_layer >= 0 ? a.warm_layer : row;
+    if (row >= (a.warm_layer >= 0 ? 1 : a.L)) return;  // (the grid is whole clusters)
+    if (a.clock && tid == 0) atomicMax(a.clock + 2 * SMTM_PROF_PLAN, ~device_clock_ns());  // (ends where the centres begin)
+    int sid_b, sid, code[PER];
+    const int own = frame_code_of(a, b, &sid_b);
+    const auto leaves = [&] { return own < 0 || (a.warm_layer < 0 && (own >> 16) <= l0); };  // (the same for every thread)
+    if (row == 0 && tid == 0 && (sid_b < 0 || sid_b >= a.S)) set_status(a.status, kDevInvalidArg);
+    if (PER > 1 && leaves()) return;  // (a crowd: what the others fetch should not queue behind the loads of those that leave)
+#pragma unroll
+    for (int i = 0; i < PER; ++i) code[i] = frame_code_of(a, min(tid * PER + i, a.B - 1), &sid);  // PER == 1: in flight with `own`
+    if (PER == 1 && leaves()) return;
+    const int cls = own & 0xffff;
+    int mine = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const bool hit = tid * PER + i < a.B && code[i] >= 0 && (code[i] & 0xffff) == cls &&
+                         (a.warm_layer >= 0 || (code[i] >> 16) > l0);
+        code[i] = hit ? 1 : 0;
+        mine += code[i];
+    }
+    int cnt;
+    int pos = block_exclusive_scan(mine, s_scan, &cnt);
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (code[i]) {
+            if (tid * PER + i == b) s_scan[32] = pos;  // this frame's place in the list
+            s_list[pos++] = tid * PER + i;
+        }
+    __syncthreads();
+    const int place = s_scan[32];
+    int nblk = item_blocks(cnt, a.dims[l0]);
+    while (nblk > cnt) nblk >>= 1;  // (a block needs a frame whose CTA folds it)
+    if (place >= nblk) return;
+    const ClockScope stamps(a.clock ? a.clock + 2 * SMTM_PROF_CENTERS : nullptr);
+    centre_item(a, l0, cls, place, nblk, [&](int) { return cnt; }, s_list, s_acc);
 }
 
 __global__ void k_center_norms(const float* centers, int n, int D, float* cnorm) {
@@ -1033,6 +1260,11 @@ cudaError_t memory_setup() {
     cudaError_t e = allow_max_dynamic_smem(k_update_apply);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_resize);
     // the update's kernels share SMs with the next step's pooling kernel on the pipelined route
+#define SMTM_OPT_IN(PER)                                                             \
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_update_direct<PER>);          \
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_update_direct<PER>);
+    SMTM_OPT_IN(1) SMTM_OPT_IN(4)
+#undef SMTM_OPT_IN
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_update_apply);
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_update_plan_one);
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_update_plan);
@@ -1047,10 +1279,34 @@ cudaError_t launch_center_norms(const float* centers, int n, int D, float* cnorm
     return launch_chained(k_center_norms, n, 256, 0, st, centers, n, D, cnorm);
 }
 
-cudaError_t launch_update(const UpdateArgs& a, const ResizeArgs* rz, int sm_count, cudaStream_t st, int64_t* launches) {
+cudaError_t launch_update(const UpdateArgs& a, const ResizeArgs* rz, bool beside_pooling, int sm_count, cudaStream_t st,
+                          int64_t* launches) {
     if (a.B <= 0) return cudaSuccess;
     cudaError_t e = cudaSuccess;
+    const bool tables = a.warm_layer < 0;  // a warm-up batch has no streams
+    const bool lone = tables && a.S == 1 && lone_team(a.n) <= kTeamMost;
+    const int team = lone ? lone_team(a.n) : 1;  // CTAs that share the tables of an only stream: a cluster
+    const int table_ctas = !tables ? 0 : a.S == 1 ? team : a.B;  // a CTA per frame finds out whether its frame is its stream's first
+    // A memory of many classes is refreshed by a kernel of its own with CTAs of 1024 threads (sorting a thousand
+    // keys is 55 rounds of compare-exchange: a round per barrier with 1024 threads, eight times that with the 128
+    // threads of a tables CTA); it refreshes every stream, which gives the streams without a frame in the batch
+    // the fast memory they already have.
+    const bool refresh_apart = tables && rz && a.n > 8 * kApplyThreads;
+    const bool refresh_here = tables && rz && !refresh_apart;
+    const size_t smem = lone ? lone_smem(a.n, rz ? rz->k_max : 0) : tables ? tables_smem(a.n, rz ? rz->k_max : 0, refresh_here) : 0;
+    const ResizeArgs rza = rz ? *rz : ResizeArgs{};
+    const int layers = a.warm_layer >= 0 ? 1 : a.L;
+    const bool direct = a.B <= kDirectFrames && (long long)table_ctas + (long long)a.B * layers <=
+                        (long long)(a.B <= kApplyThreads ? kDirectCtasSmall : kDirectCtas) * sm_count;
     ++*launches;
+    if (direct) {
+        const auto kernel = a.B <= kApplyThreads ? k_update_direct<1> : k_update_direct<4>;
+        const int ctas = (table_ctas + a.B * layers + team - 1) / team * team;
+        e = beside_pooling ? launch_ordered_cluster(kernel, ctas, kApplyThreads, smem, team, st, a, rza, refresh_here ? 1 : 0, table_ctas)
+                           : launch_chained_cluster(kernel, ctas, kApplyThreads, smem, team, st, a, rza, refresh_here ? 1 : 0, table_ctas);
+        if (e != cudaSuccess || !refresh_apart) return e;
+        return launch_resize(*rz, st, launches);
+    }
     const long long pairs = (long long)a.L * a.n;
     if (a.B <= kPlanOneMaxB && pairs <= 32LL * kPlanOneWords) {
         const size_t words = pairs <= kPlanCountMax ? size_t(pairs) : size_t((pairs + 31) / 32);
@@ -1059,22 +1315,13 @@ cudaError_t launch_update(const UpdateArgs& a, const ResizeArgs* rz, int sm_coun
         e = launch_chained(k_update_plan, (a.B + kUpdThreads - 1) / kUpdThreads, kUpdThreads, 0, st, a);
     }
     if (e != cudaSuccess) return e;
-    const bool tables = a.warm_layer < 0;  // a warm-up batch has no streams
-    const int table_ctas = tables ? (a.S == 1 ? 1 : a.B) : 0;  // a CTA per frame finds out whether its frame is its stream's first
     // Eq. 7: at most min(B, n) classes appear per layer; a CTA per item, and a heavy pair is several items (never
     // more than twice the rows' worth); beyond a few waves of CTAs they stride
-    const int pairs_max = std::min(a.B, a.n) * (a.warm_layer >= 0 ? 1 : a.L);
+    const int pairs_max = std::min(a.B, a.n) * layers;
     const int centre_ctas = std::min(pairs_max + pairs_max / 2 + kItemBlocksMax, 16 * sm_count);
-    // A memory of many classes is refreshed by a kernel of its own with CTAs of 1024 threads (sorting a thousand
-    // keys is 55 rounds of compare-exchange: a round per barrier with 1024 threads, eight times that with the 128
-    // threads of a tables CTA); it refreshes every stream, which gives the streams without a frame in the batch
-    // the fast memory they already have.
-    const bool refresh_apart = tables && rz && a.n > 8 * kApplyThreads;
-    const bool refresh_here = tables && rz && !refresh_apart;
-    const size_t smem = tables ? tables_smem(a.n, rz ? rz->k_max : 0, refresh_here) : 0;
     ++*launches;
-    e = launch_chained(k_update_apply, table_ctas + centre_ctas, kApplyThreads, smem, st, a, rz ? *rz : ResizeArgs{},
-                       refresh_here ? 1 : 0, table_ctas);
+    e = launch_chained_cluster(k_update_apply, (table_ctas + centre_ctas + team - 1) / team * team, kApplyThreads, smem, team, st,
+                               a, rza, refresh_here ? 1 : 0, table_ctas);
     if (e != cudaSuccess || !refresh_apart) return e;
     return launch_resize(*rz, st, launches);
 }
