@@ -978,37 +978,37 @@ __global__ void __launch_bounds__(kLightThreads) k_lookup_sparse(const SparsePar
     chain_wait();  // the exit flags are the previous kernel's
     chain_release();
     const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);
-    // The active frames of this cluster and their streams.  Exit flags and stream ids of eight tiles of frames
-    // come in one trip to memory.
-    uint8_t flags[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    int sids[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    // The active frames of this cluster and their streams: every thread looks at four consecutive frames, one trip to
+    // memory and one scan for 512.  Active = not exited at an earlier layer: where the clusters do not all fit beside the
+    // streaming kernel, one of the first may have decided a frame before the last ones begin, and an exit at this very
+    // layer leaves it active, so that every cluster gets the same list whenever it looks.
+    constexpr int kPer = 4;
     int n_active = 0;
-    for (int t0 = 0; t0 < B; t0 += kLightThreads) {
-        const int b = t0 + tid;
-        if ((t0 / kLightThreads) % 8 == 0) {
+    for (int t0 = 0; t0 < B; t0 += kPer * kLightThreads) {
+        const int b0 = t0 + tid * kPer;
+        int act[kPer], sids[kPer], mine = 0;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                flags[u] = a.done[min(b + u * kLightThreads, B - 1)];
-                sids[u] = a.stream_id ? a.stream_id[min(b + u * kLightThreads, B - 1)] : 0;
-            }
+        for (int i = 0; i < kPer; ++i) {
+            act[i] = a.exit_layer[min(b0 + i, B - 1)];
+            sids[i] = a.stream_id ? a.stream_id[min(b0 + i, B - 1)] : 0;
         }
-        uint8_t mine = 0;
-        int sid_b = 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            mine = ((t0 / kLightThreads) % 8 == u) ? flags[u] : mine;
-            sid_b = ((t0 / kLightThreads) % 8 == u) ? sids[u] : sid_b;
+        for (int i = 0; i < kPer; ++i) {
+            act[i] = (b0 + i < B && (act[i] == 0 || act[i] == a.layer + 1)) ? 1 : 0;
+            mine += act[i];
         }
-        const int act = (b < B && !mine) ? 1 : 0;
         int cnt;
-        const int pos = block_exclusive_scan(act, s_scan, &cnt);
-        if (act) {
-            const int u = n_active + pos;
-            if (u % f.groups == group && u / f.groups < kSparseFrames) {
-                my_frames[u / f.groups] = b;
-                my_sids[u / f.groups] = sid_b;
+        int u = n_active + block_exclusive_scan(mine, s_scan, &cnt);
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+            if (act[i]) {
+                const int at = u / f.groups;
+                if (u - at * f.groups == group && at < kSparseFrames) {
+                    my_frames[at] = b0 + i;
+                    my_sids[at] = sids[i];
+                }
+                ++u;
             }
-        }
         n_active += cnt;
     }
     const int nu = n_active > group ? min((n_active - group + f.groups - 1) / f.groups, kSparseFrames) : 0;
