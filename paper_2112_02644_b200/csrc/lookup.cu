@@ -71,6 +71,205 @@ __device__ __forceinline__ Top2 block_top2_keys(unsigned long long b1, unsigned 
     return t;
 }
 
+// ---- large fast memories that all frames share, scored in fp32 ---------------------------------------
+//
+// A cache with one stream scores every frame against the same slots, so a centre that has been fetched serves several
+// frames.  A cluster of P CTAs takes F frames: every CTA keeps the F semantic vectors in shared memory and scores its share
+// of the slots, a warp 32 / F slots (at most eight) at a time; where the share is too small for eight warps they divide the
+// vector length as well.  The dot products of frame f meet, through distributed shared memory, in CTA f % P of the cluster,
+// which decides it.  What bounds it: the centres' way from L2 (k D words per cluster instead of per frame) and, for small
+// problems, the trips to memory ([exit layers, slots] -> [vectors, centres] -> decision).
+constexpr int kShareMost = 8;                    // frames, and CTAs, of a cluster at most
+constexpr long long kShareWork = 4608;           // words of centres below which a CTA per frame scores
+constexpr size_t kShareSmem = 200 * 1024;
+// Frames to a cluster: eight, fewer until every SM has a CTA.  CTAs to a cluster: eight, fewer where they would queue up for a
+// place on an SM (two each) and would have at most 64 slots.  Pooling and scoring of 1x1 maps by a CTA per frame and here, us,
+// 1024 channels: 256 frames against 101 slots 24 and 18, 1024 frames 56 and 32 (in clusters of eight 48), 256 against 999 167
+// and 39, 1024 400 and 126 (in clusters of two 108, but with a fifth of the frames left 105 instead of 36); 8 frames of 32
+// channels against 70 slots 12.7 and 9.1, 600 of 64 channels 26.3 and 21.5 (in clusters of eight 28.8).
+constexpr int kShareSlots = 64;
+// F vectors [F][D] | [F / P][k_max] dot products of the frames this CTA decides | [k_max] the slots' classes | partial sums
+// [8 warps][32].
+__host__ __device__ constexpr size_t share_smem(int F, int P, int D, int k_max) {
+    return (size_t(F) * D + size_t((F + P - 1) / P + 1) * size_t((k_max + 3) / 4 * 4) + 8 * 32) * sizeof(float);
+}
+
+template <int F>
+__global__ void __launch_bounds__(kThreads, 2) k_score_shared(const LookupArgs a, int P) {
+    constexpr int T = 32 / F < 8 ? 32 / F : 8;   // slots a warp scores together
+    constexpr int kSums = T * F;                 // 32, or fewer with one or two frames
+    constexpr int kWarps = kThreads / kWarp;
+    extern __shared__ __align__(16) float smem[];
+    __shared__ float scratch[33];
+    __shared__ unsigned long long s_keys[2 * kWarps];
+    __shared__ int s_frames[F];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int k_pad = (a.k_max + 3) / 4 * 4;
+    float* sv = smem;
+    float* dots = sv + size_t(F) * a.D;
+    int32_t* s_ids = reinterpret_cast<int32_t*>(dots + (F + P - 1) / P * k_pad);
+    float* s_part = reinterpret_cast<float*>(s_ids + k_pad);
+    const int group = int(blockIdx.x) / P, rank = int(blockIdx.x) - group * P;
+    chain_wait();
+    chain_release();
+    const ClockScope stamps(a.clock ? a.clock + 2 * (SMTM_PROF_SCORE + a.layer) : nullptr);
+    // This cluster's frames: number group * F ... of those still in.  Active = not exited at an earlier layer (an exit at
+    // this very layer is a decision of this launch), so every CTA gets the same list whenever it looks.
+    const int k = a.k[0];
+    for (int j = tid; j < a.k_max; j += kThreads) s_ids[j] = a.members[j];  // in flight with the exit layers
+    if (tid < F) s_frames[tid] = -1;
+    if (a.fresh) {
+        if (tid < F && group * F + tid < a.B) s_frames[tid] = group * F + tid;
+    } else {
+        constexpr int kPer = 4;
+        __syncthreads();
+        int before = 0;
+        for (int t0 = 0; t0 < a.B && before < (group + 1) * F; t0 += kPer * kThreads) {
+            int act[kPer], mine = 0;
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+                act[i] = *reinterpret_cast<const volatile int32_t*>(a.exit_layer + min(t0 + tid * kPer + i, a.B - 1));
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                act[i] = (t0 + tid * kPer + i < a.B && (act[i] == 0 || act[i] == a.layer + 1)) ? 1 : 0;
+                mine += act[i];
+            }
+            int cnt;
+            int at = before + block_exclusive_scan(mine, reinterpret_cast<int*>(scratch), &cnt) - group * F;
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+                if (act[i]) {
+                    if (at >= 0 && at < F) s_frames[at] = t0 + tid * kPer + i;
+                    ++at;
+                }
+            before += cnt;
+        }
+    }
+    __syncthreads();
+    if (s_frames[0] < 0) return;  // no frame is left for this cluster (the same for all its CTAs)
+    cluster_arrive();             // (waited for before the first store to a peer: it has to have started)
+    const int D4 = a.D >> 2;
+    for (int f = 0; f < F; ++f) {  // (a frame too few: the first one's vector again, dropped below)
+        const float4* row = reinterpret_cast<const float4*>(a.sv + (size_t)max(s_frames[f] < 0 ? s_frames[0] : s_frames[f], 0) * a.D);
+        for (int i = tid; i < D4; i += kThreads)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(reinterpret_cast<float4*>(sv) + f * D4 + i)), "l"(row + i)
+                         : "memory");
+    }
+    // what the first of this CTA's decisions needs, in flight with the vectors
+    float clen = 0.f, old = 0.f;
+    if (tid < k && rank < F && s_frames[rank < F ? rank : 0] >= 0) {
+        clen = a.cnorm[s_ids[tid]];
+        old = a.fresh ? 0.f : a.sa[(size_t)s_frames[rank < F ? rank : 0] * a.k_max + tid];
+    }
+    // this CTA's slots, the warps' groups of them and parts of the vector length
+    const int share = (k + P - 1) / P;
+    const int lo = min(k, rank * share), hi = min(k, lo + share);
+    const int groups = (share + T - 1) / T;
+    const int parts = groups >= 5 ? 1 : groups >= 3 ? 2 : groups == 2 ? 4 : 8;
+    const int part = warp % parts, per = (D4 + parts - 1) / parts;
+    const int q_lo = min(D4, part * per), q_hi = min(D4, q_lo + per);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    cluster_wait();
+    const float4* v4 = reinterpret_cast<const float4*>(sv);
+    const auto deliver = [&](int j, int f, float v) { peer_store(peer_smem(dots + f / P * k_pad + j, f % P), v); };
+    for (int g = warp / parts; g < groups; g += kWarps / parts) {
+        const int s0 = lo + g * T;
+        float d[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) d[e] = 0.f;
+        const float4* row[T];
+#pragma unroll
+        for (int t = 0; t < T; ++t)
+            row[t] = reinterpret_cast<const float4*>(a.centers + (size_t)s_ids[min(s0 + t, a.k_max - 1)] * a.D);
+        constexpr int kAhead = T <= 4 ? 2 : 1;  // pieces of a centre a lane asks for together
+        for (int q0 = q_lo; q0 < q_hi; q0 += kAhead * kWarp) {
+            float4 c[kAhead][T];
+#pragma unroll
+            for (int h = 0; h < kAhead; ++h)
+#pragma unroll
+                for (int t = 0; t < T; ++t) c[h][t] = row[t][min(q0 + h * kWarp + lane, q_hi - 1)];
+#pragma unroll
+            for (int h = 0; h < kAhead; ++h) {
+                const int q = q0 + h * kWarp + lane;
+                if (q < q_hi) {
+#pragma unroll
+                    for (int f = 0; f < F; ++f) {
+                        const float4 x = v4[f * D4 + q];
+#pragma unroll
+                        for (int t = 0; t < T; ++t)
+                            d[t * F + f] += fmaf(c[h][t].w, x.w, fmaf(c[h][t].z, x.z, fmaf(c[h][t].y, x.y, c[h][t].x * x.x)));
+                    }
+                }
+            }
+        }
+        // kSums sums over 32 lanes, halving what a lane still holds at every step; lane l ends up with sum number l / (32 / kSums)
+#pragma unroll
+        for (int o = 16, half = kSums / 2; o > 0; o >>= 1, half >>= 1) {
+            if (half > 0) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int e = 0; e < (half > 0 ? half : 1); ++e) {
+                    const float give = up ? d[e] : d[e + half], keep = up ? d[e + half] : d[e];
+                    d[e] = keep + __shfl_xor_sync(kFull, give, o);
+                }
+            } else {
+                d[0] += __shfl_xor_sync(kFull, d[0], o);
+            }
+        }
+        const int e = lane / (kWarp / kSums);
+        if (parts > 1) {
+            if (lane % (kWarp / kSums) == 0) s_part[warp * kWarp + e] = d[0];
+        } else {
+            const int j = s0 + e / F, f = e % F;
+            if (lane % (kWarp / kSums) == 0 && j < hi) deliver(j, f, d[0]);
+        }
+    }
+    if (parts > 1) {
+        __syncthreads();
+        const int g = tid / kSums, e = tid - g * kSums, j = lo + g * T + e / F;
+        if (g < groups && j < hi) {
+            float s = 0.f;
+            for (int p = 0; p < parts; ++p) s += s_part[(g * parts + p) * kWarp + e];
+            deliver(j, e % F, s);
+        }
+    }
+    __syncwarp();
+    cluster_sync_all();  // every slot of every frame is in
+    const float weight = float(1u << a.layer);  // 2^(l-1) with l = layer + 1
+    for (int f = rank; f < F && s_frames[f] >= 0; f += P) {
+        const int b = s_frames[f];
+        const int k_b = stream_of(a, b) < 0 ? 0 : k;  // a stream id outside the cache: nothing to score against
+        float nrm = 0.f;
+        for (int i = tid; i < D4; i += kThreads) {
+            const float4 x = v4[f * D4 + i];
+            nrm = fmaf(x.x, x.x, nrm); nrm = fmaf(x.y, x.y, nrm); nrm = fmaf(x.z, x.z, nrm); nrm = fmaf(x.w, x.w, nrm);
+        }
+        nrm = block_sum(nrm, scratch);
+        unsigned long long a1 = 0ull, a2 = 0ull, c1 = 0ull, c2 = 0ull;
+        for (int j = tid; j < a.k_max; j += kThreads) {
+            float* sa = a.sa + (size_t)b * a.k_max + j;
+            if (j < k_b) {
+                if (f != rank || j != tid) {  // (the first is here already)
+                    clen = a.cnorm[s_ids[j]];
+                    old = a.fresh ? 0.f : *sa;
+                }
+                const float sim = cosine_from(dots[f / P * k_pad + j], nrm, clen);  // Eq. 1
+                const float acc = __fmaf_rn(sim, weight, old);                      // Eq. 3
+                *sa = acc;
+                keep_two(rank_key(acc, s_ids[j]), a1, a2);
+                if (a.sep) keep_two(rank_key(sim, s_ids[j]), c1, c2);  // only Eq. 2 (a diagnostic) needs it
+            } else if (a.fresh) {
+                *sa = 0.f;  // unused slots start from zero too
+            }
+        }
+        const Top2 ta = block_top2_keys(a1, a2, s_keys);
+        Top2 ts{0.f, 0.f, -1, -1};
+        if (a.sep) ts = block_top2_keys(c1, c2, s_keys);
+        if (tid == 0) decide_from_top2(a, b, ta, ts);
+    }
+}
+
 // Finishing kernel of the tensor-core path: one CTA per frame turns the frame's row of dot products into
 // similarities of its fast-memory slots and decides.  The row (its parts added) and the
 // centres' lengths come in with coalesced 16-byte loads and are parked in shared memory, from where the slots
@@ -227,6 +426,10 @@ cudaError_t launch_wait_selftest(int* status, cudaStream_t st, int64_t* launches
 cudaError_t lookup_setup() {
     cudaError_t e = allow_max_dynamic_smem(k_score_exit<4>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_score_exit<5>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_score_shared<1>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_score_shared<2>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_score_shared<4>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_score_shared<8>);
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_score_exit<4>);
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_score_exit<5>);
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_finish_dense<true>);
@@ -255,9 +458,30 @@ cudaError_t launch_finish_dense(const LookupArgs& a, const DenseDots& dots, bool
     return launch_chained(kernel, a.B, kFinishThreads, smem, st, a, dots);
 }
 
+// Frames to a cluster of k_score_shared, or 0 where a CTA per frame scores them; *ctas: CTAs of a cluster.
+static int shared_frames(const LookupArgs& a, int sm_count, int* ctas) {
+    if (a.S != 1 || a.k_max <= kFusedMaxK || (a.D & 3) || (long long)a.k_max * std::max(a.D, 64) < kShareWork) return 0;
+    const int frames = a.fresh ? a.B : (a.B + 1) / 2;  // (after a first lookup half of them are taken to be still in)
+    const auto groups = [&](int F) { return (frames + F - 1) / F; };
+    int F = kShareMost, P = kShareMost;
+    while (F > 1 && groups(F) * P < sm_count) F /= 2;
+    while (P > 1 && groups(F) * P > 2 * sm_count && a.k_max <= kShareSlots * P) P /= 2;
+    while (F > 1 && share_smem(F, P, a.D, a.k_max) > kShareSmem) F /= 2;
+    *ctas = P;
+    return share_smem(F, P, a.D, a.k_max) > kShareSmem ? 0 : F;
+}
+
 cudaError_t launch_score_exit(const LookupArgs& a, cudaStream_t st, int sm_count, int64_t* launches, int threads,
                               bool in_order) {
     if (a.B <= 0) return cudaSuccess;
+    int P = 0;
+    if (const int F = shared_frames(a, sm_count, &P)) {
+        const auto kernel = F == 1 ? k_score_shared<1> : F == 2 ? k_score_shared<2> : F == 4 ? k_score_shared<4> : k_score_shared<8>;
+        const size_t smem = share_smem(F, P, a.D, a.k_max);
+        ++*launches;
+        if (in_order) return launch_ordered_cluster(kernel, (a.B + F - 1) / F * P, kThreads, smem, P, st, a, P);
+        return launch_chained_cluster(kernel, (a.B + F - 1) / F * P, kThreads, smem, P, st, a, P);
+    }
     const auto rounds = [&](int ctas) { return (a.B + ctas * sm_count - 1) / (ctas * sm_count); };
     const auto kernel = rounds(5) < rounds(4) ? k_score_exit<5> : k_score_exit<4>;
     const size_t smem = (size_t(a.D) + 3 * size_t(a.k_max)) * sizeof(float);

@@ -1,7 +1,11 @@
-"""Scoring on the GPU: which frames a later layer's kernel takes up."""
+"""Scoring on the GPU: which frames a later layer's kernel takes up, and large fast memories that all frames share."""
+import numpy as np
 import pytest
+import torch
 
+import paper_2112_02644_b200 as smtm
 import smtm_inputs as si
+from harness import launches, run_workload
 from test_gpu_shapes import test_maps_ready_with_odd_widths as ready_steps
 
 pytestmark = pytest.mark.gpu
@@ -12,3 +16,40 @@ def test_exits_of_a_later_layer_do_not_move_the_frames_of_clusters_that_begin_la
     # that begins after the first decisions takes up the frames it would have taken up before them
     ready_steps(si.Workload("late_clusters", si.BF16, si.NCHW, B=512, stages=((256, 14, 14), (2048, 7, 7)), n=60, k_init=12,
                             k_min=8, k_max=16, S=512, T=4, tau=0.81, sigma=1.0, zipf_s=0.5, repeat_p=0.8, seed=95))
+
+
+# fast memories of more than 64 slots that all frames share: eight, four, two or one frame to a cluster, slots in whole and
+# ragged shares, warps that divide the vector length, a later layer with few frames left, one with vectors of odd widths
+def shared(name, B, n, stages, **kw):
+    kw = dict(dict(k_init=n, k_min=max(66, n // 2), k_max=n, T=3, window_W=3, sigma=0.5, zipf_s=0.8, repeat_p=0.3, seed=96), **kw)
+    return si.Workload(name, si.F16, si.NHWC, B=B, stages=stages, n=n, **kw)
+
+
+SHARED = [
+    (shared("eight_frames", 150, 101, ((1024, 2, 2), (2048, 1, 1)), tau=0.3), [(8, 8), (4, 8)]),
+    (shared("four_frames", 77, 201, ((128, 3, 3), (260, 2, 2))), [(4, 8), (2, 8)]),
+    (shared("two_frames", 38, 75, ((2048, 2, 1),)), [(2, 8)]),
+    (shared("one_frame", 5, 999, ((24, 3, 3), (1028, 1, 2)), k_min=60), [(1, 8), (1, 8)]),
+    (shared("many_slots", 301, 1999, ((136, 1, 1), (36, 2, 2)), k_min=1500, T=2), [(8, 8), (8, 8)]),
+    (shared("long_vector", 148, 66, ((9000, 1, 1),), T=2), [(4, 8)]),
+    (shared("crowd", 601, 101, ((260, 2, 1), (64, 2, 2)), T=2), [(8, 2), (8, 4)]),
+    (shared("queue", 400, 257, ((64, 3, 1),), T=2), [(8, 4)]),
+]
+
+
+@pytest.mark.parametrize("w,split", SHARED, ids=lambda v: getattr(v, "name", ""))
+def test_scoring_of_large_fast_memories_that_all_frames_share(w, split):
+    cache = smtm.smtm_cache_create(w.n, w.dims, [0.8] * w.L, [np.ones((w.n, d), np.float32) for d in w.dims], None,
+                                   k_init=w.k_init, k_min=w.k_min, k_max=w.k_max, max_batch=w.B)
+    batch = smtm.Batch(cache, w.B)
+    for l in range(w.L):
+        B, C, H, W = si.shape4(w, l)
+        x = torch.zeros((B, H, W, C), dtype=torch.float16, device="cuda")
+        call = smtm.smtm_lookup_exit if l else smtm.smtm_lookup_exit_begin
+        got = launches(lambda: call(cache, l, smtm.Fmap(x, w.dtype, w.layout, B, C, H, W), batch))
+        F, P = split[l]   # frames and CTAs of a cluster
+        assert got[-1].kernel == "k_score_shared" and "ILi%dE" % F in got[-1].variant
+        assert (got[-1].cluster, got[-1].grid) == (P, P * -(-B // F))
+    smtm.smtm_cache_destroy(cache)
+    rep = run_workload(w)
+    assert rep.frames == w.B * w.T and rep.routes == [0, 0, w.L * w.T, 0, 0]
