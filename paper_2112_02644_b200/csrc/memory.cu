@@ -1015,8 +1015,8 @@ __device__ __forceinline__ void centre_item(const UpdateArgs& a, int l0, int cls
     float nrm = 0.f;
     int q = 0;
     if ((D & 3) == 0) {
-        const int D4 = D >> 2, per_blk = (D4 + nblk - 1) / nblk;
-        const int lo4 = min(D4, blk * per_blk), hi4 = min(D4, lo4 + per_blk);  // this item's 16-byte column groups
+        const int D4 = D >> 2;
+        const int lo4 = D4 * blk / nblk, hi4 = D4 * (blk + 1) / nblk;  // this item's 16-byte column groups (never none: D4 >= nblk)
         int R = 1;                                                             // row groups
         while (R < kRowGroupsMax && 2 * R * (hi4 - lo4) <= nt) R *= 2;
         const int cpp = nt / R;                                                // column groups per sweep

@@ -28,6 +28,10 @@ def workload(name, B, n, stages=((64, 2, 2),), S=1, **kw):
     (workload("crowded", 300, 256, stages=((64, 2, 2),) * 5), ["k_update_plan_one", "k_update_apply"], 2),
     (workload("many_layers", 128, 30, stages=((64, 2, 2),) * 16), ["k_update_direct"], 1),
     (workload("wide_vector", 3, 5, stages=((16384, 1, 1),), k_max=5), ["k_update_direct"], 1),
+    # (vectors of 210 and 274 16-byte pieces in sixteen blocks: with ceil(210 / 16) pieces to a block the last one had none)
+    (workload("ragged_blocks", 300, 3, stages=((840, 1, 1), (1096, 1, 1)), k_init=3, k_max=3, tau=9.0), ["k_update_direct"], 1),
+    (workload("ragged_blocks_600", 600, 3, stages=((840, 1, 1), (1096, 1, 1)), k_init=3, k_max=3, tau=9.0),
+     ["k_update_plan_one", "k_update_apply"], 1),
     (workload("odd_vector", 130, 20, stages=((37, 3, 2), (66, 2, 2))), ["k_update_direct"], 1),
     (workload("one_frame", 1, 1, k_init=1, k_min=1, k_max=1), ["k_update_direct"], 1),
     (workload("forgets", 200, 300, forgetting=True, T=6), ["k_update_direct"], 4),
