@@ -944,7 +944,14 @@ __global__ void __launch_bounds__(kLightThreads) k_pool_sparse(const LightParams
 // through distributed shared memory to the cluster's first CTA, whose first warp adds the parts in rank
 // order and decides (Eq. 1, Eq. 3, top-2, Eq. 4, the exit rule), as the fused streaming kernel does.  One
 // cluster-wide barrier per frame; two receive buffers take turns.  P = chunks per frame <= 8, and a chunk
-// here is a chunk of the streaming kernel (<= 25 KB): a whole frame is in flight at once.
+// here is a chunk of the streaming kernel (<= 25 KB): a whole frame is in flight at once.  What bounds it beside the pooling
+// kernel is how many clusters find a place.  With a whole chunk in shared memory three CTAs fit on an SM, and 55 clusters of
+// eight not all on the chip: the last ones began when the first were done (51 frames of 2048 7x7 channels out of 512 30 us,
+// alone 17).  With kHalves one half of a chunk is on its way to shared memory and the other to registers, from where it
+// follows, and four CTAs fit: a step of 512 streams 52.5 -> 47.4 us.  Where the frames are few enough for one round the
+// second pass is the longer way (64 frames in four exit layers 62.9 us a step, 65.2 in halves; 200 frames of 512 15x15 and
+// 1024 8x8 channels 38.0 and 39.6), so halves are for batches of more than four times the clusters that fit with whole
+// chunks (a later layer has a fraction of the batch).
 constexpr int kSparseStageCap = kStageCap;
 constexpr int kSparseFrames = 64;    // frames a cluster can be given
 constexpr int kSparseSlice = 1024;   // channels of a chunk at most (as the fused kernel's slices)
@@ -954,19 +961,21 @@ struct SparseParams {
     LookupArgs a;
     int groups;  // clusters
     int gran;    // channels that must stay in one warp's share (the reducer's unit)
+    int staged;  // channels of a chunk that the stage holds
 };
 
-constexpr size_t sparse_smem(int slice) {
-    return size_t(kSparseStageCap) + size_t(slice) * 4 + 2 * size_t(kMaxCluster) * kRxRow * 4 + 2 * kSparseFrames * 4 + 64 * 4 + 64;
+constexpr size_t sparse_smem(int slice, size_t stage) {
+    return (stage + 15) / 16 * 16 + size_t(slice) * 4 + 2 * size_t(kMaxCluster) * kRxRow * 4 + 2 * kSparseFrames * 4 + 64 * 4 + 64;
 }
 
-template <class R>
-__global__ void __launch_bounds__(kLightThreads) k_lookup_sparse(const SparseParams f) {
+// (Registers for three or four CTAs to an SM beside the 128 threads of the pooling kernel.)
+template <class R, bool kHalves>
+__global__ void __launch_bounds__(kLightThreads, kHalves ? 5 : 4) k_lookup_sparse(const SparseParams f) {
     extern __shared__ uint8_t smem_raw[];
     const NchwParams& p = f.e;
     const LookupArgs& a = f.a;
     uint8_t* stage = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 15) & ~uintptr_t(15));
-    float* sv_s = reinterpret_cast<float*>(stage + kSparseStageCap);       // [chunk_channels] this CTA's slice
+    float* sv_s = reinterpret_cast<float*>(stage + ((size_t(f.staged) * p.ch_bytes + 15) & ~size_t(15)));  // [chunk_channels] this CTA's slice
     float* rx = sv_s + p.chunk_channels;                                   // [2][P][kRxRow] (used in the first CTA)
     int* my_frames = reinterpret_cast<int*>(rx + 2 * kMaxCluster * kRxRow);  // [kSparseFrames]
     int* my_sids = my_frames + kSparseFrames;                              // [kSparseFrames] their stream ids
@@ -1016,22 +1025,24 @@ __global__ void __launch_bounds__(kLightThreads) k_lookup_sparse(const SparsePar
     const int c0 = rank * p.chunk_channels;
     const int nch = min(p.chunk_channels, p.C - c0);   // channels of this CTA's slice (a multiple of 4)
     const int vectors = nch * p.ch_bytes / 16;
-    const int units = (nch + f.gran - 1) / f.gran;
-    const int u_lo = min(units, warp * ((units + 3) / 4)), u_hi = min(units, u_lo + (units + 3) / 4);
-    const int w_c0 = u_lo * f.gran, w_nch = min(nch, u_hi * f.gran) - w_c0;
     const int n4 = nch >> 2;
     const int pp = (n4 + kWarp - 1) / kWarp;       // 16-byte pieces of a centre's slice per lane (at most 8)
     const int spr = max(1, 8 / max(pp, 1));        // slots a warp scores per trip to memory
     const float weight = float(1u << a.layer);     // 2^(l-1) with l = layer + 1
-    constexpr int kLoads = (kSparseStageCap / 16 + kLightThreads - 1) / kLightThreads;  // 13: a whole chunk in flight
+    constexpr int kLoads = (kSparseStageCap / 2 / 16 + kLightThreads - 1) / kLightThreads;  // 7: the second half of a chunk
+    const int first = kHalves ? min(nch, f.staged) : nch, v_first = first * p.ch_bytes / 16;
     for (int k_it = 0; k_it < nu; ++k_it) {
         const int b = my_frames[k_it];
         const int sid = stream_checked(a, my_sids[k_it]);
         const uint4* src = reinterpret_cast<const uint4*>(p.x + (long long)b * p.frame_bytes + (long long)c0 * p.ch_bytes);
         uint4* dst = reinterpret_cast<uint4*>(stage);
-        uint4 r[kLoads];
+        for (int v = tid; v < v_first; v += kLightThreads)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + v)), "l"(src + v) : "memory");
+        uint4 r[kHalves ? kLoads : 1];
+        if (kHalves) {
 #pragma unroll
-        for (int u = 0; u < kLoads; ++u) r[u] = load_once(src + min(u * kLightThreads + tid, vectors - 1));
+            for (int u = 0; u < kLoads; ++u) r[u] = load_once(src + min(v_first + u * kLightThreads + tid, vectors - 1));
+        }
         // the frame's fast memory: its size and this warp's classes (slot j = warp + 4 i), in flight with the chunk
         const int32_t* mem = a.members + (size_t)max(sid, 0) * a.k_max;
         const int k = sid < 0 ? 0 : min(a.k[sid], kFusedMaxK);
@@ -1043,13 +1054,25 @@ __global__ void __launch_bounds__(kLightThreads) k_lookup_sparse(const SparsePar
             ids[0] = lane < a.k_max ? mem[lane] : 0;
             ids[1] = lane + kWarp < a.k_max ? mem[lane + kWarp] : 0;
         }
-#pragma unroll
-        for (int u = 0; u < kLoads; ++u)
-            if (u * kLightThreads + tid < vectors) dst[u * kLightThreads + tid] = r[u];
+        const auto pool = [&](int h0, int hn) {  // the channels h0 .. of the chunk, by all warps: whole units each
+            const int share = ((hn + f.gran - 1) / f.gran + 3) / 4 * f.gran;
+            const int w_c0 = min(hn, warp * share), w_nch = min(hn, w_c0 + share) - w_c0;
+            if (w_nch > 0)
+                R::run(stage + size_t(w_c0) * p.ch_bytes, 0, w_nch, lane, p.sv + (long long)b * p.C + c0 + h0 + w_c0, sv_s + h0 + w_c0,
+                       p.inv_hw, p);
+        };
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        if (w_nch > 0)
-            R::run(stage + size_t(w_c0) * p.ch_bytes, 0, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, sv_s + w_c0, p.inv_hw, p);
-        __syncthreads();  // the slice is complete; the stage is free
+        pool(0, first);
+        __syncthreads();  // the first part of the slice is complete, the stage free
+        if (kHalves && first < nch) {
+#pragma unroll
+            for (int u = 0; u < kLoads; ++u)
+                if (v_first + u * kLightThreads + tid < vectors) dst[u * kLightThreads + tid] = r[u];
+            __syncthreads();
+            pool(first, nch - first);
+            __syncthreads();
+        }
         const uint32_t out = peer_smem(rx + ((k_it & 1) * kMaxCluster + rank) * kRxRow, 0);
         const float4* v4 = reinterpret_cast<const float4*>(sv_s);
         // the centres' lengths and the carry, for the finisher: in flight with the centre slices below
@@ -2015,8 +2038,10 @@ template <class R>
 cudaError_t carveout_pipelined() {
     cudaError_t e = prefer_max_smem_carveout(k_encode_nchw<R>);
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_pool_sparse<R>);
-    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_lookup_sparse<R>);
-    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_lookup_sparse<R>);
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_lookup_sparse<R, false>);
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_lookup_sparse<R, true>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_lookup_sparse<R, false>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_lookup_sparse<R, true>);
     return e;
 }
 
@@ -2164,6 +2189,7 @@ Reducer plan_sparse(const EncodeArgs& e, const LookupArgs& a, SparseParams* f) {
     const Reducer r = plan_nchw(e, &f->e);
     if (r == kNone) return kNone;
     if (f->e.chunks_per_frame > kMaxCluster || (f->e.chunk_channels & 3) || f->e.chunk_channels > kSparseSlice) return kNone;
+    f->staged = f->e.chunk_channels;
     f->gran = share_granularity(r, f->e);
     return r;
 }
@@ -2179,17 +2205,23 @@ cudaError_t launch_lookup_sparse(const EncodeArgs& e, const LookupArgs& a, int s
     if (r == kNone) return cudaErrorInvalidValue;
     f.a = a;
     const int P = f.e.chunks_per_frame;
-    // about three CTAs to an SM (they sit beside a streaming kernel); enough clusters that none is given more
+    // three or four CTAs to an SM (they sit beside a streaming kernel); enough clusters that none is given more
     // frames than it can list
-    int groups = std::max(1, std::min(e.B, 3 * sm_count / P));
+    const bool halves = e.B > 4 * (3 * sm_count / P);
+    if (halves) {
+        const int unit = unit_reducer(r) ? f.e.chunk_channels / 32 : any_width_reducer(r) ? aligned_channels(f.e.ch_bytes) : 1;
+        f.staged = std::min(f.staged, ((f.staged + 1) / 2 + unit - 1) / unit * unit);
+        if (f.staged < 4 * f.gran) f.gran = unit;  // (few channels: a warp takes fewer than it could)
+    }
+    int groups = std::max(1, std::min(e.B, (halves ? 4 : 3) * sm_count / P));
     groups = std::max(groups, (e.B + kSparseFrames - 1) / kSparseFrames);
     f.groups = groups;
-    const size_t smem = sparse_smem(f.e.chunk_channels);
+    const size_t smem = sparse_smem(f.e.chunk_channels, size_t(f.staged) * f.e.ch_bytes);
     cudaError_t err = cudaSuccess;
     ++*launches;
     // (in stream order, without the early start: the clusters would wait on the SMs for the scoring kernel before
     // them and keep the next step's pooling CTAs out meanwhile)
-#define SMTM_LAUNCH(...) err = launch_ordered_cluster(k_lookup_sparse<__VA_ARGS__>, P * groups, kLightThreads, smem, P, st, f)
+#define SMTM_LAUNCH(...) err = launch_ordered_cluster(halves ? k_lookup_sparse<__VA_ARGS__, true> : k_lookup_sparse<__VA_ARGS__, false>, P * groups, kLightThreads, smem, P, st, f)
     SMTM_FOR_REDUCER(r, SMTM_LAUNCH)
 #undef SMTM_LAUNCH
     return err;

@@ -18,6 +18,16 @@ def test_exits_of_a_later_layer_do_not_move_the_frames_of_clusters_that_begin_la
                             k_min=8, k_max=16, S=512, T=4, tau=0.81, sigma=1.0, zipf_s=0.5, repeat_p=0.8, seed=95))
 
 
+# batches large enough for the clusters that take a frame's chunks in halves: a last chunk shorter than half a chunk, channels
+# that are no whole vectors, chunks of one unit of channels
+@pytest.mark.parametrize("dt,stages", [
+    (si.BF16, ((64, 9, 9), (840, 8, 8))), (si.F16, ((32, 8, 8), (296, 9, 11), (1100, 5, 5))), (si.F32, ((16, 8, 8), (16, 40, 40))),
+    (si.F32, ((64, 7, 7), (1028, 7, 7)))], ids=lambda v: str(v) if isinstance(v, tuple) else None)
+def test_later_layers_of_large_batches(dt, stages):
+    ready_steps(si.Workload("halves", dt, si.NCHW, B=450, stages=stages, n=40, k_init=8, k_min=4, k_max=12, S=450, T=3, tau=0.75,
+                            sigma=1.0, zipf_s=0.5, repeat_p=0.8, seed=97))
+
+
 # fast memories of more than 64 slots that all frames share: eight, four, two or one frame to a cluster, slots in whole and
 # ragged shares, warps that divide the vector length, a later layer with few frames left, one with vectors of odd widths
 def shared(name, B, n, stages, **kw):
