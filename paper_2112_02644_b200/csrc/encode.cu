@@ -1605,6 +1605,7 @@ __global__ void __launch_bounds__(kThreadsNhwcLookup, E::kSize == 4 ? 3 : 2) k_l
     constexpr int T = kThreadsNhwcLookup;
     const int CG = C / V;  // 16-byte vectors per pixel
     const uint4* f = reinterpret_cast<const uint4*>(x + (long long)b * HW * C * E::kSize);
+    constexpr bool kOwnNorm = E::kSize == 2;
     float nrm = 0.f;
     for (int cg0 = 0; cg0 < CG; cg0 += T) {
         const int cgs = min(CG - cg0, T);  // column groups handled in this sweep
@@ -1638,12 +1639,12 @@ __global__ void __launch_bounds__(kThreadsNhwcLookup, E::kSize == 4 ? 3 : 2) k_l
             s *= inv_hw;
             sv_s[cg0 * V + c] = s;
             sv_out[(long long)b * C + cg0 * V + c] = s;
-            nrm = fmaf(s, s, nrm);
+            if (!kOwnNorm) nrm = fmaf(s, s, nrm);
         }
         __syncthreads();
     }
-    nrm = block_sum(nrm, scratch);  // also orders the shared writes above
-    score_frame(a, b, pf, sv_s, nrm, s_cur, s_acc);
+    if (!kOwnNorm) nrm = block_sum(nrm, scratch);
+    score_frame<kOwnNorm>(a, b, pf, sv_s, nrm, s_cur, s_acc);
 }
 
 // ---- NCHW without a stage: a warp per run of channels, straight from global memory -------------
@@ -1949,6 +1950,7 @@ Reducer plan_frame(const EncodeArgs& a, const LookupArgs& l, int sm_count, Frame
     const auto slice_of = [&](int parts) { return ((a.C + parts - 1) / parts + unit - 1) / unit * unit; };
     const bool many = l.k_max >= kFrameManySlots;
     const int wanted = many ? kFrameStageWantedMany : kFrameStageWanted, least = many ? kFrameStageLeastMany : kFrameStageLeast;
+    const int frames = l.fresh ? a.B : (a.B + 1) / 2;  // (after a first lookup half of them are taken to be still in)
     int best = 0;
     for (int P = 1; P <= kMaxCluster; P *= 2) {
         const int slice = slice_of(P);
@@ -1956,7 +1958,7 @@ Reducer plan_frame(const EncodeArgs& a, const LookupArgs& l, int sm_count, Frame
         if (P > 1 && slice * (P - 1) >= a.C) break;  // a CTA without channels
         if (slice > kFrameSlice || bytes > kFrameStageCap) continue;
         best = P;
-        if (bytes <= least || (bytes <= wanted && 2LL * a.B * P > sm_count)) break;
+        if (bytes <= least || (bytes <= wanted && 2LL * frames * P > sm_count)) break;
     }
     if (best == 0 || (long long)a.B * a.C * p.ch_bytes > kFrameBatchMost) return kNone;
     if (best > 1 && (long long)a.B * best > (many ? 4LL : 2LL) * kFrameResident * sm_count) return kNone;

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kThreads, kCtas) k_score_exit(const LookupArgs
         nrm = fmaf(v, v, nrm);
     }
     nrm = block_sum(nrm, scratch);  // also orders the shared writes above
-    score_frame(a, b, pf, sv, nrm, s_cur, s_acc);
+    score_frame<false>(a, b, pf, sv, nrm, s_cur, s_acc);
 }
 
 // The best two keys of the CTA, valid in thread 0.  (b1, b2): this thread's best two; s_keys: [2 * warps].

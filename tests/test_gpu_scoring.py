@@ -6,7 +6,7 @@ import torch
 import paper_2112_02644_b200 as smtm
 import smtm_inputs as si
 from harness import launches, run_workload
-from test_gpu_shapes import test_maps_ready_with_odd_widths as ready_steps
+from test_gpu_shapes import kernels_of_lookup, test_maps_ready_with_odd_widths as ready_steps
 
 pytestmark = pytest.mark.gpu
 
@@ -16,6 +16,13 @@ def test_exits_of_a_later_layer_do_not_move_the_frames_of_clusters_that_begin_la
     # that begins after the first decisions takes up the frames it would have taken up before them
     ready_steps(si.Workload("late_clusters", si.BF16, si.NCHW, B=512, stages=((256, 14, 14), (2048, 7, 7)), n=60, k_init=12,
                             k_min=8, k_max=16, S=512, T=4, tau=0.81, sigma=1.0, zipf_s=0.5, repeat_p=0.8, seed=95))
+
+
+# clusters of the kernel of small frames after a first lookup, when half of the frames are taken to be still in
+@pytest.mark.parametrize("B,begin,cluster", [(128, True, 1), (128, False, 2), (148, False, 2), (149, False, 1), (74, True, 2)])
+def test_clusters_of_later_lookups_of_small_frames(B, begin, cluster):
+    got = kernels_of_lookup(si.F16, si.NCHW, B, 256, 8, 8, 8, begin)
+    assert [(g.kernel, g.cluster) for g in got] == [("k_lookup_frame", cluster)]
 
 
 # batches large enough for the clusters that take a frame's chunks in halves: a last chunk shorter than half a chunk, channels
