@@ -287,7 +287,8 @@ smtm_status_t smtm_cache_get_counters(smtm_cache_t* cache, int64_t* h_out /*[SMT
  * layer i (i < SMTM_MAX_LAYERS: the fused lookup kernel, or the pooling kernel
  * of the other routes), for the scoring kernel of layer i where pooling and
  * scoring are separate kernels (SMTM_PROF_SCORE + i), for the update (the plan
- * kernel SMTM_PROF_PLAN; the CTAs of the apply kernel that fold centres,
+ * kernel SMTM_PROF_PLAN, or, where the update is one kernel, from its begin to
+ * the first centre that is folded; the CTAs of that kernel that fold centres,
  * _CENTERS, and those that keep the tables, _TABLES; the refresh of the fast
  * memories where it is a kernel of its own, _REFRESH) and for the dense route
  * (the tensor-core scorer SMTM_PROF_SCORE_TC and the decision kernel after it,
