@@ -163,6 +163,15 @@ __device__ __forceinline__ void peer_store(uint32_t addr, unsigned long long v) 
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
 }
 
+// The same with the store's bytes counted on a barrier of the CTA that receives them (both addresses that CTA's): whoever
+// waits for the barrier sees the value.  A barrier of the whole cluster costs as much as what lies before it (every thread's
+// earlier stores, to global memory too, have to be visible first: 1400 cycles of a lookup), this a trip between two SMs.
+__device__ __forceinline__ void peer_store_counted(uint32_t addr, float v, uint32_t bar_addr) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)),
+                 "r"(bar_addr)
+                 : "memory");
+}
+
 // Arrival on a barrier of any CTA of the cluster; orders this thread's earlier writes before it.
 __device__ __forceinline__ void peer_arrive(uint32_t bar_addr) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_addr) : "memory");

@@ -1238,11 +1238,19 @@ __device__ __forceinline__ void fetch_centres(const LookupArgs& a, const FrameSl
     }
 }
 
+// A part's value for the CTA that decides: counted on its barrier, or (bar == 0, a cluster of one) a plain store.
+__device__ __forceinline__ void deliver(uint32_t addr, float v, uint32_t bar) {
+    if (bar) peer_store_counted(addr, v, bar);
+    else peer_store(addr, v);
+}
+// What the deciding CTA's barrier has to count: a dot product per slot and a squared length from every part.
+__device__ __forceinline__ uint32_t parts_bytes(int P, int k) { return uint32_t(P) * uint32_t(k + 1) * 4u; }
+
 // Eq. 1's partial dot products of this warp's slots over the slice, into this part's row of the receive buffer in the
-// cluster's first CTA (`row`: its address there).  c: the pieces of the first slots, fetched already.  Eight sums are
+// cluster's first CTA (`row`: its address there; bar: 0, or the barrier there that counts what arrives).  c: the pieces of the first slots, fetched already.  Eight sums are
 // reduced over the warp together, halving what is left to exchange at every step: nine shuffles for eight.
 __device__ __forceinline__ void score_slots(const LookupArgs& a, const FrameSlots& s, int lg, int c0, int n4,
-                                            const float4* v4, uint32_t row, float4 (&c)[8]) {
+                                            const float4* v4, uint32_t row, uint32_t bar, float4 (&c)[8]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int per_trip = 8 >> lg;
     for (int i0 = 0; warp + kFrameWarps * i0 < s.k; i0 += per_trip) {
@@ -1273,12 +1281,12 @@ __device__ __forceinline__ void score_slots(const LookupArgs& a, const FrameSlot
         d[0] += __shfl_xor_sync(kFull, d[0], 2);
         d[0] += __shfl_xor_sync(kFull, d[0], 1);
         const int e = lane >> 2, j = warp + kFrameWarps * (i0 + (e >> lg));  // this lane's sum is number lane >> 2
-        if ((lane & 3) == 0 && (e & ((1 << lg) - 1)) == 0 && j < s.k) peer_store(row + j * 4, d[0]);
+        if ((lane & 3) == 0 && (e & ((1 << lg) - 1)) == 0 && j < s.k) deliver(row + j * 4, d[0], bar);
     }
 }
 
 // Squared length of the slice, by one warp.
-__device__ __forceinline__ void slice_norm(const float4* v4, int n4, uint32_t row) {
+__device__ __forceinline__ void slice_norm(const float4* v4, int n4, uint32_t row, uint32_t bar) {
     const int lane = threadIdx.x & 31;
     float nn = 0.f;
     for (int q = lane; q < n4; q += kWarp) {
@@ -1287,7 +1295,7 @@ __device__ __forceinline__ void slice_norm(const float4* v4, int n4, uint32_t ro
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nn += __shfl_xor_sync(kFull, nn, o);
-    if (lane == 0) peer_store(row + kFusedMaxK * 4, nn);
+    if (lane == 0) deliver(row + kFusedMaxK * 4, nn, bar);
 }
 
 // The decision by the first warp of the cluster's first CTA once every part's row is in: the parts added in rank
@@ -1340,6 +1348,7 @@ template <class R>
 __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FrameParams f) {
     extern __shared__ __align__(128) uint8_t frame_smem[];  // the map's slice | [slice] semantic vector | [P][kRxRow] receive rows
     __shared__ uint64_t landed[kFrameWarps];  // per warp: its share of the map
+    __shared__ uint64_t delivered;            // the first CTA's: every part's values
     const NchwParams& p = f.e;
     const LookupArgs& a = f.a;
     const int P = f.parts;
@@ -1353,6 +1362,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FramePa
     const uint64_t stream_once = l2_evict_first_policy();
     if (lane == 0) {
         mbar_init(&landed[warp], 1);
+        if (warp == 0) mbar_init(&delivered, 1);
         mbar_init_fence();
     }
     __syncwarp();
@@ -1375,6 +1385,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FramePa
     const bool decides = rank == 0 && warp == 0;
     const int sid = stream_checked(a, sid_raw);
     const FrameSlots slots = fetch_slots(a, sid, decides);
+    if (P > 1 && decides && lane == 0) mbar_expect_tx(&delivered, parts_bytes(P, slots.k));
     const int n4 = nch >> 2, lg = pieces_log2(n4);
     float4 cen[8];
     fetch_centres(a, slots, 0, lg, c0, 0, n4, cen);
@@ -1386,12 +1397,13 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FramePa
     }
     __syncthreads();
     if (P > 1) cluster_wait();
-    const uint32_t row = peer_smem(rx + rank * kRxRow, 0);
+    const uint32_t row = peer_smem(rx + rank * kRxRow, 0), bar = P > 1 ? peer_smem(&delivered, 0) : 0u;
     const float4* v4 = reinterpret_cast<const float4*>(sv_s);
-    if (warp == kFrameWarps - 1) slice_norm(v4, n4, row);
-    score_slots(a, slots, lg, c0, n4, v4, row, cen);
-    if (P > 1) cluster_sync_all(); else __syncthreads();  // every part has been delivered
-    if (decides) decide_parts(a, b, slots, rx, P, clen, sa_old);
+    if (warp == kFrameWarps - 1) slice_norm(v4, n4, row, bar);
+    score_slots(a, slots, lg, c0, n4, v4, row, bar, cen);
+    if (P == 1) __syncthreads();
+    if (decides && (P == 1 || mbar_wait_cluster_bounded(&delivered, 0, p.status)))  // every part has been delivered
+        decide_parts(a, b, slots, rx, P, clen, sa_old);
 }
 
 // ---- NHWC, small fast memory: pooling, scoring and the decision by a cluster per frame ---------------
@@ -1430,10 +1442,10 @@ __device__ __forceinline__ int fold_phases(float* part, int phases, int cols) {
     return groups;
 }
 
-// Sums pixels [px0, px1) of a frame over this CTA, U loads of a thread in flight; emit(c, sum) gets each column's; `part`:
-// T / cgs x cgs * V floats.
-template <class E, int T, int U, class Emit>
-__device__ __forceinline__ void column_sums(const uint8_t* frame, int C, int px0, int px1, float* part, Emit emit) {
+// Sums pixels [px0, px1) of a frame over this CTA, U loads of a thread in flight; emit(c, sum) gets each column's, after one
+// call of before() by all threads; `part`: T / cgs x cgs * V floats.
+template <class E, int T, int U, class Before, class Emit>
+__device__ __forceinline__ void column_sums(const uint8_t* frame, int C, int px0, int px1, float* part, Before before, Emit emit) {
     constexpr int V = E::kPerVec;
     const int CG = C / V;  // 16-byte vectors per pixel
     const uint4* f = reinterpret_cast<const uint4*>(frame);
@@ -1473,6 +1485,7 @@ __device__ __forceinline__ void column_sums(const uint8_t* frame, int C, int px0
         }
         __syncthreads();
         const int cols = cgs * V, rows = fold_phases<T>(part, phases, cols);
+        if (cg0 == 0) before();
         for (int c = threadIdx.x; c < cols; c += T) {
             float s = 0.f;
             for (int q = 0; q < rows; ++q) s += part[q * cols + c];
@@ -1480,6 +1493,12 @@ __device__ __forceinline__ void column_sums(const uint8_t* frame, int C, int px0
         }
         __syncthreads();
     }
+}
+
+// Column c's sum over this CTA's pixels to the CTA whose slice it belongs to: psum there holds a row of `slice` per CTA.
+__device__ __forceinline__ void send_column(float* psum, uint64_t* bar, int c, int slice, int rank, float s) {
+    const int r = c / slice;
+    peer_store_counted(peer_smem(psum + rank * slice + (c - r * slice), r), s, peer_smem(bar, r));
 }
 
 // Pooling alone: CTA `rank` of a frame's cluster sums a run of its pixels, then slice `rank` of the columns over the
@@ -1491,10 +1510,15 @@ __device__ __forceinline__ void column_sums(const uint8_t* frame, int C, int px0
 template <class E, int kLoads>
 __global__ void __launch_bounds__(kFrameThreads, kLoads == 2 ? 8 : kLoads == 4 ? 6 : 4) k_encode_nhwc(const uint8_t* x, const uint8_t* skip, float* sv, int C, int HW, float inv_hw, int P,
                                                                   int pixels, int slice, __nv_bfloat16* hi, __nv_bfloat16* lo,
-                                                                  unsigned long long* clock) {
-    extern __shared__ __align__(16) float nhwc_smem[];  // column sums [C] (clusters only) | phases' sums
+                                                                  int* status, unsigned long long* clock) {
+    extern __shared__ __align__(16) float nhwc_smem[];  // column sums of this CTA's slice [P][slice] (clusters only) | phases' sums
+    __shared__ uint64_t summed;                         // every CTA's sums of this slice are in
     float* psum = nhwc_smem;
     const int b = int(blockIdx.x) / P, rank = int(blockIdx.x) - b * P;
+    if (P > 1 && threadIdx.x == 0) {
+        mbar_init(&summed, 1);
+        mbar_init_fence();
+    }
     chain_wait();
     chain_release();
     const ClockScope stamps(clock);
@@ -1512,66 +1536,74 @@ __global__ void __launch_bounds__(kFrameThreads, kLoads == 2 ? 8 : kLoads == 4 ?
     };
     const uint8_t* frame = x + (long long)b * HW * C * E::kSize;
     if (P == 1) {
-        column_sums<E, kFrameThreads, kLoads>(frame, C, 0, HW, psum, write);
+        column_sums<E, kFrameThreads, kLoads>(frame, C, 0, HW, psum, [] {}, write);
         return;
     }
-    column_sums<E, kFrameThreads, kLoads>(frame, C, px0, px1, psum + C, [&](int c, float s) { psum[c] = s; });
-    cluster_sync_all();
+    cluster_arrive();  // (waited for before the first store to a peer: it has to have started)
     const int c0 = rank * slice, c1 = min(C, c0 + slice);
+    if (threadIdx.x == 0 && c1 > c0) mbar_expect_tx(&summed, uint32_t(P) * uint32_t(c1 - c0) * 4u);
+    column_sums<E, kFrameThreads, kLoads>(frame, C, px0, px1, psum + P * slice, [] { cluster_wait(); },
+                                          [&](int c, float s) { send_column(psum, &summed, c, slice, rank, s); });
+    if (c1 <= c0 || !mbar_wait_cluster_bounded(&summed, 0, status)) return;
     for (int c = c0 + threadIdx.x; c < c1; c += kFrameThreads) {
         float s = 0.f;
-        for (int r = 0; r < P; ++r) s += peer_load(peer_smem(psum + c, r));
+        for (int r = 0; r < P; ++r) s += psum[r * slice + (c - c0)];
         write(c, s);
     }
-    cluster_sync_all();  // no CTA leaves while a peer reads its sums
 }
 
 template <class E>
 __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame_nhwc(const FrameNhwcParams f) {
-    extern __shared__ __align__(16) float nhwc_smem[];  // column sums [C] | slice [slice] | receive rows [P][kRxRow] | phases' sums
+    extern __shared__ __align__(16) float nhwc_smem[];  // column sums of this CTA's slice [P][slice] | slice [slice] | receive rows [P][kRxRow] | phases' sums
+    __shared__ uint64_t summed, delivered;              // every CTA's sums of this slice; the first CTA's: every part's values
     const LookupArgs& a = f.a;
     const int P = f.parts;
     float* psum = nhwc_smem;
-    float* sv_s = psum + f.C;
+    float* sv_s = psum + P * f.slice;
     float* rx = sv_s + f.slice;
     float* part = rx + P * kRxRow;
     const int warp = threadIdx.x >> 5;
     const int b = int(blockIdx.x) / P, rank = int(blockIdx.x) - b * P;
+    if (threadIdx.x == 0) {
+        mbar_init(&summed, 1);
+        mbar_init(&delivered, 1);
+        mbar_init_fence();
+    }
     chain_wait();
     chain_release();
     const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);
     const int sid_raw = a.stream_id ? a.stream_id[b] : 0;  // in flight with the exit flag
     // (no CTA of the cluster can have decided yet: the decision comes after a barrier all of them arrive on)
     if (!a.fresh && a.done[b]) return;
+    cluster_arrive();  // (waited for before the first store to a peer: it has to have started)
     const bool decides = rank == 0 && warp == 0;
-    const FrameSlots slots = fetch_slots(a, stream_checked(a, sid_raw), decides);  // in flight with the map
-    const int px0 = rank * f.pixels, px1 = min(f.HW, px0 + f.pixels);
-    column_sums<E, kFrameThreads, 8>(f.x + (long long)b * f.HW * f.C * E::kSize, f.C, px0, px1, part,
-                                        [&](int c, float s) { psum[c] = s; });
     const int c0 = rank * f.slice, nch = max(0, min(f.slice, f.C - c0));
+    const FrameSlots slots = fetch_slots(a, stream_checked(a, sid_raw), decides);  // in flight with the map
+    if (threadIdx.x == 0 && nch > 0) mbar_expect_tx(&summed, uint32_t(P) * uint32_t(nch) * 4u);
+    const int px0 = rank * f.pixels, px1 = min(f.HW, px0 + f.pixels);
+    column_sums<E, kFrameThreads, 8>(f.x + (long long)b * f.HW * f.C * E::kSize, f.C, px0, px1, part, [] { cluster_wait(); },
+                                     [&](int c, float s) { send_column(psum, &summed, c, f.slice, rank, s); });
+    if (decides && threadIdx.x == 0) mbar_expect_tx(&delivered, parts_bytes(P, slots.k));
     const int n4 = nch >> 2, lg = pieces_log2(n4);
     float4 cen[8];
     fetch_centres(a, slots, 0, lg, c0, 0, n4, cen);  // in flight with the exchange
     float clen[2] = {0.f, 0.f}, sa_old[2] = {0.f, 0.f};
     if (decides) fetch_lengths(a, b, slots, clen, sa_old);
-    if (P > 1) cluster_sync_all();
+    if (nch > 0) mbar_wait_cluster_bounded(&summed, 0, a.status);
     for (int c = threadIdx.x; c < nch; c += kFrameThreads) {
         float s = 0.f;
-        if (P > 1)
-            for (int r = 0; r < P; ++r) s += peer_load(peer_smem(psum + c0 + c, r));
-        else
-            s = psum[c];
+        for (int r = 0; r < P; ++r) s += psum[r * f.slice + c];
         s *= f.inv_hw;
         sv_s[c] = s;
         f.sv[(long long)b * f.C + c0 + c] = s;
     }
     __syncthreads();
-    const uint32_t row = peer_smem(rx + rank * kRxRow, 0);
+    const uint32_t row = peer_smem(rx + rank * kRxRow, 0), bar = peer_smem(&delivered, 0);
     const float4* v4 = reinterpret_cast<const float4*>(sv_s);
-    if (warp == kFrameWarps - 1) slice_norm(v4, n4, row);
-    score_slots(a, slots, lg, c0, n4, v4, row, cen);
-    if (P > 1) cluster_sync_all(); else __syncthreads();  // every part has been delivered (and every peer's sums are read)
-    if (decides) decide_parts(a, b, slots, rx, P, clen, sa_old);
+    if (warp == kFrameWarps - 1) slice_norm(v4, n4, row, bar);
+    score_slots(a, slots, lg, c0, n4, v4, row, bar, cen);
+    if (decides && mbar_wait_cluster_bounded(&delivered, 0, a.status))  // every part has been delivered
+        decide_parts(a, b, slots, rx, P, clen, sa_old);
 }
 
 // ---- NHWC, small fast memory: pooling, scoring and the decision by one CTA per frame ---------------
@@ -2005,11 +2037,11 @@ bool plan_frame_nhwc(const EncodeArgs& a, const LookupArgs* l, int sm_count, Fra
     return true;
 }
 
-// Shared memory of the column sums: the sums (of a CTA of a cluster) and the phases' parts.
+// Shared memory of the column sums: the slice's sums (a row per CTA of a cluster) and the phases' parts.
 size_t nhwc_smem_bytes(const EncodeArgs& a, const FrameNhwcParams& f) {
     const int V = a.dtype == SMTM_F32 ? 4 : 8;
     const int cgs = std::min(a.C / V, kFrameThreads);
-    return ((f.parts > 1 ? size_t(a.C) : 0) + size_t(kFrameThreads / cgs) * cgs * V) * sizeof(float);
+    return ((f.parts > 1 ? size_t(f.parts) * f.slice : 0) + size_t(kFrameThreads / cgs) * cgs * V) * sizeof(float);
 }
 
 template <class R>
@@ -2086,7 +2118,7 @@ cudaError_t launch_encode(const EncodeArgs& a, int sm_count, cudaStream_t st, in
 #define SMTM_LAUNCH(E) \
     e = launch_chained_cluster(loads == 2 ? k_encode_nhwc<E, 2> : loads == 4 ? k_encode_nhwc<E, 4> : k_encode_nhwc<E, 8>, a.B * f.parts, kFrameThreads, nhwc_smem_bytes(a, f), f.parts, st, f.x, a.skip, \
                                a.sv, a.C, f.HW, f.inv_hw, f.parts, f.pixels, f.slice, static_cast<__nv_bfloat16*>(a.sv_hi), \
-                               static_cast<__nv_bfloat16*>(a.sv_lo), a.clock)
+                               static_cast<__nv_bfloat16*>(a.sv_lo), a.status, a.clock)
             SMTM_FOR_TYPE(a.dtype, SMTM_LAUNCH)
 #undef SMTM_LAUNCH
             return e;
