@@ -1022,6 +1022,7 @@ __global__ void __launch_bounds__(kLightThreads, kHalves ? 5 : 4) k_lookup_spars
     }
     const int nu = n_active > group ? min((n_active - group + f.groups - 1) / f.groups, kSparseFrames) : 0;
     __syncthreads();
+    if (P > 1) cluster_arrive_relaxed();  // (waited for before the first store to a peer: it has to have started)
     const int c0 = rank * p.chunk_channels;
     const int nch = min(p.chunk_channels, p.C - c0);   // channels of this CTA's slice (a multiple of 4)
     const int vectors = nch * p.ch_bytes / 16;
@@ -1073,6 +1074,7 @@ __global__ void __launch_bounds__(kLightThreads, kHalves ? 5 : 4) k_lookup_spars
             pool(first, nch - first);
             __syncthreads();
         }
+        if (P > 1 && k_it == 0) cluster_wait();
         const uint32_t out = peer_smem(rx + ((k_it & 1) * kMaxCluster + rank) * kRxRow, 0);
         const float4* v4 = reinterpret_cast<const float4*>(sv_s);
         // the centres' lengths and the carry, for the finisher: in flight with the centre slices below
@@ -1156,7 +1158,8 @@ __global__ void __launch_bounds__(kLightThreads, kHalves ? 5 : 4) k_lookup_spars
             if (lane == 0) decide_from_top2(a, b, ta, ts);
         }
     }
-    if (P > 1) cluster_sync_all();  // no CTA leaves while a peer may still write to its shared memory
+    if (P > 1 && nu == 0) cluster_wait();
+    else if (P > 1) cluster_sync_all();  // no CTA leaves while a peer may still write to its shared memory
 }
 
 // ---- lookup of small frames: a cluster of small CTAs per frame, nothing persistent -----------------

@@ -19,3 +19,19 @@ def test_what_the_kernel_before_writes_is_read_by_ordinary_loads():
     for f, text in src.items():
         for params in re.findall(r"__global__[^{;]*?\bk_\w+\(([^)]*)\)", text):
             assert not re.search(r"const[^,]*__restrict__", params), (f, params)
+
+
+def test_a_peer_is_known_to_have_started_before_its_shared_memory_is_written():
+    # the CTAs of a cluster need not begin together: a barrier all of them have arrived on comes before the first store
+    stores, checked = r"peer_store|peer_arrive|send_column\(|score_slots\(|slice_norm\(|deliver\(", set()
+    for f, text in sources().items():
+        for body in re.split(r"\n__(?:global|device)__|\ntemplate", text):
+            store = re.search(stores, body)
+            name = re.search(r"\b(k_\w+|tables_of_lone_stream)\(", body)
+            if not (store and name and name.start() < body.index("{")):
+                continue
+            wait = re.search(r"cluster_wait\(\)|cluster_sync_all\(\)", body)
+            assert wait and wait.start() < store.start(), (f, name.group(1))
+            checked.add(name.group(1))
+    assert checked >= {"k_lookup_nchw", "k_lookup_sparse", "k_lookup_frame", "k_lookup_frame_nhwc", "k_encode_nhwc", "k_score_shared",
+                       "tables_of_lone_stream"}
