@@ -163,9 +163,7 @@ smtm_status_t smtm_encode(smtm_cache_t* cache, int32_t layer, const smtm_fmap_t*
  * when  SA_H > 0  and  SA_H - SA_SH > tau * max(SA_SH, 0)  (Eq. 4's AC > tau,
  * division-free, evaluated in fp32), which sets d_done, d_exit_layer = layer+1
  * and d_pred.  Fewer than two members never exit.  A zero-length vector has
- * similarity 0 to everything.  The fused route decides inside the streaming
- * kernel and tells the frames that are still in from d_exit_layer (0, or this
- * very layer when another CTA of the same launch has just decided the frame). */
+ * similarity 0 to everything. */
 smtm_status_t smtm_lookup_exit(smtm_cache_t* cache, int32_t layer, const smtm_fmap_t* fmap,
                                const smtm_batch_t* batch, void* stream);
 

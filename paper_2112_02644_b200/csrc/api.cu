@@ -333,12 +333,16 @@ smtm_status_t lookup_impl(smtm_cache* c, int32_t layer, const smtm_fmap_t* f, co
         // those do not serve, small CTAs pool them and small CTAs score them
         if (timing) SMTM_CUDA(record_timing(timing[0], st));
         const bool whole = launch_lookup_sparse_supported(e, a);
+        a.pending = whole ? 1 : 0;
         if (whole)
             SMTM_CUDA(launch_lookup_sparse(e, a, c->sm_count, st, &c->launches));
         else
             SMTM_CUDA(launch_pool_sparse(e, c->sm_count, st, &c->launches));
         if (timing) SMTM_CUDA(record_timing(timing[1], st));
-        if (!whole) SMTM_CUDA(launch_score_exit(a, st, c->sm_count, &c->launches, kPipelinedScoreThreads));
+        if (whole)
+            SMTM_CUDA(launch_settle_exits(a, st, &c->launches));
+        else
+            SMTM_CUDA(launch_score_exit(a, st, c->sm_count, &c->launches, kPipelinedScoreThreads));
         return SMTM_OK;
     }
     if (pipelined_nhwc) {

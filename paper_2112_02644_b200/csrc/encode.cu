@@ -612,14 +612,9 @@ __global__ void __launch_bounds__(kThreadsFused, 1) k_lookup_nchw(const FusedPar
     const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);  // profiling
     for (int t0 = 0; !a.fresh && t0 < a.B; t0 += kThreadsFused) {
         const int b = t0 + threadIdx.x;
-        // Active = not exited at an earlier layer.  A finisher of this launch may already have
-        // decided the frame: an exit at this very layer leaves it active, so every CTA gets
-        // the same list whenever it looks.
-        int act = 0;
-        if (b < a.B) {
-            const int el = *reinterpret_cast<const volatile int32_t*>(a.exit_layer + b);
-            act = (el == 0 || el == a.layer + 1) ? 1 : 0;
-        }
+        // (A finisher of this launch may already have decided the frame: its exit is pending, the flag is what it was
+        // before, so every CTA gets the same list whenever it looks.)
+        const int act = (b < a.B && !a.done[b]) ? 1 : 0;
         int cnt;
         const int pos = block_exclusive_scan(act, s_scan, &cnt);
         if (act) {
@@ -988,9 +983,9 @@ __global__ void __launch_bounds__(kLightThreads, kHalves ? 5 : 4) k_lookup_spars
     chain_release();
     const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);
     // The active frames of this cluster and their streams: every thread looks at four consecutive frames, one trip to
-    // memory and one scan for 512.  Active = not exited at an earlier layer: where the clusters do not all fit beside the
-    // streaming kernel, one of the first may have decided a frame before the last ones begin, and an exit at this very
-    // layer leaves it active, so that every cluster gets the same list whenever it looks.
+    // memory and one scan for 512.  Where the clusters do not all fit beside the streaming kernel, one of the first may have
+    // decided a frame before the last ones begin: its exit is pending, the flag is what it was before the launch, so that
+    // every cluster gets the same list whenever it looks.
     constexpr int kPer = 4;
     int n_active = 0;
     for (int t0 = 0; t0 < B; t0 += kPer * kLightThreads) {
@@ -998,12 +993,12 @@ __global__ void __launch_bounds__(kLightThreads, kHalves ? 5 : 4) k_lookup_spars
         int act[kPer], sids[kPer], mine = 0;
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
-            act[i] = a.exit_layer[min(b0 + i, B - 1)];
+            act[i] = a.done[min(b0 + i, B - 1)];
             sids[i] = a.stream_id ? a.stream_id[min(b0 + i, B - 1)] : 0;
         }
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
-            act[i] = (b0 + i < B && (act[i] == 0 || act[i] == a.layer + 1)) ? 1 : 0;
+            act[i] = (b0 + i < B && act[i] == 0) ? 1 : 0;
             mine += act[i];
         }
         int cnt;
@@ -2367,6 +2362,7 @@ cudaError_t launch_lookup_fused(const EncodeArgs& e, const LookupArgs& a, int sm
         return cudaSuccess;
     const int P = best_P;
     f.a = a;
+    f.a.pending = a.fresh ? 0 : 1;
     f.parts = P;
     f.chunks_per_unit = cpf / P;
     f.slice_cap = f.chunks_per_unit * f.e.chunk_channels;
@@ -2379,7 +2375,7 @@ cudaError_t launch_lookup_fused(const EncodeArgs& e, const LookupArgs& a, int sm
     if (timing) record_timing(timing[1], st);
     ++*launches;
     *served = kServedFused;
-    return err;
+    return err == cudaSuccess && f.a.pending ? launch_settle_exits(f.a, st, launches) : err;
 }
 
 cudaError_t launch_row_norm2(const float* sv, const uint8_t* skip, int B, int D, float* out, cudaStream_t st,

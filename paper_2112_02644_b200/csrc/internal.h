@@ -141,6 +141,7 @@ struct LookupArgs {
     int S;                    // streams of the cache: a frame whose stream id lies outside [0, S) is not looked up
     int* status;              // device sticky status word
     int fresh;                // the batch starts here: the carry is taken as SA = 0, nobody done, and is overwritten
+    int pending;              // exits are left pending in exit_layer and made final by k_settle_exits (see decide_core)
     float tau;
     const float* sv;          // [B][D]
     const float* centers;     // [n][D]
@@ -159,7 +160,8 @@ struct LookupArgs {
     unsigned long long* clock;  // nullptr, or the profiled step's stamps [SMTM_PROF_KERNELS][2] (see ClockScope)
 };
 // threads: CTA size (a multiple of 32, at most 256; 0 = 256).  Smaller CTAs fit beside a streaming kernel.
-// in_order: without the early start (see launch_ordered).
+// in_order: without the early start (see launch_ordered).  A large crowd that is scored by clusters is followed by
+// k_settle_exits.
 cudaError_t launch_score_exit(const LookupArgs& a, cudaStream_t st, int sm_count, int64_t* launches, int threads = 0,
                               bool in_order = false);
 // Encode + score + exit in one kernel (fast memories of at most 64 entries): NCHW shapes the streaming pipeline serves,
@@ -170,6 +172,7 @@ constexpr int kFusedMaxK = 64;  // fast-memory capacity the fused path supports 
 // Lookup (pooling, scoring, decision) of the frames still in at a later layer by clusters of small CTAs that fit
 // beside a streaming kernel: NCHW shapes the streaming pipeline cuts into at most 8 chunks per frame.
 bool launch_lookup_sparse_supported(const EncodeArgs& e, const LookupArgs& a);
+// (a.pending has to be set; launch_settle_exits follows.)
 cudaError_t launch_lookup_sparse(const EncodeArgs& e, const LookupArgs& a, int sm_count, cudaStream_t st, int64_t* launches);
 // What the device answered when asked how many clusters of 2, 4, 8 CTAs of each variant of the fused
 // kernel it runs at once (0 = not asked yet, -1 = refused); kept per cache, i.e. per device.
@@ -209,6 +212,8 @@ size_t dense_centers_split_bytes(int n, int D);
 // beside_pooling: the next batch's pooling kernel runs meanwhile (launched in stream order, see launch_ordered).
 cudaError_t launch_finish_dense(const LookupArgs& a, const DenseDots& dots, bool beside_pooling, cudaStream_t st,
                                 int64_t* launches);
+// Makes the exits that a lookup with a.pending has left pending final.
+cudaError_t launch_settle_exits(const LookupArgs& a, cudaStream_t st, int64_t* launches);
 // One warp that waits, bounded, on a barrier nobody arrives on (the self-test of the time-out path).
 cudaError_t launch_wait_selftest(int* status, cudaStream_t st, int64_t* launches);
 cudaError_t launch_batch_reset(float* sa, uint8_t* done, int32_t* exit_layer, int32_t* pred, int B, int k_max,

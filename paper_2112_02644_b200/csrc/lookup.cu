@@ -94,6 +94,15 @@ __host__ __device__ constexpr size_t share_smem(int F, int P, int D, int k_max) 
     return (size_t(F) * D + size_t((F + P - 1) / P + 1) * size_t((k_max + 3) / 4 * 4) + 8 * 32) * sizeof(float);
 }
 
+// Which frames: those of F consecutive ones that are still in, decided by the same cluster, so that nobody else's decision
+// can change them.  Where that would leave much undone by clusters whose frames have mostly left (more CTAs than the chip
+// holds, or much work to a CTA), every CTA lists the frames still in for itself and a cluster takes the next F of the list;
+// their exits stay pending until the launch is over.  Half of the frames still in, us, as they lie and listed: 256 frames
+// of 2048 channels against 101 classes 24.8 and 20.7, 600 of 1024 against 301 40.2 and 31.4, 64 of 64 (a frame to a cluster:
+// nothing to gain) 11.0 and 13.4; the few that are left as they lie and would be faster listed are crowds of short vectors
+// (600 of 64 channels against 75 classes 18.3 and 13.9).
+constexpr int kShareOwnWork = 1 << 17, kShareOwnWorkCrowd = 1 << 14;  // products to a CTA; the second in clusters of fewer than eight
+
 template <int F>
 __global__ void __launch_bounds__(kThreads, 2) k_score_shared(const LookupArgs a, int P) {
     constexpr int T = 32 / F < 8 ? 32 / F : 8;   // slots a warp scores together
@@ -113,14 +122,20 @@ __global__ void __launch_bounds__(kThreads, 2) k_score_shared(const LookupArgs a
     chain_wait();
     chain_release();
     const ClockScope stamps(a.clock ? a.clock + 2 * (SMTM_PROF_SCORE + a.layer) : nullptr);
-    // This cluster's frames: number group * F ... of those still in.  Active = not exited at an earlier layer (an exit at
-    // this very layer is a decision of this launch), so every CTA gets the same list whenever it looks.
+    // This cluster's frames.
     const int k = a.k[0];
-    for (int j = tid; j < a.k_max; j += kThreads) s_ids[j] = a.members[j];  // in flight with the exit layers
-    if (tid < F) s_frames[tid] = -1;
-    if (a.fresh) {
-        if (tid < F && group * F + tid < a.B) s_frames[tid] = group * F + tid;
+    for (int j = tid; j < a.k_max; j += kThreads) s_ids[j] = a.members[j];  // in flight with the exit flags
+    if (!a.pending) {
+        if (warp == 0) {
+            const int b = group * F + lane;
+            const bool in = lane < F && b < a.B && (a.fresh || !a.done[min(b, a.B - 1)]);
+            const unsigned m = __ballot_sync(kFull, in);
+            if (lane < F) s_frames[lane] = -1;
+            __syncwarp();
+            if (in) s_frames[__popc(m & ((1u << lane) - 1u))] = b;
+        }
     } else {
+        if (tid < F) s_frames[tid] = -1;
         constexpr int kPer = 4;
         __syncthreads();
         int before = 0;
@@ -128,10 +143,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_score_shared(const LookupArgs a
             int act[kPer], mine = 0;
 #pragma unroll
             for (int i = 0; i < kPer; ++i)
-                act[i] = *reinterpret_cast<const volatile int32_t*>(a.exit_layer + min(t0 + tid * kPer + i, a.B - 1));
+                act[i] = a.done[min(t0 + tid * kPer + i, a.B - 1)];
 #pragma unroll
             for (int i = 0; i < kPer; ++i) {
-                act[i] = (t0 + tid * kPer + i < a.B && (act[i] == 0 || act[i] == a.layer + 1)) ? 1 : 0;
+                act[i] = (t0 + tid * kPer + i < a.B && act[i] == 0) ? 1 : 0;
                 mine += act[i];
             }
             int cnt;
@@ -268,6 +283,21 @@ __global__ void __launch_bounds__(kThreads, 2) k_score_shared(const LookupArgs a
         if (a.sep) ts = block_top2_keys(c1, c2, s_keys);
         if (tid == 0) decide_from_top2(a, b, ta, ts);
     }
+}
+
+// Turns the exits that a lookup has left pending (see decide_core) into exit flags, exit layers and labels.  One trip to memory
+// after the lookup (512 streams, a step 48.7 -> 49.5 us; in stream order, without the early start, 49.7).
+constexpr int kSettleThreads = 128;
+__global__ void __launch_bounds__(kSettleThreads) k_settle_exits(const LookupArgs a) {
+    chain_wait();
+    chain_release();
+    const int b = blockIdx.x * kSettleThreads + threadIdx.x;
+    if (b >= a.B) return;
+    const int gone = a.done[b], left = a.exit_layer[b];
+    if (gone || left >= 0) return;
+    a.done[b] = 1;
+    a.exit_layer[b] = a.layer + 1;
+    a.pred[b] = -1 - left;
 }
 
 // Finishing kernel of the tensor-core path: one CTA per frame turns the frame's row of dot products into
@@ -425,6 +455,7 @@ cudaError_t launch_wait_selftest(int* status, cudaStream_t st, int64_t* launches
 
 cudaError_t lookup_setup() {
     cudaError_t e = allow_max_dynamic_smem(k_score_exit<4>);
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_settle_exits);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_score_exit<5>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_score_shared<1>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_score_shared<2>);
@@ -458,6 +489,11 @@ cudaError_t launch_finish_dense(const LookupArgs& a, const DenseDots& dots, bool
     return launch_chained(kernel, a.B, kFinishThreads, smem, st, a, dots);
 }
 
+cudaError_t launch_settle_exits(const LookupArgs& a, cudaStream_t st, int64_t* launches) {
+    ++*launches;
+    return launch_chained(k_settle_exits, (a.B + kSettleThreads - 1) / kSettleThreads, kSettleThreads, 0, st, a);
+}
+
 // Frames to a cluster of k_score_shared, or 0 where a CTA per frame scores them; *ctas: CTAs of a cluster.
 static int shared_frames(const LookupArgs& a, int sm_count, int* ctas) {
     if (a.S != 1 || a.k_max <= kFusedMaxK || (a.D & 3) || (long long)a.k_max * std::max(a.D, 64) < kShareWork) return 0;
@@ -478,9 +514,14 @@ cudaError_t launch_score_exit(const LookupArgs& a, cudaStream_t st, int sm_count
     if (const int F = shared_frames(a, sm_count, &P)) {
         const auto kernel = F == 1 ? k_score_shared<1> : F == 2 ? k_score_shared<2> : F == 4 ? k_score_shared<4> : k_score_shared<8>;
         const size_t smem = share_smem(F, P, a.D, a.k_max);
+        const int ctas = (a.B + F - 1) / F * P;
+        LookupArgs s = a;
+        const long long work = (long long)F * ((a.k_max + P - 1) / P) * a.D;
+        s.pending = !a.fresh && F > 1 && (4 * ctas > 9 * sm_count || work > (P < kShareMost ? kShareOwnWorkCrowd : kShareOwnWork));
         ++*launches;
-        if (in_order) return launch_ordered_cluster(kernel, (a.B + F - 1) / F * P, kThreads, smem, P, st, a, P);
-        return launch_chained_cluster(kernel, (a.B + F - 1) / F * P, kThreads, smem, P, st, a, P);
+        const cudaError_t e = in_order ? launch_ordered_cluster(kernel, ctas, kThreads, smem, P, st, s, P)
+                                       : launch_chained_cluster(kernel, ctas, kThreads, smem, P, st, s, P);
+        return e == cudaSuccess && s.pending ? launch_settle_exits(s, st, launches) : e;
     }
     const auto rounds = [&](int ctas) { return (a.B + ctas * sm_count - 1) / (ctas * sm_count); };
     const auto kernel = rounds(5) < rounds(4) ? k_score_exit<5> : k_score_exit<4>;

@@ -134,7 +134,10 @@ __device__ __forceinline__ void decide_frame(const LookupArgs& a, int b, const f
 
 // Lane-0 part of the decision without the global counters: Eq. 4 / Eq. 2 from the two best
 // cumulative (ta) and single-layer (ts) similarities, the exit rule in fp32 and the frame's
-// outputs.  Returns bit 0 = the frame exits, bit 1 = its AC lies within 1e-4 of the threshold.
+// outputs.  a.pending: kernels whose CTAs list the frames still in for themselves, at different times, go by the exit flags as
+// they were before the launch, so a decision must not change them while the launch runs.  An exit is then left in
+// exit_layer as -1 - class (0 for every other frame that was in), and k_settle_exits writes what it means.
+// Returns bit 0 = the frame exits, bit 1 = its AC lies within 1e-4 of the threshold.
 __device__ __forceinline__ int decide_core(const LookupArgs& a, int b, const Top2& ta, const Top2& ts) {
     float ac = 0.f, sep = 0.f;
     bool leave = false;
@@ -149,7 +152,9 @@ __device__ __forceinline__ int decide_core(const LookupArgs& a, int b, const Top
         a.top[2 * b] = ta.id1;
         a.top[2 * b + 1] = ta.id2;
     }
-    if (leave) {
+    if (leave && a.pending) {
+        a.exit_layer[b] = -1 - ta.id1;
+    } else if (leave) {
         a.done[b] = 1;
         a.exit_layer[b] = a.layer + 1;
         a.pred[b] = ta.id1;
