@@ -70,3 +70,23 @@ def test_scoring_of_large_fast_memories_that_all_frames_share(w, split):
     smtm.smtm_cache_destroy(cache)
     rep = run_workload(w)
     assert rep.frames == w.B * w.T and rep.routes == [0, 0, w.L * w.T, 0, 0]
+
+
+# maps of one pixel and equal channels, against centres with a single entry: a similarity is off by the rounding of the squared
+# length, of its root, of one product and of the division.  Each is at most 2^-24 and 3.5e-8 in the mean square; a square root
+# halves what the sum is off by, and a sum of D / 512 terms to a lane after sixteen in a tree is off by some 1.3e-7 (in fp32 on
+# the CPU; a lane that adds D / 32 terms one by one is off by 4.7e-7 and 1.9e-6)
+@pytest.mark.parametrize("D", [2048, 8192])
+def test_lengths_of_long_vectors_in_nhwc_lookups(D):
+    B, k = 300, 4
+    cents = np.zeros((k, D), np.float32)
+    cents[np.arange(k), np.arange(k) * 7] = 1.0
+    cache = smtm.smtm_cache_create(k, [D], [0.8], [cents], None, k_init=k, k_min=k, k_max=k, max_batch=B)
+    batch = smtm.Batch(cache, B)
+    x = torch.linspace(0.3, 1.7, B, device="cuda").half()[:, None, None, None].expand(B, 1, 1, D).contiguous()
+    fmap = smtm.Fmap(x, si.F16, si.NHWC, B, D, 1, 1)
+    assert [g.kernel for g in launches(lambda: smtm.smtm_lookup_exit_begin(cache, 0, fmap, batch))] == ["k_lookup_nhwc"]
+    smtm.smtm_lookup_exit_begin(cache, 0, fmap, batch)
+    off = batch.sa.double().cpu() * D ** 0.5 - 1.0
+    smtm.smtm_cache_destroy(cache)
+    assert float(off.square().mean().sqrt()) <= 1.2e-7
