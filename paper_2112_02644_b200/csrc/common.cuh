@@ -206,6 +206,14 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_
     }
 }
 
+// The same for a barrier that counts what the peers store into this CTA's shared memory (peer_store_counted).  Whoever gives up
+// stays for a second wait: what comes late should not find the CTA gone.  False also when it was complete by then.
+__device__ __forceinline__ bool mbar_wait_peers(uint64_t* bar, uint32_t parity, int* status) {
+    if (mbar_wait_cluster_bounded(bar, parity, status)) return true;
+    (void)mbar_wait_cluster_bounded(bar, parity, status);
+    return false;
+}
+
 // All threads of all CTAs of the cluster.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }  // (nothing written before has to be seen)

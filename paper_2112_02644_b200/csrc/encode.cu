@@ -1236,6 +1236,10 @@ __device__ __forceinline__ void fetch_centres(const LookupArgs& a, const FrameSl
     }
 }
 
+// An entry of the semantic vector whose pixels did not arrive before the wait for them gave up (which the status word records):
+// it makes every similarity of the frame a NaN, and a NaN exceeds no threshold, so that nothing is decided from it.
+constexpr float kNeverArrived = __builtin_nanf("");
+
 // A part's value for the CTA that decides: counted on its barrier, or (bar == 0, a cluster of one) a plain store.
 __device__ __forceinline__ void deliver(uint32_t addr, float v, uint32_t bar) {
     if (bar) peer_store_counted(addr, v, bar);
@@ -1390,8 +1394,11 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FramePa
     float clen[2] = {0.f, 0.f}, sa_old[2] = {0.f, 0.f};
     if (decides) fetch_lengths(a, b, slots, clen, sa_old);
     if (bytes) {
-        if (!mbar_wait_bounded(&landed[warp], 0, p.status)) mbar_wait_bounded(&landed[warp], 0, p.status);  // (let the copy land before leaving)
-        R::run(stage, 0, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, sv_s + w_c0, p.inv_hw, p);
+        // (a second wait: let the copy land before leaving)
+        if (mbar_wait_bounded(&landed[warp], 0, p.status) || mbar_wait_bounded(&landed[warp], 0, p.status))
+            R::run(stage, 0, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, sv_s + w_c0, p.inv_hw, p);
+        else
+            for (int c = lane; c < w_nch; c += kWarp) sv_s[w_c0 + c] = kNeverArrived;
     }
     __syncthreads();
     if (P > 1) cluster_wait();
@@ -1400,7 +1407,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FramePa
     if (warp == kFrameWarps - 1) slice_norm(v4, n4, row, bar);
     score_slots(a, slots, lg, c0, n4, v4, row, bar, cen);
     if (P == 1) __syncthreads();
-    if (decides && (P == 1 || mbar_wait_cluster_bounded(&delivered, 0, p.status)))  // every part has been delivered
+    if (decides && (P == 1 || mbar_wait_peers(&delivered, 0, p.status)))  // every part has been delivered
         decide_parts(a, b, slots, rx, P, clen, sa_old);
 }
 
@@ -1542,7 +1549,7 @@ __global__ void __launch_bounds__(kFrameThreads, kLoads == 2 ? 8 : kLoads == 4 ?
     if (threadIdx.x == 0 && c1 > c0) mbar_expect_tx(&summed, uint32_t(P) * uint32_t(c1 - c0) * 4u);
     column_sums<E, kFrameThreads, kLoads>(frame, C, px0, px1, psum + P * slice, [] { cluster_wait(); },
                                           [&](int c, float s) { send_column(psum, &summed, c, slice, rank, s); });
-    if (c1 <= c0 || !mbar_wait_cluster_bounded(&summed, 0, status)) return;
+    if (c1 <= c0 || !mbar_wait_peers(&summed, 0, status)) return;
     for (int c = c0 + threadIdx.x; c < c1; c += kFrameThreads) {
         float s = 0.f;
         for (int r = 0; r < P; ++r) s += psum[r * slice + (c - c0)];
@@ -1587,20 +1594,20 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame_nhwc(const Fr
     fetch_centres(a, slots, 0, lg, c0, 0, n4, cen);  // in flight with the exchange
     float clen[2] = {0.f, 0.f}, sa_old[2] = {0.f, 0.f};
     if (decides) fetch_lengths(a, b, slots, clen, sa_old);
-    if (nch > 0) mbar_wait_cluster_bounded(&summed, 0, a.status);
+    const bool complete = nch <= 0 || mbar_wait_peers(&summed, 0, a.status);
     for (int c = threadIdx.x; c < nch; c += kFrameThreads) {
         float s = 0.f;
         for (int r = 0; r < P; ++r) s += psum[r * f.slice + c];
-        s *= f.inv_hw;
+        s = complete ? s * f.inv_hw : kNeverArrived;
         sv_s[c] = s;
-        f.sv[(long long)b * f.C + c0 + c] = s;
+        if (complete) f.sv[(long long)b * f.C + c0 + c] = s;
     }
     __syncthreads();
     const uint32_t row = peer_smem(rx + rank * kRxRow, 0), bar = peer_smem(&delivered, 0);
     const float4* v4 = reinterpret_cast<const float4*>(sv_s);
     if (warp == kFrameWarps - 1) slice_norm(v4, n4, row, bar);
     score_slots(a, slots, lg, c0, n4, v4, row, bar, cen);
-    if (decides && mbar_wait_cluster_bounded(&delivered, 0, a.status))  // every part has been delivered
+    if (decides && mbar_wait_peers(&delivered, 0, a.status))  // every part has been delivered
         decide_parts(a, b, slots, rx, P, clen, sa_old);
 }
 

@@ -35,3 +35,15 @@ def test_a_peer_is_known_to_have_started_before_its_shared_memory_is_written():
             checked.add(name.group(1))
     assert checked >= {"k_lookup_nchw", "k_lookup_sparse", "k_lookup_frame", "k_lookup_frame_nhwc", "k_encode_nhwc", "k_score_shared",
                        "tables_of_lone_stream"}
+
+
+def test_a_wait_that_gives_up_is_heeded():
+    # no vector and no decision is made of what has not arrived, and a CTA that peers store into (counted on its barrier) stays
+    # for a second wait
+    for f, text in sources().items():
+        if f != "lookup.cu":   # (its self-test of the waits has nothing to make of the result)
+            # ((void), and the ring's copies that are left to land: the CTA only stays)
+            assert not re.findall(r"(?<!\(void)[;{})]\s*mbar_wait_\w+\(&(?!full\[s\])\w+[^;]*", text), f
+    encode = sources()["encode.cu"]
+    for bar in ("delivered", "summed"):
+        assert set(re.findall(r"(\w+)\(&%s, 0, [\w.]*status\)" % bar, encode)) == {"mbar_wait_peers"}
