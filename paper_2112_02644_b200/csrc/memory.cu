@@ -89,7 +89,7 @@ constexpr int kItemBlocksMax = 16;
 // Column blocks for a pair with `rows` frames at a layer whose vector has D entries: a CTA of the apply kernel
 // should not load more than about eight 16-byte pieces per thread.  A power of two, at most 16, and no block
 // narrower than 32 columns; vectors that are not a whole number of 16-byte pieces are never cut.
-__device__ __forceinline__ int item_blocks(int rows, int D) {
+__host__ __device__ __forceinline__ int item_blocks(int rows, int D) {
     if (D & 3) return 1;
     const int D4 = D >> 2;
     const long long want = ((long long)rows * D4 + 8 * kApplyThreads - 1) / (8 * kApplyThreads);
@@ -1177,6 +1177,9 @@ __global__ void __launch_bounds__(kApplyThreads, 8) k_update_apply(const UpdateA
 // makes what it needs of it by itself: CTA (layer, frame) fetches the state of all frames (PER consecutive ones a thread),
 // leaves when its own frame has no label or stopped before the layer, and else counts and lists the frames of its frame's
 // pair in ascending index.  The pair's column blocks are dealt to the CTAs of its first frames, in order; the others leave.
+// A frame of a vector that is worth several blocks by itself (more than 4096 channels) has that many CTAs, and as many again
+// for the blocks that a few frames together are rounded up to, while they are at most two to an SM: one frame of 65536
+// channels 98 us with a CTA, 17 by two launches, 11 so, three frames of one class of 16384 channels 17.1, 7.5 and 5.9.
 // No CTA waits for another, and the sums are those of the two launches.  What bounds it: trips to memory (three here, five
 // and a launch there), and with many frames the state that every CTA fetches, so the two launches stay beyond the lines
 // below.  Update with refresh, 200 classes, by two launches and by one: 16 frames in one layer of 256 channels 6.9 and 5.1
@@ -1186,9 +1189,9 @@ __global__ void __launch_bounds__(kApplyThreads, 8) k_update_apply(const UpdateA
 constexpr int kDirectFrames = 512;
 constexpr int kDirectCtas = 9, kDirectCtasSmall = 16;  // CTAs per SM at most; the second with a frame per thread
 
-template <int PER>
+template <int PER, bool kLong>
 __global__ void __launch_bounds__(kApplyThreads, 6) k_update_direct(const UpdateArgs a, const ResizeArgs rz, int do_resize,
-                                                                     int table_ctas) {
+                                                                     int table_ctas, int parts) {
     static_assert(PER * kApplyThreads <= kCenTile, "a pair's frames fit one listing");
     extern __shared__ __align__(16) unsigned long long s_dyn[];
     __shared__ int s_list[kCenTile];
@@ -1202,7 +1205,12 @@ __global__ void __launch_bounds__(kApplyThreads, 6) k_update_direct(const Update
         return;
     }
     const int tid = threadIdx.x;
-    const int at = int(blockIdx.x) - table_ctas, row = at / a.B, b = at - row * a.B;
+    int at = int(blockIdx.x) - table_ctas, part = 0;
+    if (kLong) {  // parts: CTAs per frame and layer
+        part = at % parts;
+        at /= parts;
+    }
+    const int row = at / a.B, b = at - row * a.B;
     const int l0 = a.warm_layer >= 0 ? a.warm_layer : row;
     if (row >= (a.warm_layer >= 0 ? 1 : a.L)) return;  // (the grid is whole clusters)
     if (a.clock && tid == 0) atomicMax(a.clock + 2 * SMTM_PROF_PLAN, ~device_clock_ns());  // (ends where the centres begin)
@@ -1232,9 +1240,9 @@ __global__ void __launch_bounds__(kApplyThreads, 6) k_update_direct(const Update
             s_list[pos++] = tid * PER + i;
         }
     __syncthreads();
-    const int place = s_scan[32];
+    const int place = kLong ? s_scan[32] * parts + part : s_scan[32];
     int nblk = item_blocks(cnt, a.dims[l0]);
-    while (nblk > cnt) nblk >>= 1;  // (a block needs a frame whose CTA folds it)
+    while (nblk > (kLong ? cnt * parts : cnt)) nblk >>= 1;  // (a block needs a CTA that folds it)
     if (place >= nblk) return;
     const ClockScope stamps(a.clock ? a.clock + 2 * SMTM_PROF_CENTERS : nullptr);
     centre_item(a, l0, cls, place, nblk, [&](int) { return cnt; }, s_list, s_acc);
@@ -1260,10 +1268,10 @@ cudaError_t memory_setup() {
     cudaError_t e = allow_max_dynamic_smem(k_update_apply);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_resize);
     // the update's kernels share SMs with the next step's pooling kernel on the pipelined route
-#define SMTM_OPT_IN(PER)                                                             \
-    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_update_direct<PER>);          \
-    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_update_direct<PER>);
-    SMTM_OPT_IN(1) SMTM_OPT_IN(4)
+#define SMTM_OPT_IN(...)                                                                     \
+    if (e == cudaSuccess) e = allow_max_dynamic_smem(k_update_direct<__VA_ARGS__>);          \
+    if (e == cudaSuccess) e = prefer_max_smem_carveout(k_update_direct<__VA_ARGS__>);
+    SMTM_OPT_IN(1, false) SMTM_OPT_IN(4, false) SMTM_OPT_IN(1, true) SMTM_OPT_IN(4, true)
 #undef SMTM_OPT_IN
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_update_apply);
     if (e == cudaSuccess) e = prefer_max_smem_carveout(k_update_plan_one);
@@ -1296,14 +1304,20 @@ cudaError_t launch_update(const UpdateArgs& a, const ResizeArgs* rz, bool beside
     const size_t smem = lone ? lone_smem(a.n, rz ? rz->k_max : 0) : tables ? tables_smem(a.n, rz ? rz->k_max : 0, refresh_here) : 0;
     const ResizeArgs rza = rz ? *rz : ResizeArgs{};
     const int layers = a.warm_layer >= 0 ? 1 : a.L;
-    const bool direct = a.B <= kDirectFrames && (long long)table_ctas + (long long)a.B * layers <=
+    int parts = 1;  // CTAs of k_update_direct per frame and layer
+    for (int l = 0; l < a.L; ++l)
+        if (a.warm_layer < 0 || l == a.warm_layer) parts = std::max(parts, item_blocks(1, a.dims[l]));
+    if (parts > 1) parts = std::min(2 * parts, kItemBlocksMax);
+    while (parts > 1 && (long long)a.B * layers * parts > 2LL * sm_count) parts /= 2;
+    const bool direct = a.B <= kDirectFrames && (long long)table_ctas + (long long)a.B * layers * parts <=
                         (long long)(a.B <= kApplyThreads ? kDirectCtasSmall : kDirectCtas) * sm_count;
     ++*launches;
     if (direct) {
-        const auto kernel = a.B <= kApplyThreads ? k_update_direct<1> : k_update_direct<4>;
-        const int ctas = (table_ctas + a.B * layers + team - 1) / team * team;
-        e = beside_pooling ? launch_ordered_cluster(kernel, ctas, kApplyThreads, smem, team, st, a, rza, refresh_here ? 1 : 0, table_ctas)
-                           : launch_chained_cluster(kernel, ctas, kApplyThreads, smem, team, st, a, rza, refresh_here ? 1 : 0, table_ctas);
+        const auto kernel = a.B <= kApplyThreads ? (parts > 1 ? k_update_direct<1, true> : k_update_direct<1, false>)
+                                                 : (parts > 1 ? k_update_direct<4, true> : k_update_direct<4, false>);
+        const int ctas = (table_ctas + a.B * layers * parts + team - 1) / team * team;
+        e = beside_pooling ? launch_ordered_cluster(kernel, ctas, kApplyThreads, smem, team, st, a, rza, refresh_here ? 1 : 0, table_ctas, parts)
+                           : launch_chained_cluster(kernel, ctas, kApplyThreads, smem, team, st, a, rza, refresh_here ? 1 : 0, table_ctas, parts);
         if (e != cudaSuccess || !refresh_apart) return e;
         return launch_resize(*rz, st, launches);
     }

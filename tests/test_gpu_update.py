@@ -88,3 +88,20 @@ def test_frames_of_no_stream_beside_an_only_stream():
     sid = np.zeros(w.B, np.int32)
     sid[[0, 7, 150, 299]] = 1, -2, 5, 9
     _run(w, sid)
+
+
+# vectors of more than 4096 channels have several CTAs per frame in the one launch, fewer where the frames are many: one block, a
+# block more than frames, as many blocks as there are, and (by the frames) one CTA each again; every frame of one class, and a
+# layer of short vectors beside the long ones
+@pytest.mark.parametrize("B,stages,parts,zipf", [
+    (1, ((4100, 1, 1),), 4, 0.0), (3, ((4096, 1, 1),), 1, 0.0), (3, ((8192, 1, 1), (36, 2, 2)), 4, 9.0),
+    (2, ((32772, 1, 1),), 16, 9.0), (40, ((8200, 1, 1),), 4, 0.5), (100, ((16388, 1, 1),), 2, 9.0), (150, ((4104, 1, 1),), 1, 9.0)])
+def test_updates_of_long_vectors(B, stages, parts, zipf):
+    w = workload("long", B, 6, stages=stages, k_init=3, k_max=6, zipf_s=zipf, tau=9.0)
+    cache = smtm.smtm_cache_create(w.n, w.dims, [0.8] * w.L, [np.ones((w.n, d), np.float32) for d in w.dims], None, k_init=3,
+                                   k_min=3, k_max=6, window_W=2, max_batch=B)
+    batch = smtm.Batch(cache, B)
+    got = launches(lambda: smtm.smtm_cache_update_resize(cache, batch, None))
+    smtm.smtm_cache_destroy(cache)
+    assert [(g.kernel, g.grid) for g in got] == [("k_update_direct", 1 + B * w.L * parts)]
+    assert run_workload(w).frames == B * w.T
