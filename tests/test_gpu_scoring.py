@@ -25,14 +25,37 @@ def test_clusters_of_later_lookups_of_small_frames(B, begin, cluster):
     assert [(g.kernel, g.cluster) for g in got] == [("k_lookup_frame", cluster)]
 
 
-# batches large enough for the clusters that take a frame's chunks in halves: a last chunk shorter than half a chunk, channels
-# that are no whole vectors, chunks of one unit of channels
+# later layers of large batches on the pipelined route: chunks in halves with a last one shorter than half a chunk, and of four
+# channels; three whole chunks; channels that are no run of whole vectors (not pipelined); nine chunks (pooled and scored apart)
 @pytest.mark.parametrize("dt,stages", [
     (si.BF16, ((64, 9, 9), (840, 8, 8))), (si.F16, ((32, 8, 8), (296, 9, 11), (1100, 5, 5))), (si.F32, ((16, 8, 8), (16, 40, 40))),
     (si.F32, ((64, 7, 7), (1028, 7, 7)))], ids=lambda v: str(v) if isinstance(v, tuple) else None)
 def test_later_layers_of_large_batches(dt, stages):
     ready_steps(si.Workload("halves", dt, si.NCHW, B=450, stages=stages, n=40, k_init=8, k_min=4, k_max=12, S=450, T=3, tau=0.75,
                             sigma=1.0, zipf_s=0.5, repeat_p=0.8, seed=97))
+
+
+# ... and the clusters that take chunks in halves, by the reducer: channels of odd widths from 128 bytes on and below (the halves
+# meet on a 16-byte boundary), units of channels of 7x7 and 14x14 maps, whole vectors, a last chunk of one run of channels
+@pytest.mark.parametrize("dt,stages,reducers", [
+    (si.F16, ((64, 8, 8), (520, 9, 11), (2048, 5, 5)), ["TeamVectorsINS_3F16ELb1E", "LanePerChannelINS_3F16E"]),
+    (si.BF16, ((64, 8, 8), (516, 9, 10), (2056, 5, 5)), ["TeamVectorsINS_4BF16ELb1E", "LanePerChannelINS_4BF16E"]),
+    (si.F32, ((64, 7, 7), (1024, 7, 7), (640, 6, 6)), ["UnitPerLaneINS_3F32ELi49E", "TeamVectorsINS_3F32ELb0E"]),
+    (si.BF16, ((64, 8, 8), (320, 14, 14), (1288, 7, 7)), ["UnitPerLaneINS_4BF16ELi196E", "UnitPerLaneINS_4BF16ELi49E"]),
+], ids=lambda v: str(v) if isinstance(v, tuple) else None)
+def test_chunks_in_halves(dt, stages, reducers):
+    w = si.Workload("in_halves", dt, si.NCHW, B=450, stages=stages, n=40, k_init=8, k_min=4, k_max=12, S=450, T=3, tau=0.75,
+                    sigma=1.0, zipf_s=0.5, repeat_p=0.8, seed=97)
+    dtype = {si.F32: torch.float32, si.F16: torch.float16, si.BF16: torch.bfloat16}[dt]
+    cache = smtm.smtm_cache_create(w.n, w.dims, [0.8] * w.L, [np.ones((w.n, d), np.float32) for d in w.dims], None, n_streams=w.S,
+                                   k_init=8, k_min=4, k_max=12, max_batch=w.B, flags=smtm.FLAG_MAPS_READY)
+    batch = smtm.Batch(cache, w.B, stream_id=si.stream_ids(w))
+    for l, reducer in enumerate(reducers, 1):
+        x = torch.zeros(si.shape4(w, l), dtype=dtype, device="cuda")
+        got = launches(lambda: smtm.smtm_lookup_exit(cache, l, smtm.Fmap(x, dt, w.layout, *si.shape4(w, l)), batch))
+        assert got[0].kernel == "k_lookup_sparse" and reducer in got[0].variant and "Lb1EEEvNS" in got[0].variant, got[0]
+    smtm.smtm_cache_destroy(cache)
+    ready_steps(w)
 
 
 # fast memories of more than 64 slots that all frames share: eight, four, two or one frame to a cluster, slots in whole and
