@@ -38,7 +38,7 @@ struct smtm_cache {
     unsigned long long mark_capture[2]; // the stream capture each was recorded in (0 = none)
     bool mark_valid[2];
     int mark_next;                      // which of the two the next first lookup records
-    int32_t* d_jobs;             // scratch of the update: [4] counters, [L][n] (layer, class) pairs to fold, [16][L][n] work items
+    int32_t* d_items;            // scratch of the update: [4] counters, [16][L][n] work items
     float* d_norm_part;          // scratch of the update: [L][n][16] squared lengths of the blocks of a centre folded by several CTAs
     int32_t* d_ticket;           // scratch of the update: [L][n] tickets of those CTAs (zero between updates)
     unsigned long long* d_epoch; // [2] device: update calls so far, and the plan kernel's ticket
@@ -128,7 +128,7 @@ void free_all(smtm_cache* c) {
     if (c->ev_pool) cudaEventDestroy(c->ev_pool);
     for (cudaEvent_t e : c->ev_mark)
         if (e) cudaEventDestroy(e);
-    cudaFree(c->d_jobs);
+    cudaFree(c->d_items);
     cudaFree(c->d_norm_part);
     cudaFree(c->d_ticket);
     cudaFree(c->hb.d_sa);
@@ -414,9 +414,8 @@ smtm_status_t update_impl(smtm_cache* c, const smtm_batch_t* b, const int32_t* d
     a.warm_layer = -1;
     a.plan.frame_code = c->d_plan;
     a.plan.class_tag = c->d_tags;
-    a.plan.job_count = c->d_jobs;
-    a.plan.jobs = c->d_jobs + 4;
-    a.plan.items = c->d_jobs + 4 + size_t(c->L) * c->n;
+    a.plan.item_count = c->d_items;
+    a.plan.items = c->d_items + 4;
     a.norm_part = c->d_norm_part;
     a.ticket = c->d_ticket;
     a.plan.epoch = c->d_epoch;
@@ -562,7 +561,7 @@ smtm_status_t smtm_cache_create(const smtm_config_t* cfg, const float* const* h_
             ok = cudaMalloc(&c->d_cen_split[l], dense_centers_split_bytes(n, c->dims[l])) == cudaSuccess;
     }
     ok = ok && dev_alloc(&c->d_tags, size_t(c->L) * n) == cudaSuccess;
-    ok = ok && dev_alloc(&c->d_jobs, 4 + 17 * size_t(c->L) * n) == cudaSuccess;
+    ok = ok && dev_alloc(&c->d_items, 4 + 16 * size_t(c->L) * n) == cudaSuccess;
     ok = ok && dev_alloc(&c->d_norm_part, 16 * size_t(c->L) * n) == cudaSuccess;
     ok = ok && dev_alloc(&c->d_ticket, size_t(c->L) * n) == cudaSuccess;
     ok = ok && dev_alloc(&c->d_epoch, 2) == cudaSuccess;
@@ -600,7 +599,7 @@ smtm_status_t smtm_cache_create(const smtm_config_t* cfg, const float* const* h_
     if (e == cudaSuccess) e = cudaMemset(c->d_counters, 0, SMTM_CTR_COUNT * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_tags, 0, size_t(c->L) * n * sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemset(c->d_jobs, 0, (4 + 17 * size_t(c->L) * n) * sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMemset(c->d_items, 0, (4 + 16 * size_t(c->L) * n) * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(c->d_epoch, 0, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(c->d_ticket, 0, size_t(c->L) * n * sizeof(int32_t));
     if (e == cudaSuccess)
@@ -692,9 +691,8 @@ smtm_status_t smtm_cache_warmup(smtm_cache_t* c, int32_t layer, const smtm_fmap_
     a.warm_layer = layer;
     a.plan.frame_code = c->d_plan;
     a.plan.class_tag = c->d_tags;
-    a.plan.job_count = c->d_jobs;
-    a.plan.jobs = c->d_jobs + 4;
-    a.plan.items = c->d_jobs + 4 + size_t(c->L) * c->n;
+    a.plan.item_count = c->d_items;
+    a.plan.items = c->d_items + 4;
     a.norm_part = c->d_norm_part;
     a.ticket = c->d_ticket;
     a.plan.epoch = c->d_epoch;

@@ -222,11 +222,6 @@ __device__ __forceinline__ void cluster_sync_all() {
     cluster_arrive();
     cluster_wait();
 }
-__device__ __forceinline__ float peer_load(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
 
 // ---- element widening -----------------------------------------------------------------
 

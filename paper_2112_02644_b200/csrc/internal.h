@@ -227,9 +227,8 @@ cudaError_t launch_center_norms(const float* centers, int n, int D, float* cnorm
 struct UpdatePlan {
     int32_t* frame_code;             // [max_batch] per frame: final label | stop layer (the paper's l) << 16, or -1 without a label
     unsigned long long* class_tag;   // [L][n] number of the last update call that touched (layer, class)
-    int32_t* job_count;              // [0], [1]: (layer, class) pairs listed by this call ([number & 1]) and, zeroed, for the
-                                     // next; [2]: this call's count, published by the plan kernel's last CTA; [3]: its items
-    int32_t* jobs;                   // [L][n] the (layer << 16 | class) pairs Eq. 7 touches in this call, in no particular order
+    int32_t* item_count;             // [0], [1]: items listed by this call ([number & 1]) and, zeroed, for the next (the plan by
+                                     // many CTAs); [2]: this call's count, published for the apply kernel
     int32_t* items;                  // [16][L][n] work items of the apply kernel: a pair, or one of the column blocks a heavy pair is cut into
     unsigned long long* epoch;       // [2] device: [0] number of update calls completed so far, [1] CTAs of the plan
                                      // kernel that are through (zero between calls).  The number lives on the

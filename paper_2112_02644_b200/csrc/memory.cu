@@ -78,10 +78,9 @@ __device__ __forceinline__ int frame_code_of(const UpdateArgs& a, int b, int* si
 // ---- plan -----------------------------------------------------------------------------------
 //
 // What the plan leaves for the kernels that follow: per frame its final label and stop layer packed into one
-// word (label | stop layer << 16, or -1 for a frame without a label); the list of
-// pairs (layer, class) Eq. 7 touches (`jobs`, job_count[2] of them); and the list of work items of the apply
-// kernel (`items`, job_count[3] of them): a pair whose frames are many is cut into several items, each a
-// block of the vector's columns, so that no CTA folds more than a few rows per thread.
+// word (label | stop layer << 16, or -1 for a frame without a label); and the list of work items of the apply
+// kernel (`items`, item_count[2] of them), which cover the pairs (layer, class) Eq. 7 touches: a pair whose frames are many
+// is cut into several items, each a block of the vector's columns, so that no CTA folds more than a few rows per thread.
 //   item = layer << 16 | class | block << 20 | log2(blocks) << 24      (class < 2^13, layer < 2^4, blocks <= 16)
 
 constexpr int kItemBlocksMax = 16;
@@ -115,28 +114,24 @@ __global__ void __launch_bounds__(kUpdThreads) k_update_plan(const UpdateArgs a)
         if (code >= 0) {
             const int lab = code & 0xffff;
             // Eq. 7 touches the layers up to the stop layer: the first frame to stamp (layer, class)
-            // with the call's number lists the pair as a job, and as a single item (this form of the plan
-            // does not count the frames of a pair)
+            // with the call's number lists the pair as a single item (this form of the plan does not count the
+            // frames of a pair)
             const int l_lo = a.warm_layer >= 0 ? a.warm_layer : 0;
             const int l_hi = a.warm_layer >= 0 ? a.warm_layer + 1 : code >> 16;
             for (int l = l_lo; l < l_hi; ++l)
                 if (atomicExch(a.plan.class_tag + (size_t)l * a.n + lab, epoch) != epoch) {
-                    const int at = atomicAdd(a.plan.job_count + (epoch & 1), 1);
-                    a.plan.jobs[at] = (l << 16) | lab;
-                    a.plan.items[at] = (l << 16) | lab;
+                    a.plan.items[atomicAdd(a.plan.item_count + (epoch & 1), 1)] = (l << 16) | lab;
                 }
         }
     }
-    if (b == 0) a.plan.job_count[(epoch + 1) & 1] = 0;  // the next call's counter (the call before this one is over)
+    if (b == 0) a.plan.item_count[(epoch + 1) & 1] = 0;  // the next call's counter (the call before this one is over)
     // the last CTA through makes the number current for the kernels that follow and publishes the
-    // number of jobs (every CTA's appends are complete and visible before its ticket)
+    // number of items (every CTA's appends are complete and visible before its ticket)
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(a.plan.epoch + 1, 1ull) == gridDim.x - 1) {
         __threadfence();
-        const int jobs = *reinterpret_cast<volatile int32_t*>(a.plan.job_count + (epoch & 1));
-        a.plan.job_count[2] = jobs;
-        a.plan.job_count[3] = jobs;
+        a.plan.item_count[2] = *reinterpret_cast<volatile int32_t*>(a.plan.item_count + (epoch & 1));
         a.plan.epoch[1] = 0;
         a.plan.epoch[0] = epoch;
     }
@@ -153,13 +148,13 @@ constexpr int kPlanCountMax = 8192;   // pairs that get a counter each
 
 __global__ void __launch_bounds__(kPlanOneThreads) k_update_plan_one(const UpdateArgs a) {
     extern __shared__ int s_plan[];  // counters [pairs] or bitmap words
-    __shared__ int s_jobs, s_items;
+    __shared__ int s_items;
     const int tid = threadIdx.x;
     const int pairs = a.L * a.n;
     const bool counted = pairs <= kPlanCountMax;
     const int words = counted ? pairs : (pairs + 31) / 32;
     for (int i = tid; i < words; i += kPlanOneThreads) s_plan[i] = 0;
-    if (tid == 0) s_jobs = s_items = 0;
+    if (tid == 0) s_items = 0;
     chain_wait();
     chain_release();
     const ClockScope stamps(a.clock ? a.clock + 2 * SMTM_PROF_PLAN : nullptr);
@@ -179,11 +174,8 @@ __global__ void __launch_bounds__(kPlanOneThreads) k_update_plan_one(const Updat
                     atomicAdd(&s_plan[pair], 1);
                 } else {
                     const unsigned int bit = 1u << (pair & 31);
-                    if (!(atomicOr(reinterpret_cast<unsigned int*>(&s_plan[pair >> 5]), bit) & bit)) {
-                        const int at = atomicAdd(&s_jobs, 1);
-                        a.plan.jobs[at] = (l << 16) | lab;
-                        a.plan.items[at] = (l << 16) | lab;
-                    }
+                    if (!(atomicOr(reinterpret_cast<unsigned int*>(&s_plan[pair >> 5]), bit) & bit))
+                        a.plan.items[atomicAdd(&s_items, 1)] = (l << 16) | lab;
                 }
             }
         }
@@ -194,17 +186,13 @@ __global__ void __launch_bounds__(kPlanOneThreads) k_update_plan_one(const Updat
             const int rows = s_plan[pair];
             if (rows == 0) continue;
             const int l = pair / a.n, code = (l << 16) | (pair - l * a.n);
-            a.plan.jobs[atomicAdd(&s_jobs, 1)] = code;
             const int nb = item_blocks(rows, a.dims[l]), lg = ilog2_pow2(nb);
             const int at = atomicAdd(&s_items, nb);
             for (int k = 0; k < nb; ++k) a.plan.items[at + k] = code | (k << 20) | (lg << 24);
         }
         __syncthreads();
     }
-    if (tid == 0) {
-        a.plan.job_count[2] = s_jobs;
-        a.plan.job_count[3] = counted ? s_items : s_jobs;
-    }
+    if (tid == 0) a.plan.item_count[2] = s_items;
 }
 
 // ---- Eq. 5 / Eq. 6 ------------------------------------------------------------------------
@@ -762,7 +750,7 @@ __device__ void tables_of_frame(const UpdateArgs& a, const ResizeArgs& rz, int g
         s_scan[32] = 0;
         s_part[31] = 0ull;
     }
-    const bool lone = g < 0;
+    const bool lone = PER == 0 && g < 0;  // (up to 1024 classes an only stream has tables_of_lone_stream)
     if (lone) g = 0;
     const int s = (a.stream_id && !lone) ? a.stream_id[g] : 0;
     if (s < 0 || s >= a.S) return;  // no such stream (the same for every thread; the plan kernel records the error)
@@ -1157,7 +1145,7 @@ __global__ void __launch_bounds__(kApplyThreads, 8) k_update_apply(const UpdateA
 #pragma unroll
     for (int i = 0; i < kCenPer; ++i) first_tile[i] = a.plan.frame_code[min(int(threadIdx.x) * kCenPer + i, a.B - 1)];
     int item = a.plan.items[min(first, kItemBlocksMax * a.L * a.n - 1)];
-    const int n_items = a.plan.job_count[3];
+    const int n_items = a.plan.item_count[2];
     if (first >= n_items) return;
     const ClockScope stamps(a.clock ? a.clock + 2 * SMTM_PROF_CENTERS : nullptr);
     for (int it = first; it < n_items; it += stride) {
