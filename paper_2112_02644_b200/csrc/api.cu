@@ -331,18 +331,14 @@ smtm_status_t lookup_impl(smtm_cache* c, int32_t layer, const smtm_fmap_t* f, co
         if (begin) return pooled_first_lookup(c, e, a, st, timing, profiled_step_begins, false);
         // a later layer: the frames still in are few; clusters of small CTAs look them up whole, or, for shapes
         // those do not serve, small CTAs pool them and small CTAs score them
+        if (launch_lookup_sparse_supported(e, a)) {
+            SMTM_CUDA(launch_lookup_sparse(e, a, c->sm_count, st, &c->launches, timing));
+            return SMTM_OK;
+        }
         if (timing) SMTM_CUDA(record_timing(timing[0], st));
-        const bool whole = launch_lookup_sparse_supported(e, a);
-        a.pending = whole ? 1 : 0;
-        if (whole)
-            SMTM_CUDA(launch_lookup_sparse(e, a, c->sm_count, st, &c->launches));
-        else
-            SMTM_CUDA(launch_pool_sparse(e, c->sm_count, st, &c->launches));
+        SMTM_CUDA(launch_pool_sparse(e, c->sm_count, st, &c->launches));
         if (timing) SMTM_CUDA(record_timing(timing[1], st));
-        if (whole)
-            SMTM_CUDA(launch_settle_exits(a, st, &c->launches));
-        else
-            SMTM_CUDA(launch_score_exit(a, st, c->sm_count, &c->launches, kPipelinedScoreThreads));
+        SMTM_CUDA(launch_score_exit(a, st, c->sm_count, &c->launches, kPipelinedScoreThreads));
         return SMTM_OK;
     }
     if (pipelined_nhwc) {

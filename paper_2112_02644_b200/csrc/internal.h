@@ -172,8 +172,9 @@ constexpr int kFusedMaxK = 64;  // fast-memory capacity the fused path supports 
 // Lookup (pooling, scoring, decision) of the frames still in at a later layer by clusters of small CTAs that fit
 // beside a streaming kernel: NCHW shapes the streaming pipeline cuts into at most 8 chunks per frame.
 bool launch_lookup_sparse_supported(const EncodeArgs& e, const LookupArgs& a);
-// (a.pending has to be set; launch_settle_exits follows.)
-cudaError_t launch_lookup_sparse(const EncodeArgs& e, const LookupArgs& a, int sm_count, cudaStream_t st, int64_t* launches);
+// timing: as for launch_lookup_fused.
+cudaError_t launch_lookup_sparse(const EncodeArgs& e, const LookupArgs& a, int sm_count, cudaStream_t st, int64_t* launches,
+                                 const cudaEvent_t* timing);
 // What the device answered when asked how many clusters of 2, 4, 8 CTAs of each variant of the fused
 // kernel it runs at once (0 = not asked yet, -1 = refused); kept per cache, i.e. per device.
 struct FusedCaps {

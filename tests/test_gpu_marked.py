@@ -22,6 +22,7 @@ READY = smtm.FLAG_MAPS_READY
 CASES = [
     (_w("frame_nchw", si.F16, si.NCHW, 100, ((64, 9, 9), (256, 4, 4)), 40, 12, 100), 0, "k_lookup_frame"),
     (_w("streamed_nchw", si.F32, si.NCHW, 300, ((1024, 7, 7), (1024, 7, 7)), 20, 4), 0, "k_lookup_nchw"),
+    (_w("streamed_few", si.BF16, si.NCHW, 13, ((256, 56, 56), (256, 56, 56)), 20, 10), 0, "k_lookup_nchw"),
     (_w("frame_nhwc", si.F16, si.NHWC, 3, ((64, 50, 50), (104, 31, 31)), 20, 6), 0, "k_lookup_frame_nhwc"),
     (_w("nhwc", si.BF16, si.NHWC, 260, ((64, 8, 8), (128, 4, 4)), 20, 6, 260), 0, "k_lookup_nhwc"),
     (_w("apart", si.F16, si.NCHW, 70, ((64, 4, 4), (36, 5, 5)), 80, 70, 70), 0, "k_score_exit"),
