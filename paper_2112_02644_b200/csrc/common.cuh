@@ -206,12 +206,21 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_
     }
 }
 
-// The same for a barrier that counts what the peers store into this CTA's shared memory (peer_store_counted).  Whoever gives up
-// stays for a second wait: what comes late should not find the CTA gone.  False also when it was complete by then.
-__device__ __forceinline__ bool mbar_wait_peers(uint64_t* bar, uint32_t parity, int* status) {
-    if (mbar_wait_cluster_bounded(bar, parity, status)) return true;
-    (void)mbar_wait_cluster_bounded(bar, parity, status);
-    return false;
+// The same for what arrives in this CTA's shared memory by itself (bulk copies; kCluster: what peers store, counted on the
+// barrier): after its limit, which is recorded, it stays for as long again, so that what comes late does not find the CTA gone.
+// False: it never came.
+template <bool kCluster>
+__device__ __forceinline__ bool mbar_wait_arrivals(uint64_t* bar, uint32_t parity, int* status) {
+    if (kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
+    const long long t0 = clock64();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 256; ++i)
+            if (kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
+        const long long waited = clock64() - t0;
+        if (waited > (1ll << 31)) set_status(status, kDevTimeout);
+        if (waited > (1ll << 32)) return false;
+    }
 }
 
 // All threads of all CTAs of the cluster.

@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(kThreadsFused, 1) k_lookup_nchw(const FusedPar
             Top2 ts{0.f, 0.f, -1, -1};
             if (a.sep) ts = warp_top2_keys(s_cur, ids, k, lane);  // only Eq. 2 (a diagnostic) needs it
             if (lane == 0) {
-                const int r = decide_core(a, b, ta, ts);
+                const int r = decide_core<true>(a, b, ta, ts);
                 s_ctr[0] += 1u;  // only this lane touches the tallies until the CTA is done
                 if (r & 2) s_ctr[1] += 1u;
                 if (r & 1) s_ctr[2] += 1u;
@@ -1170,7 +1170,7 @@ __global__ void __launch_bounds__(kLightThreads, kHalves ? 5 : 4) k_lookup_spars
             const Top2 ta = warp_top2_keys(s_acc, ids, k, lane);
             Top2 ts{0.f, 0.f, -1, -1};
             if (a.sep) ts = warp_top2_keys(s_cur, ids, k, lane);  // only Eq. 2 (a diagnostic) needs it
-            if (lane == 0) decide_from_top2(a, b, ta, ts);
+            if (lane == 0) decide_from_top2<true>(a, b, ta, ts);
         }
     }
     if (P > 1 && nu == 0) cluster_wait();
@@ -1414,8 +1414,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FramePa
     float clen[2] = {0.f, 0.f}, sa_old[2] = {0.f, 0.f};
     if (decides) fetch_lengths(a, b, slots, clen, sa_old);
     if (bytes) {
-        // (a second wait: let the copy land before leaving)
-        if (mbar_wait_bounded(&landed[warp], 0, p.status) || mbar_wait_bounded(&landed[warp], 0, p.status))
+        if (__builtin_expect(mbar_wait_arrivals<false>(&landed[warp], 0, p.status), 1))
             R::run(stage, 0, w_nch, lane, p.sv + (long long)b * p.C + c0 + w_c0, sv_s + w_c0, p.inv_hw, p);
         else
             for (int c = lane; c < w_nch; c += kWarp) sv_s[w_c0 + c] = kNeverArrived;
@@ -1427,7 +1426,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FramePa
     if (warp == kFrameWarps - 1) slice_norm(v4, n4, row, bar);
     score_slots(a, slots, lg, c0, n4, v4, row, bar, cen);
     if (P == 1) __syncthreads();
-    if (decides && (P == 1 || mbar_wait_peers(&delivered, 0, p.status)))  // every part has been delivered
+    if (decides && (P == 1 || mbar_wait_arrivals<true>(&delivered, 0, p.status)))  // every part has been delivered
         decide_parts(a, b, slots, rx, P, clen, sa_old);
 }
 
@@ -1569,7 +1568,7 @@ __global__ void __launch_bounds__(kFrameThreads, kLoads == 2 ? 8 : kLoads == 4 ?
     if (threadIdx.x == 0 && c1 > c0) mbar_expect_tx(&summed, uint32_t(P) * uint32_t(c1 - c0) * 4u);
     column_sums<E, kFrameThreads, kLoads>(frame, C, px0, px1, psum + P * slice, [] { cluster_wait(); },
                                           [&](int c, float s) { send_column(psum, &summed, c, slice, rank, s); });
-    if (c1 <= c0 || !mbar_wait_peers(&summed, 0, status)) return;
+    if (c1 <= c0 || !mbar_wait_arrivals<true>(&summed, 0, status)) return;
     for (int c = c0 + threadIdx.x; c < c1; c += kFrameThreads) {
         float s = 0.f;
         for (int r = 0; r < P; ++r) s += psum[r * slice + (c - c0)];
@@ -1614,7 +1613,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame_nhwc(const Fr
     fetch_centres(a, slots, 0, lg, c0, 0, n4, cen);  // in flight with the exchange
     float clen[2] = {0.f, 0.f}, sa_old[2] = {0.f, 0.f};
     if (decides) fetch_lengths(a, b, slots, clen, sa_old);
-    const bool complete = nch <= 0 || mbar_wait_peers(&summed, 0, a.status);
+    const bool complete = nch <= 0 || mbar_wait_arrivals<true>(&summed, 0, a.status);
     for (int c = threadIdx.x; c < nch; c += kFrameThreads) {
         float s = 0.f;
         for (int r = 0; r < P; ++r) s += psum[r * f.slice + c];
@@ -1627,7 +1626,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame_nhwc(const Fr
     const float4* v4 = reinterpret_cast<const float4*>(sv_s);
     if (warp == kFrameWarps - 1) slice_norm(v4, n4, row, bar);
     score_slots(a, slots, lg, c0, n4, v4, row, bar, cen);
-    if (decides && mbar_wait_peers(&delivered, 0, a.status))  // every part has been delivered
+    if (decides && mbar_wait_arrivals<true>(&delivered, 0, a.status))  // every part has been delivered
         decide_parts(a, b, slots, rx, P, clen, sa_old);
 }
 

@@ -125,10 +125,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_score_shared(const LookupArgs a
     // This cluster's frames.
     const int k = a.k[0];
     for (int j = tid; j < a.k_max; j += kThreads) s_ids[j] = a.members[j];  // in flight with the exit flags
-    if (!a.pending) {
+    if (a.fresh) {
+        if (tid < F) s_frames[tid] = group * F + tid < a.B ? group * F + tid : -1;
+    } else if (F == 1 || !a.pending) {
         if (warp == 0) {
             const int b = group * F + lane;
-            const bool in = lane < F && b < a.B && (a.fresh || !a.done[min(b, a.B - 1)]);
+            const bool in = lane < F && b < a.B && !a.done[min(b, a.B - 1)];
             const unsigned m = __ballot_sync(kFull, in);
             if (lane < F) s_frames[lane] = -1;
             __syncwarp();
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_score_shared(const LookupArgs a
         const Top2 ta = block_top2_keys(a1, a2, s_keys);
         Top2 ts{0.f, 0.f, -1, -1};
         if (a.sep) ts = block_top2_keys(c1, c2, s_keys);
-        if (tid == 0) decide_from_top2(a, b, ta, ts);
+        if (tid == 0) decide_from_top2<(F > 1)>(a, b, ta, ts);
     }
 }
 

@@ -43,7 +43,7 @@ def test_a_wait_that_gives_up_is_heeded():
     for f, text in sources().items():
         if f != "lookup.cu":   # (its self-test of the waits has nothing to make of the result)
             # ((void), and the ring's copies that are left to land: the CTA only stays)
-            assert not re.findall(r"(?<!\(void)[;{})]\s*mbar_wait_\w+\(&(?!full\[s\])\w+[^;]*", text), f
+            assert not re.findall(r"(?<!\(void)[;{})]\s*mbar_wait_[\w<>]+\(&(?!full\[s\])\w+[^;]*", text), f
     encode = sources()["encode.cu"]
     for bar in ("delivered", "summed"):
-        assert set(re.findall(r"(\w+)\(&%s, 0, [\w.]*status\)" % bar, encode)) == {"mbar_wait_peers"}
+        assert set(re.findall(r"([\w<>]+)\(&%s, 0, [\w.]*status\)" % bar, encode)) == {"mbar_wait_arrivals<true>"}
