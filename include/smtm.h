@@ -212,10 +212,11 @@ smtm_status_t smtm_lookup_exit_static(smtm_cache_t* cache, int32_t layer, const 
  * (saturating at 2^20), TS[label] = 0, TS of every other class + 1.  For every
  * class j and layer l0 the frames with label j and stop layer >= l0 are folded
  * into the centre in ascending b:  SC = (SC m + sum SV) / (m + q), m += q
- * (summed as four interleaved partial sums added in a fixed order).
- * Tables and centres are kept by different CTAs of one kernel, after a small
- * kernel that plans the work; everything is enqueued on `stream`.  The call's
- * bookkeeping lives on the device: a captured update may be replayed any number
+ * (summed as up to eight interleaved partial sums added in an order that the
+ * batch and the cache's sizes fix).
+ * Tables and centres are kept by different CTAs of one kernel, for large batches
+ * after a small kernel that plans the work; everything is enqueued on `stream`.
+ * The call's bookkeeping lives on the device: a captured update may be replayed any number
  * of times. */
 smtm_status_t smtm_cache_update(smtm_cache_t* cache, const smtm_batch_t* batch,
                                 const int32_t* d_fallback_label, void* stream);
@@ -321,7 +322,8 @@ smtm_status_t smtm_cache_get_launches(smtm_cache_t* cache, int64_t* h_out);
  * route has served so far.  The route is chosen from the shape and the cache's flags:
  *   SMTM_ROUTE_FUSED  pooling, Eq. 1, Eq. 3, Eq. 4 and the exit rule in one kernel
  *                     (fast memories of at most 64 entries; NCHW shapes the streaming kernel serves, and
- *                     NHWC shapes whose pixel rows are multiples of 16 bytes, of at most 8192 channels);
+ *                     NHWC shapes whose pixel rows are multiples of 16 bytes, of at most 8192 channels; a later
+ *                     layer of many large NCHW frames has a small second kernel that writes the exits out);
  *   SMTM_ROUTE_DENSE  fast memories above 64 entries: pooling, then Eq. 1's dot products against
  *                     every class on the tensor cores, then a finishing kernel;
  *   SMTM_ROUTE_PLAIN  everything else: CUDA-core kernels, pooling and scoring apart (NCHW frames of megabytes

@@ -27,8 +27,7 @@ __device__ __forceinline__ void set_status(int* status, int code) {
 // visible; nothing that reads or writes global memory comes before it.  A CTA may be resident while the kernel before
 // still writes, so what that kernel writes (centres, their lengths, flags, vectors, dot products) is read by ordinary
 // loads: __ldg and const __restrict__ parameters ask for data that nothing writes while the kernel is there, and may be
-// moved above the wait.  (The stash of vectors in the update is complete before the plan kernel, its predecessor, lets it
-// in.)  chain_release() lets
+// moved above the wait.  chain_release() lets
 // the next kernel's CTAs in as soon as all of this kernel's have called it.  Kernels call it
 // right after chain_wait(): a kernel then only ever shares the device with its direct
 // neighbours (released before the wait, a chain of small kernels would let a much later

@@ -993,8 +993,8 @@ __global__ void __launch_bounds__(kLightThreads, kHalves ? 5 : 4) k_lookup_spars
     chain_wait();  // the exit flags are the previous kernel's
     chain_release();
     const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);
-    // The active frames of this cluster and their streams: the cluster's own, or from a list.  Every thread looks at four consecutive frames, one trip to
-    // memory and one scan for 512.  Where the clusters do not all fit beside the streaming kernel, one of the first may have
+    // The active frames of this cluster and their streams: the cluster's own, or from a list, for which every thread looks
+    // at four consecutive frames, one trip to memory and one scan for 512.  Where the clusters do not all fit beside the streaming kernel, one of the first may have
     // decided a frame before the last ones begin: its exit is pending, the flag is what it was before the launch, so that
     // every cluster gets the same list whenever it looks.
     constexpr int kPer = 4;
@@ -1201,8 +1201,8 @@ constexpr int kFrameStageLeast = 8 * 1024, kFrameStageLeastMany = 4 * 1024;     
 constexpr int kFrameManySlots = 32, kFrameResident = 2;                           // CTAs an SM holds
 constexpr int kCrowdSlots = 8, kCrowdNarrowSlots = 16, kCrowdFrame = 128 * 1024;
 constexpr long long kFrameBatchMost = 64ll << 20;  // bytes of the batch above which the streaming kernel takes over
-// When a cluster shares a frame of an NHWC map (its CTAs have half the threads of the CTA that takes a frame alone, and meet
-// at two barriers).  Lookups: up to half as many frames as SMs, frames of 96 KB and more, six pixels a thread of the CTA it
+// When a cluster shares a frame of an NHWC map (its CTAs have half the threads of the CTA that takes a frame alone, and wait
+// for one another's column sums).  Lookups: up to half as many frames as SMs, frames of 96 KB and more, six pixels a thread of the CTA it
 // replaces and more, as many CTAs as the chip holds at once (768 KB: twice as many).  With 32 slots and more the clusters also share the scoring: a CTA on every SM at least; so do, with 16, the handful of
 // frames of a stream or a few.  In
 // geometric mean over 525 lookups of 1 .. 2048 frames 20 % faster than a CTA per frame; the line it replaces, which let four
@@ -1392,7 +1392,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame(const FramePa
     chain_release();
     const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);
     const int sid_raw = a.stream_id ? a.stream_id[b] : 0;  // in flight with the exit flag
-    // (no CTA of the cluster can have decided yet: the decision comes after a barrier all of them arrive on)
+    // (the cluster cannot have decided yet: the decision waits for what every CTA delivers after all its threads are past here)
     if (!a.fresh && a.done[b]) return;
     if (P > 1) cluster_arrive();  // (waited for before the first store to a peer: it has to have started)
     const uint32_t bytes = uint32_t(w_nch) * uint32_t(p.ch_bytes);
@@ -1597,7 +1597,7 @@ __global__ void __launch_bounds__(kFrameThreads, 2) k_lookup_frame_nhwc(const Fr
     chain_release();
     const ClockScope stamps(a.clock ? a.clock + 2 * a.layer : nullptr);
     const int sid_raw = a.stream_id ? a.stream_id[b] : 0;  // in flight with the exit flag
-    // (no CTA of the cluster can have decided yet: the decision comes after a barrier all of them arrive on)
+    // (the cluster cannot have decided yet: the decision waits for what every CTA delivers after all its threads are past here)
     if (!a.fresh && a.done[b]) return;
     cluster_arrive();  // (waited for before the first store to a peer: it has to have started)
     const bool decides = rank == 0 && warp == 0;

@@ -78,15 +78,17 @@ __device__ __forceinline__ Top2 block_top2_keys(unsigned long long b1, unsigned 
 // of the slots, a warp 32 / F slots (at most eight) at a time; where the share is too small for eight warps they divide the
 // vector length as well.  The dot products of frame f meet, through distributed shared memory, in CTA f % P of the cluster,
 // which decides it.  What bounds it: the centres' way from L2 (k D words per cluster instead of per frame) and, for small
-// problems, the trips to memory ([exit layers, slots] -> [vectors, centres] -> decision).
+// problems, the trips to memory ([exit flags, slots] -> [vectors, centres] -> decision).
 constexpr int kShareMost = 8;                    // frames, and CTAs, of a cluster at most
-constexpr long long kShareWork = 4608;           // words of centres below which a CTA per frame scores
+// Words of centres (at least 64 to a slot) below which a CTA per frame scores: 65 to 71 slots of up to 64 channels, 10.4 us for
+// 8 frames of one pixel and 22 for 600, where the clusters, from 72 slots on 6.9 and 17, would be faster too.
+constexpr long long kShareWork = 4608;
 constexpr size_t kShareSmem = 200 * 1024;
 // Frames to a cluster: eight, fewer until every SM has a CTA.  CTAs to a cluster: eight, fewer where they would queue up for a
 // place on an SM (two each) and would have at most 64 slots.  Pooling and scoring of 1x1 maps by a CTA per frame and here, us,
 // 1024 channels: 256 frames against 101 slots 24 and 18, 1024 frames 56 and 32 (in clusters of eight 48), 256 against 999 167
 // and 39, 1024 400 and 126 (in clusters of two 108, but with a fifth of the frames left 105 instead of 36); 8 frames of 32
-// channels against 70 slots 12.7 and 9.1, 600 of 64 channels 26.3 and 21.5 (in clusters of eight 28.8).
+// channels against 72 slots 10.9 and 6.9, 600 of 64 channels 23 and 17.
 constexpr int kShareSlots = 64;
 // F vectors [F][D] | [F / P][k_max] dot products of the frames this CTA decides | [k_max] the slots' classes | partial sums
 // [8 warps][32].

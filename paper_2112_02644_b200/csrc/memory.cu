@@ -15,8 +15,8 @@
 // a grid of small CTAs (128 threads, a few KB of shared memory) with two kinds of work: the
 // first B CTAs look after the tables, one per frame (the CTA of a stream's first frame in the
 // batch applies all of the stream's frames to its tables and, when asked, refreshes its fast
-// memory by Eq. 5 / Eq. 6; the others leave at once; the tables of an only stream are shared by a
-// cluster of up to eight); the remaining CTAs take the listed pairs,
+// memory by Eq. 5 / Eq. 6; the others leave at once; an only stream has a cluster of up to eight
+// instead); the remaining CTAs take the listed pairs,
 // one each, and fold the pair's frames into the centre (Eq. 7; a pair with many frames is several items, each
 // a block of the vector's columns).  Small CTAs on purpose: there
 // are hundreds of independent pieces of work, each a short chain of dependent trips to L2, so
@@ -753,7 +753,7 @@ __device__ void tables_of_frame(const UpdateArgs& a, const ResizeArgs& rz, int g
     const bool lone = PER == 0 && g < 0;  // (up to 1024 classes an only stream has tables_of_lone_stream)
     if (lone) g = 0;
     const int s = (a.stream_id && !lone) ? a.stream_id[g] : 0;
-    if (s < 0 || s >= a.S) return;  // no such stream (the same for every thread; the plan kernel records the error)
+    if (s < 0 || s >= a.S) return;  // no such stream (the same for every thread; whoever makes the frame's code records the error)
     const int per = PER ? PER : (a.n + nt - 1) / nt;
     const int c_lo = min(a.n, tid * per), c_hi = min(a.n, c_lo + per);
     int32_t* ft = a.ft + (size_t)s * a.n;
@@ -1125,8 +1125,8 @@ __device__ __forceinline__ void tables_cta(const UpdateArgs& a, const ResizeArgs
         tables_of_frame<0, kPlanned>(a, rz, g, do_resize, dyn, s_list, s_scan, s_part);
 }
 
-// The apply kernel: CTAs [0, table_ctas) are tables CTAs, one per frame (a single one for a cache with one stream);
-// the others take the listed items.
+// The apply kernel: CTAs [0, table_ctas) are tables CTAs, one per frame (for a cache with one stream one for every 128
+// classes, a cluster, beyond 1024 a single one); the others take the listed items.
 __global__ void __launch_bounds__(kApplyThreads, 8) k_update_apply(const UpdateArgs a, const ResizeArgs rz, int do_resize,
                                                                     int table_ctas) {
     extern __shared__ __align__(16) unsigned long long s_dyn[];
@@ -1168,7 +1168,9 @@ __global__ void __launch_bounds__(kApplyThreads, 8) k_update_apply(const UpdateA
 // A frame of a vector that is worth several blocks by itself (more than 4096 channels) has that many CTAs, and as many again
 // for the blocks that a few frames together are rounded up to, while they are at most two to an SM: one frame of 65536
 // channels 98 us with a CTA, 17 by two launches, 11 so, three frames of one class of 16384 channels 17.1, 7.5 and 5.9.
-// No CTA waits for another, and the sums are those of the two launches.  What bounds it: trips to memory (three here, five
+// No CTA waits for another.  A pair is cut into at most as many blocks as its frames have CTAs, and into blocks at all where
+// the plan does not count frames (more than 8192 pairs), so the order in which rows and squared lengths are added, and with it
+// the last bits of a centre and its length, may differ from the two launches'.  What bounds it: trips to memory (three here, five
 // and a launch there), and with many frames the state that every CTA fetches, so the two launches stay beyond the lines
 // below.  Update with refresh, 200 classes, by two launches and by one: 16 frames in one layer of 256 channels 6.9 and 5.1
 // us, 128 frames in 13 layers 9.3 and 6.7, 256 in two of 1024 channels 8.7 and 7.2, 512 in two 9.1 and 7.7; 512 streams in
